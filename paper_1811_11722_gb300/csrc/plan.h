@@ -77,7 +77,8 @@ struct Plan {
   SavedProblem saved;
   // what plan_rebase needs to move the plan to another lattice
   int param_kind = 0;       // launches hold RuleParams<float> (1), RuleParams<double> (2),
-                            // GeneralParams<float> (3), GeneralParams<double> (4); 0: fixed lattice
+                            // GeneralParams<float> (3), GeneralParams<double> (4), FxParams (5);
+                            // 0: fixed lattice
   int grid_occ = 1;         // CTAs per SM the launch shape assumes
   bool grid_capped = true;  // the launch shape honours a cap on CTAs (rule plans; not deformed ones)
 };
@@ -117,6 +118,12 @@ int plan_build(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, co
                qmc_transform t, const qmc_integrand* f, const TuneChoice& tune, const qmc_eps* eps = nullptr);
 int build_deformed_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
                         const qmc_transform& t, const qmc_integrand* f, const TuneChoice& tune);
+// FP64 sectors in 64-bit fixed point (fixed64.cu): builds the plan's launches,
+// or QMC_EUNSUPPORTED (nothing written) for integrands outside its range.
+int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
+                  const qmc_transform& t, const qmc_integrand* f, const TuneChoice& tune);
+int fx_rebase(Plan* pl, uint64_t n, const uint64_t* g, int max_ctas);
+void fx_reshift(Plan* pl, const double* shifts);
 int plan_alloc(Plan* pl, cudaStream_t stream, bool async);
 void plan_free(Plan* pl, cudaStream_t stream);
 int launch_rule(const Plan* pl, const Workspace& ws, cudaStream_t stream, const SampleIO& sio);

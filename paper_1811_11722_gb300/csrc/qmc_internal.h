@@ -141,6 +141,29 @@ __host__ __device__ inline void fill_pairs(RuleParams<R>& P, int d) {
     P.cp[nu + s] = make_float2(-(float)P.cF[s], -(float)P.cF[s]);
 }
 
+// FP64 sectors in fixed point (fixed64.cuh): parameters of one launch, up to
+// kMcMax shift rows, two per CTA row.  Offsets of n, tiles and L as in RuleParams.
+struct FxParams {
+  uint64_t n;
+  uint64_t tiles;
+  int32_t L;
+  int32_t d;
+  int32_t m_launch;
+  int32_t k_base;
+  int32_t nblk;
+  int32_t tr;
+  double value_scale;           // constant factor of every value (applied by the final pass)
+  Recip rc;
+  uint32_t g[kDFast];
+  uint32_t step[kDFast][3];     // fraction (kThreads g_i mod n) / n to 96 bits, low word first
+  uint64_t shift[kMcMax][kDFast];
+  uint64_t u0, uk;              // U: constant term in Q(k-1), recentring constant of its cross terms
+  uint32_t uh[kDFast], ul[kDFast];  // linear coefficients: high word; low word / 8
+  uint64_t f0;                  // F: constant term in Q(k-2)
+  uint64_t fl[kDFast], fk[kDFast];  // rows: linear coefficient in Q(k-1), recentring constant
+  uint32_t fh[kDFast * (kDFast + 1) / 2], fq[kDFast * (kDFast + 1) / 2];  // q_ij, row by row
+};
+
 // Several integrands on one lattice (shared-lattice sweep): the rule's
 // parameters plus the (c, c) pairs of each integrand of this launch's chunk.
 constexpr int kMultiChunk = 8;  // integrands fused into one launch
