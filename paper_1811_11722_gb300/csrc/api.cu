@@ -230,6 +230,29 @@ Recip reciprocal(uint64_t n) {
   return r;
 }
 
+// floor(idx 2^64 / n) within 1, as frac64
+static uint64_t fraction64(uint32_t idx, const Recip& rc) {
+  return (uint64_t)idx * rc.rhi + (uint64_t)(((unsigned __int128)idx * rc.rlo) >> 64);
+}
+
+// The centred form's z has an absolute error of 2^-25, so U and F get a
+// relative one of up to 2^-25 (sum of |coefficients|) / (constant term) at the
+// corner z = 0.  Emulated against 64 bits, the values' rms error is no larger
+// than the other form's up to a ratio of about 4 (d = 2), 8 (3), 32 (4), 128
+// (5) and 256 (6): the corner's share of the cube shrinks with d.  The line
+// stays below those.
+int korobov_form(int d, const std::vector<double>& cu, const std::vector<double>& cf) {
+  const double most = std::ldexp(1.0, d <= 4 ? d : d + 1);
+  for (const std::vector<double>* c : {&cu, &cf}) {
+    double sum = 0.0;
+    for (double v : *c) sum += std::fabs(v);
+    if (!(sum <= most * (*c)[0])) return 3;
+  }
+  return kKorCentred;
+}
+
+double korobov_scale(int form, int d) { return std::pow(form == kKorCentred ? 140.0 / 64.0 : 140.0, (double)d); }
+
 // Korobov z(s) = C sum_k binom(a,k) (-1)^k s^(a+k+1)/(a+k+1), C = (2a+1)!/(a!)^2.
 void korobov_coefs(int alpha, double* kor /*8*/) {
   double C = 1.0;
@@ -281,6 +304,7 @@ void fill_common(RuleParams<R>& P, int32_t d, uint64_t n, const uint64_t* g, con
   for (int i = 0; i < d; ++i) {
     P.g[i] = (uint32_t)g[i];
     P.gstep[i] = (uint32_t)(((uint64_t)kThreads * g[i]) % n);
+    P.fstep[i] = fraction64(P.gstep[i], P.rc);
   }
   double kor[8];
   korobov_coefs(P.alpha > 0 ? P.alpha : 1, kor);
@@ -421,8 +445,9 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
       }
       for (size_t i = 0; i < cu.size(); ++i) base.cU[i] = (R)cu[i];
       for (size_t i = 0; i < cf.size(); ++i) base.cF[i] = (R)cf[i];
-      if (base.tr == TR_KOROBOV) base.value_scale = std::pow((double)base.kor[7], (double)d);
+      if (base.tr == TR_KOROBOV) base.value_scale = korobov_scale(3, d);
       if (fp32 && !tune.no_jit && jit_enabled()) {
+        const int form = base.tr == TR_KOROBOV ? korobov_form(d, pack_dense(f->U, d, 1), pack_dense(f->F, d, 2)) : 0;
         // run-time specialised, packed, exactly `orders` orders; one logarithm
         // per value when U, F > 0 on the cube and bF = -bU
         fill_pairs(base, d);
@@ -432,11 +457,11 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
         const bool log1 = positive && eps->bF == -eps->bU;
         void* fn = nullptr;
         int occ = 0;
-        if (jit_eps_f32(d, jmc, NE, base.tr, base.tr == TR_KOROBOV ? 3 : 0, log1, !positive, cu, cf, &fn, &occ) ==
-            QMC_OK) {
+        if (jit_eps_f32(d, jmc, NE, base.tr, form, log1, !positive, cu, cf, &fn, &occ) == QMC_OK) {
           jit_fn = fn;
           jit_occ = occ;
           mc = jmc;
+          if (base.tr == TR_KOROBOV) base.value_scale = korobov_scale(form, d);
         }
       }
     } else {
@@ -454,6 +479,8 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
       mc = 16;
     }
     const bool m21 = f->aU == -2 && f->aF == -1;
+    if (fp32 && KU == 1 && base.tr == TR_KOROBOV && base.alpha == 3)
+      base.alpha = korobov_form(d, pack_dense(f->U, d, 1), pack_dense(f->F, d, 2));
     if (KU > 0 && d <= kDFast && m21 && !tune.force_general) {
       switch (d) {
 #define QMC_D_CASE(DD) \
@@ -476,7 +503,7 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
       for (size_t i = 0; i < cu.size(); ++i) base.cU[i] = (R)cu[i];
       for (size_t i = 0; i < cf.size(); ++i) base.cF[i] = (R)cf[i];
       if (fp32 && KU == 1 && KF == 2) fill_pairs(base, d);
-      if (base.tr == TR_KOROBOV) base.value_scale = std::pow((double)base.kor[7], (double)d);
+      if (base.tr == TR_KOROBOV) base.value_scale = korobov_scale(base.alpha, d);
       if (fp32 && KU == 1 && KF == 2 && !tune.no_jit && jit_enabled()) {
         void* fn = nullptr;
         int occ = 0;
@@ -497,7 +524,7 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
               imm[(size_t)kk * d + i] =
                   (uint32_t)((shift_fixed64(shifts[(size_t)(kk < m ? kk : 0) * d + i]) + 0x80000000ull) >> 32);
         }
-        if (jit_sector_f32(d, mc, base.tr, base.tr == TR_KOROBOV ? 3 : 0, base.check_finite != 0, cu, cf, smacc,
+        if (jit_sector_f32(d, mc, base.tr, base.tr == TR_KOROBOV ? base.alpha : 0, base.check_finite != 0, cu, cf, smacc,
                            tune.minb, &fn, &occ, &sm, use_imm ? imm.data() : nullptr) == QMC_OK) {
           pl->imm = use_imm ? 1 : 0;
           jit_fn = fn;
@@ -507,6 +534,7 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
       }
     } else {
       general = true;
+      base.alpha = t.kind == QMC_TRANSFORM_KOROBOV ? t.alpha : 0;
     }
   } else if (f->kind == QMC_F_SECTOR_DEFORMED) {
     return fail(QMC_EUNSUPPORTED, "deformed sector integrands are served by the complex kernels");
@@ -657,6 +685,7 @@ static void rebase_rule(RuleParams<R>& P, int d, uint64_t n, const uint64_t* g, 
   for (int i = 0; i < d; ++i) {
     P.g[i] = (uint32_t)g[i];
     P.gstep[i] = (uint32_t)(((uint64_t)kThreads * g[i]) % n);
+    P.fstep[i] = fraction64(P.gstep[i], P.rc);
   }
   P.L = L;
   P.tiles = tiles;

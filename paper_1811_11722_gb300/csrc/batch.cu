@@ -267,6 +267,7 @@ static int persist_build(BatchPlan* bp, int32_t count, const qmc_problem* proble
     fill_common(base, q.d, q.n, q.g, q.t, &f);
     auto cu = pack_dense(f.U, q.d, 1);
     auto cf = pack_dense(f.F, q.d, 2);
+    if (base.tr == TR_KOROBOV) base.alpha = korobov_form(q.d, cu, cf);
     prescale_slots(cu.data(), q.d, 1, fx_sigma(base.tr));
     prescale_slots(cf.data(), q.d, 2, fx_sigma(base.tr));
     for (size_t i = 0; i < cu.size(); ++i) base.cU[i] = (float)cu[i];
@@ -277,7 +278,7 @@ static int persist_build(BatchPlan* bp, int32_t count, const qmc_problem* proble
     sec.m = q.m;
     sec.n = q.n;
     sec.nitems = (int)((q.n + chunk - 1) / chunk);
-    sec.final_scale = base.tr == TR_KOROBOV ? std::pow((double)base.kor[7], (double)q.d) : 1.0;
+    sec.final_scale = base.tr == TR_KOROBOV ? korobov_scale(base.alpha, q.d) : 1.0;
     bp->ps_off.push_back((size_t)bp->total_m * 2);
     bp->total_m += q.m;
     bp->max_m = std::max(bp->max_m, q.m);
@@ -467,6 +468,7 @@ static void persist_descriptors(const BatchPlan* bp, std::vector<PjSector>* secs
       PjSector& S = secs[s];
       S.d = P.d;
       S.tr = P.tr;
+      S.alpha = P.alpha;
       S.check = P.check_finite != 0;
       S.n = P.n;
       S.rc = P.rc;

@@ -272,10 +272,34 @@ __device__ __forceinline__ uint32_t dither32(uint64_t j, int i) {
 // of the integral against the FP64 rule.  The product of the d independent
 // factors rounds without that bias, and its cube is formed from an exact
 // square (two-product) with one final rounding.
+//
+// ALPHA == kKorCentred: the caller's base carries an extra 2^31 (fx_bias), so
+// X read as signed is T = 2^32 (x - 1/2).  With v = 2x - 1 and u = 1 - v^2 =
+// 4x(1-x), weight 3 is z = 1/2 + v (16 + 8u + 6u^2 + 5u^3) / 32: seven
+// operations for z and the weight's factor u, against nine and three integer
+// ones for the form on min(x, 1-x), which has to put z on its half of the cube.
+// d = 8, n = 16777213, m = 16: 1.25 -> KORT ms.  z carries an absolute error of
+// 2^-25 where the other form's is relative to z, which matters when U or F
+// comes near zero at the cube's corner: korobov_form() keeps such integrands
+// on the other form.  w then collects 4x(1-x), and 140/64 per dimension is
+// left to the final pass.
+template <int ALPHA>
+__host__ __device__ constexpr uint32_t fx_bias() {
+  return ALPHA == kKorCentred ? 0x80000000u : 0u;
+}
+
 template <int TR, int ALPHA>
 __device__ __forceinline__ float coord_fx(uint32_t X, const float* kor, float& w) {
   if constexpr (TR == TR_NONE) {
     return __uint2float_rn(X);  // z 2^32
+  } else if constexpr (ALPHA == kKorCentred) {
+    const float T = __int2float_rn((int32_t)X);
+    const float u = __fmaf_rn(__fmul_rn(T, -0x1p-62f), T, 1.0f);
+    float q = __fmaf_rn(5 * 0x1p-36f, u, 6 * 0x1p-36f);
+    q = __fmaf_rn(q, u, 8 * 0x1p-36f);
+    q = __fmaf_rn(q, u, 16 * 0x1p-36f);
+    w = __fmul_rn(w, u);
+    return __fmaf_rn(T, q, 0.5f);
   } else {
     const float a = fabsf(__int2float_rn((int32_t)X));
     if constexpr (TR == TR_BAKER) {
@@ -306,6 +330,14 @@ template <int TR, int ALPHA>
 __device__ __forceinline__ float2 coord_fx2(uint32_t Xa, uint32_t Xb, const float* kor, float2& w) {
   if constexpr (TR == TR_NONE) {
     return make_float2(__uint2float_rn(Xa), __uint2float_rn(Xb));
+  } else if constexpr (ALPHA == kKorCentred) {
+    const float2 T = make_float2(__int2float_rn((int32_t)Xa), __int2float_rn((int32_t)Xb));
+    const float2 u = fma2(mul2(T, make_float2(-0x1p-62f, -0x1p-62f)), T, make_float2(1.0f, 1.0f));
+    float2 q = fma2(make_float2(5 * 0x1p-36f, 5 * 0x1p-36f), u, make_float2(6 * 0x1p-36f, 6 * 0x1p-36f));
+    q = fma2(q, u, make_float2(8 * 0x1p-36f, 8 * 0x1p-36f));
+    q = fma2(q, u, make_float2(16 * 0x1p-36f, 16 * 0x1p-36f));
+    w = mul2(w, u);
+    return fma2(T, q, make_float2(0.5f, 0.5f));
   } else {
     const float2 a = make_float2(fabsf(__int2float_rn((int32_t)Xa)), fabsf(__int2float_rn((int32_t)Xb)));
     if constexpr (TR == TR_BAKER) {

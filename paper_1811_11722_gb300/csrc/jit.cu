@@ -464,7 +464,7 @@ int persist_sources(const std::vector<PjSector>& secs, const std::vector<PjDesc>
     const std::string nm = "qmc_sp_" + std::to_string(q);
     src += "struct " + nm + " {\n";
     src += "  static constexpr int D = " + std::to_string(S.d) + ", TR = " + std::to_string(S.tr) +
-           ", ALPHA = " + std::to_string(S.tr == TR_KOROBOV ? 3 : 0) + ", MC = " + std::to_string(Dq.mc) +
+           ", ALPHA = " + std::to_string(S.tr == TR_KOROBOV ? S.alpha : 0) + ", MC = " + std::to_string(Dq.mc) +
            ", M = " + std::to_string(Dq.m) + ", KBASE = " + std::to_string(Dq.kbase) + ";\n";
     src += std::string("  static constexpr bool CHECK = ") + (S.check ? "true" : "false") + ";\n";
     if (!rt) {  // the lattice as constants (with run-time lattices it comes from the launch)

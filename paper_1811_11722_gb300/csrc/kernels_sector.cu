@@ -25,6 +25,8 @@ namespace qmc {
     if (tr == TR_NONE) QMC_SECTOR_CK(R, MC, TR_NONE, 0, KU, KF);                  \
     if (tr == TR_BAKER) QMC_SECTOR_CK(R, MC, TR_BAKER, 0, KU, KF);                \
     if (tr == TR_KOROBOV && alpha == 3) QMC_SECTOR_CK(R, MC, TR_KOROBOV, 3, KU, KF); \
+    if constexpr (sizeof(R) == 4 && KU == 1)                                         \
+      if (tr == TR_KOROBOV && alpha == kKorCentred) QMC_SECTOR_CK(R, MC, TR_KOROBOV, kKorCentred, KU, KF); \
   } while (0)
 
 template <>

@@ -50,11 +50,13 @@ int build_multi_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
   RuleParams<float> base;
   fill_common(base, d, n, g, t, &fs[0]);
   base.m_total = m;
-  const int TR = base.tr, ALPHA = kor3 ? 3 : 0;
+  const int TR = base.tr;
+  int form = kor3 ? kKorCentred : 0;  // one coordinate for all: centred only if it serves every integrand
   // dense slots of every integrand
   std::vector<std::pair<std::vector<double>, std::vector<double>>> polys(count);
   for (int s = 0; s < count; ++s) {
     polys[s] = {pack_dense(fs[s].U, d, 1), pack_dense(fs[s].F, d, 2)};
+    if (kor3 && form == kKorCentred) form = korobov_form(d, polys[s].first, polys[s].second);
     prescale_slots(polys[s].first.data(), d, 1, fx_sigma(TR));  // coordinates arrive divided by fx_sigma
     prescale_slots(polys[s].second.data(), d, 2, fx_sigma(TR));
   }
@@ -65,7 +67,7 @@ int build_multi_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
   auto compile = [&](int c) {
     const int s0 = c * kMultiChunk, s1 = std::min(count, s0 + kMultiChunk);
     std::vector<std::pair<std::vector<double>, std::vector<double>>> part(polys.begin() + s0, polys.begin() + s1);
-    rcs[c] = jit_multi_f32(d, kMultiMc, TR, ALPHA, check, part, &fn[c], &occ[c]);
+    rcs[c] = jit_multi_f32(d, kMultiMc, TR, form, check, part, &fn[c], &occ[c]);
   };
   {
     const int hw = std::max(1u, std::thread::hardware_concurrency());
@@ -104,7 +106,7 @@ int build_multi_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
   pl->mc = kMultiMc;
   pl->func = nullptr;
   pl->value_scale = 1.0;
-  pl->final_scale = base.tr == TR_KOROBOV ? std::pow((double)base.kor[7], (double)d) : 1.0;
+  pl->final_scale = kor3 ? korobov_scale(form, d) : 1.0;
   for (int k0 = 0; k0 < m; k0 += kMultiMc) {
     const int mk = std::min(kMultiMc, m - k0);
     for (int c = 0; c < chunks; ++c) {

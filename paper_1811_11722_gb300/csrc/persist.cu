@@ -42,7 +42,7 @@ __device__ __noinline__ void persist_item(const RuleParams<float>& P, uint64_t j
     for (int s = 0; s < steps; ++s) {
       uint32_t base[D];
 #pragma unroll
-      for (int i = 0; i < D; ++i) base[i] = sec_base<float>(idx[i], P.rc, jt + (uint64_t)s * kThreads, i);
+      for (int i = 0; i < D; ++i) base[i] = sec_base<float, ALPHA>(idx[i], P.rc, jt + (uint64_t)s * kThreads, i);
 #pragma unroll
       for (int p = 0; p < MC / 2; ++p) {
         float2 v = sector_value2<D, TR, ALPHA, 1, 2, DensePolys>(P, base, p);
@@ -105,8 +105,13 @@ __device__ __forceinline__ void persist_dispatch_tr(const RuleParams<float>& P, 
     if (check) persist_item<D, TR_BAKER, 0, true>(P, j0, j1, item, nitems, partial, counters, red);
     else persist_item<D, TR_BAKER, 0, false>(P, j0, j1, item, nitems, partial, counters, red);
   } else if (P.tr == TR_KOROBOV) {
-    if (check) persist_item<D, TR_KOROBOV, 3, true>(P, j0, j1, item, nitems, partial, counters, red);
-    else persist_item<D, TR_KOROBOV, 3, false>(P, j0, j1, item, nitems, partial, counters, red);
+    if (P.alpha == kKorCentred) {
+      if (check) persist_item<D, TR_KOROBOV, kKorCentred, true>(P, j0, j1, item, nitems, partial, counters, red);
+      else persist_item<D, TR_KOROBOV, kKorCentred, false>(P, j0, j1, item, nitems, partial, counters, red);
+    } else {
+      if (check) persist_item<D, TR_KOROBOV, 3, true>(P, j0, j1, item, nitems, partial, counters, red);
+      else persist_item<D, TR_KOROBOV, 3, false>(P, j0, j1, item, nitems, partial, counters, red);
+    }
   } else {
     if (check) persist_item<D, TR_NONE, 0, true>(P, j0, j1, item, nitems, partial, counters, red);
     else persist_item<D, TR_NONE, 0, false>(P, j0, j1, item, nitems, partial, counters, red);

@@ -80,7 +80,7 @@ __device__ __forceinline__ void pj_sweep(uint64_t j0, uint64_t chunk, uint32_t i
     for (int s = 0; s < steps; ++s) {
       uint32_t base[D];
 #pragma unroll
-      for (int i = 0; i < D; ++i) base[i] = sec_base<float>(idx[i], rc, jt + (uint64_t)s * kThreads, i);
+      for (int i = 0; i < D; ++i) base[i] = sec_base<float, ALPHA>(idx[i], rc, jt + (uint64_t)s * kThreads, i);
 #pragma unroll
       for (int p = 0; p < MC / 2; ++p) {
         float2 z[D];

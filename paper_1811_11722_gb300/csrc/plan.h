@@ -118,6 +118,12 @@ int plan_build(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, co
                qmc_transform t, const qmc_integrand* f, const TuneChoice& tune, const qmc_eps* eps = nullptr);
 int build_deformed_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
                         const qmc_transform& t, const qmc_integrand* f, const TuneChoice& tune);
+// Weight code of the FP32 sector kernels under Korobov weight 3 for dense
+// slots cu, cf (degrees 1 and 2): kKorCentred where every sum of |coefficients|
+// is at most korobov_form's multiple of the constant term, else 3; and the
+// constant left to the final pass for a code.
+int korobov_form(int d, const std::vector<double>& cu, const std::vector<double>& cf);
+double korobov_scale(int form, int d);
 // FP64 sectors in 64-bit fixed point (fixed64.cu): builds the plan's launches,
 // or QMC_EUNSUPPORTED (nothing written) for integrands outside its range.
 int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
@@ -145,7 +151,7 @@ int jit_eps_f32(int D, int MC, int NE, int TR, int ALPHA, bool log1, bool check,
 // One sector of a run-time specialised persistent batch: its rule as the
 // packed FP32 sector path sees it (prescaled dense slots of U and F).
 struct PjSector {
-  int d = 0, tr = 0;
+  int d = 0, tr = 0, alpha = 0;
   bool check = false;
   uint64_t n = 0;
   Recip rc{0, 0};

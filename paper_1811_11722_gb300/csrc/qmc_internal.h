@@ -30,6 +30,10 @@ constexpr int kEpsAcc = 24;     // shifts x orders accumulated by one epsilon la
 
 enum TransformCode { TR_NONE = 0, TR_BAKER = 1, TR_KOROBOV = 2 };
 
+// Korobov weight 3 in the form centred on x = 1/2 (coord_fx), as a weight code
+// of the FP32 sector kernels beside the plain 3; korobov_form() chooses.
+constexpr int kKorCentred = -3;
+
 // Integrand code inside kernels.
 enum FKind { FK_CONST = 0, FK_SEPEXP = 1, FK_SECTOR = 2, FK_DEFORMED = 3, FK_TRIG = 4 };
 
@@ -67,6 +71,7 @@ struct RuleParams {
   Recip rc;
   uint32_t g[QMC_DMAX];
   uint32_t gstep[QMC_DMAX];     // (kThreads * g_i) mod n
+  uint64_t fstep[QMC_DMAX];     // its fraction gstep / n, 64 bits
   uint64_t shift64[kMcMax][QMC_DMAX];
   uint32_t shift32[kMcMax][QMC_DMAX];
   uint32_t shiftx[kMcMax][QMC_DMAX];    // FP32 sector path: Delta rounded to 32-bit fixed point

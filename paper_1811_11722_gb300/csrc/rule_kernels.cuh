@@ -217,18 +217,51 @@ __device__ __forceinline__ R eps_point(const RuleParams<R>& P, const typename Se
 }
 
 // Per-point base of coordinate i at point j (FP32: 32-bit fixed point plus the
-// dither of point j, dimension i; FP64: 64-bit fixed point).
-template <typename R>
+// dither of point j, dimension i, plus the weight code's bias; FP64: 64-bit
+// fixed point).
+template <typename R, int ALPHA = 0>
 __device__ __forceinline__ typename SecBase<R>::T sec_base(uint32_t idx, const Recip& rc, uint64_t j, int i) {
-  if constexpr (sizeof(R) == 4) return base32(frac64(idx, rc)) + dither32(j, i);
+  if constexpr (sizeof(R) == 4) return base32(frac64(idx, rc)) + dither32(j, i) + fx_bias<ALPHA>();
   else return frac64(idx, rc);
 }
 
-template <typename R>
+template <typename R, int ALPHA = 0>
 __device__ __forceinline__ double sec_coord_used(const RuleParams<R>& P, typename SecBase<R>::T b, int k, int i) {
-  if constexpr (sizeof(R) == 4) return (double)(uint32_t)(b + P.shiftx[k][i]) * 0x1p-32;
+  if constexpr (sizeof(R) == 4) return (double)(uint32_t)(b - fx_bias<ALPHA>() + P.shiftx[k][i]) * 0x1p-32;
   else return coord_used<R>(b + shift_of(P, k, i));
 }
+
+// The bases of a thread's successive points (kThreads apart) in the FP32
+// sector sweeps.  The fraction of g j / n advances by a constant modulo 1, so
+// it is carried in 64-bit fixed point, half a unit of 2^-32 added once for the
+// rounding: per point and dimension two adds for it, one for the dither's
+// Weyl sequence (top 7 bits as a signed number), a shift and an add, against
+// the index step, its comparison and a 128-bit reciprocal product.  The step's
+// floor is off by 2^-64 a point, 2^-55 over a tile.
+template <int D, int ALPHA>
+struct FxWalk {
+  uint64_t p[D];
+  uint32_t h[D];
+  static __device__ __forceinline__ uint32_t weyl(int i) { return 0x9E3779B9u ^ ((uint32_t)i * 0x632BE5AAu); }
+  __device__ __forceinline__ void start(const RuleParams<float>& P, uint64_t j) {
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      p[i] = frac64(lattice_index(j, P.g[i], P.n), P.rc) + 0x80000000ull + ((uint64_t)fx_bias<ALPHA>() << 32);
+      h[i] = (uint32_t)j * weyl(i);
+    }
+  }
+  __device__ __forceinline__ void bases(uint32_t* b) const {
+#pragma unroll
+    for (int i = 0; i < D; ++i) b[i] = (uint32_t)(p[i] >> 32) + (uint32_t)((int32_t)h[i] >> 25);
+  }
+  __device__ __forceinline__ void step(const RuleParams<float>& P) {
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      p[i] += P.fstep[i];
+      h[i] += (uint32_t)kThreads * weyl(i);
+    }
+  }
+};
 
 template <typename R, int D, int TR, int ALPHA, int KU, int KF, class POLY>
 __device__ void sector_sample(const RuleParams<R>& P, const SampleIO& sio) {
@@ -241,9 +274,9 @@ __device__ void sector_sample(const RuleParams<R>& P, const SampleIO& sio) {
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     uint32_t idx = lattice_index(j, P.g[i], P.n);
-    base[i] = sec_base<R>(idx, P.rc, j, i);
+    base[i] = sec_base<R, ALPHA>(idx, P.rc, j, i);
     if (sio.idx) sio.idx[(size_t)s * D + i] = idx;
-    if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<R>(P, base[i], k, i);
+    if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<R, ALPHA>(P, base[i], k, i);
   }
   R v = sector_value<R, D, TR, ALPHA, KU, KF, POLY>(P, base, k);
   sio.values[2 * (size_t)s] = (double)v * (double)P.value_scale;
@@ -332,13 +365,22 @@ __device__ __forceinline__ void sector_body(const RuleParams<R>& P, double* __re
     if (j0 >= P.n) continue;
     uint64_t left = (P.n - j0 + kThreads - 1) / kThreads;
     const int steps = left < (uint64_t)P.L ? (int)left : P.L;
-    uint32_t idx[D];
+    uint32_t idx[sizeof(R) == 4 ? 1 : D];
+    FxWalk<sizeof(R) == 4 ? D : 1, ALPHA> walk;
+    if constexpr (sizeof(R) == 4) {
+      walk.start(P, j0);
+    } else {
 #pragma unroll
-    for (int i = 0; i < D; ++i) idx[i] = lattice_index(j0, P.g[i], P.n);
+      for (int i = 0; i < D; ++i) idx[i] = lattice_index(j0, P.g[i], P.n);
+    }
     for (int s = 0; s < steps; ++s) {
       typename SecBase<R>::T base[D];
+      if constexpr (sizeof(R) == 4) {
+        walk.bases(base);
+      } else {
 #pragma unroll
-      for (int i = 0; i < D; ++i) base[i] = sec_base<R>(idx[i], P.rc, j0 + (uint64_t)s * kThreads, i);
+        for (int i = 0; i < D; ++i) base[i] = sec_base<R>(idx[i], P.rc, j0 + (uint64_t)s * kThreads, i);
+      }
       if constexpr (kPack) {
 #pragma unroll
         for (int p = 0; p < MC / 2; ++p) {
@@ -364,8 +406,12 @@ __device__ __forceinline__ void sector_body(const RuleParams<R>& P, double* __re
           acc[kk].add(v);
         }
       }
+      if constexpr (sizeof(R) == 4) {
+        walk.step(P);
+      } else {
 #pragma unroll
-      for (int i = 0; i < D; ++i) idx[i] = index_step(idx[i], P.gstep[i], n);
+        for (int i = 0; i < D; ++i) idx[i] = index_step(idx[i], P.gstep[i], n);
+      }
       if constexpr (sizeof(R) == 4 && !kPackFold) {
         if ((s & fold_mask<TR>()) == fold_mask<TR>()) {
           if constexpr (kPack) unpack_runs<MC>(run2, acc);
@@ -795,9 +841,9 @@ __device__ __forceinline__ void eps_body2(const RuleParams<float>& P, double* __
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       uint32_t idx = lattice_index(j, P.g[i], P.n);
-      base[i] = sec_base<float>(idx, P.rc, j, i);
+      base[i] = sec_base<float, ALPHA>(idx, P.rc, j, i);
       if (sio.idx) sio.idx[(size_t)s * D + i] = idx;
-      if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<float>(P, base[i], k, i);
+      if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<float, ALPHA>(P, base[i], k, i);
       z[i] = coord_fx<TR, ALPHA>(base[i] + P.shiftx[k][i], P.kor, w);
     }
     float U, F;
@@ -811,7 +857,6 @@ __device__ __forceinline__ void eps_body2(const RuleParams<float>& P, double* __
     }
     return;
   }
-  const uint32_t n = (uint32_t)P.n;
   float2 run2[NE][MC / 2];
   Acc<float> acc[NE][MC];
   unsigned nbad[NE];
@@ -829,13 +874,11 @@ __device__ __forceinline__ void eps_body2(const RuleParams<float>& P, double* __
     if (j0 >= P.n) continue;
     uint64_t left = (P.n - j0 + kThreads - 1) / kThreads;
     const int steps = left < (uint64_t)P.L ? (int)left : P.L;
-    uint32_t idx[D];
-#pragma unroll
-    for (int i = 0; i < D; ++i) idx[i] = lattice_index(j0, P.g[i], P.n);
+    FxWalk<D, ALPHA> walk;
+    walk.start(P, j0);
     for (int st = 0; st < steps; ++st) {
       uint32_t base[D];
-#pragma unroll
-      for (int i = 0; i < D; ++i) base[i] = sec_base<float>(idx[i], P.rc, j0 + (uint64_t)st * kThreads, i);
+      walk.bases(base);
 #pragma unroll
       for (int p = 0; p < MC / 2; ++p) {
         float2 z[D];
@@ -869,8 +912,7 @@ __device__ __forceinline__ void eps_body2(const RuleParams<float>& P, double* __
           if (o + 1 < NE) v = mul2(v, mul2(L, make_float2(P.eps_inv[o], P.eps_inv[o])));
         }
       }
-#pragma unroll
-      for (int i = 0; i < D; ++i) idx[i] = index_step(idx[i], P.gstep[i], n);
+      walk.step(P);
       if ((st & fold_mask<TR>()) == fold_mask<TR>()) {
 #pragma unroll
         for (int o = 0; o < NE; ++o) {
@@ -956,7 +998,6 @@ __device__ __forceinline__ void multi_body(const MultiParams& M, double* __restr
                                            unsigned long long* __restrict__ counters) {
   static_assert(MC % 2 == 0, "shift pairs");
   const RuleParams<float>& P = M.base;
-  const uint32_t n = (uint32_t)P.n;
   float2 run2[SC][MC / 2];
   Acc<float> acc[SC][MC];
   unsigned nbad[SC];
@@ -982,13 +1023,11 @@ __device__ __forceinline__ void multi_body(const MultiParams& M, double* __restr
     if (j0 >= P.n) continue;
     uint64_t left = (P.n - j0 + kThreads - 1) / kThreads;
     const int steps = left < (uint64_t)P.L ? (int)left : P.L;
-    uint32_t idx[D];
-#pragma unroll
-    for (int i = 0; i < D; ++i) idx[i] = lattice_index(j0, P.g[i], P.n);
+    FxWalk<D, ALPHA> walk;
+    walk.start(P, j0);
     for (int st = 0; st < steps; ++st) {
       uint32_t base[D];
-#pragma unroll
-      for (int i = 0; i < D; ++i) base[i] = sec_base<float>(idx[i], P.rc, j0 + (uint64_t)st * kThreads, i);
+      walk.bases(base);
 #pragma unroll
       for (int p = 0; p < MC / 2; ++p) {
         float2 z[D];
@@ -1014,8 +1053,7 @@ __device__ __forceinline__ void multi_body(const MultiParams& M, double* __restr
           else run2[s][p] = add2(run2[s][p], v);
         }
       }
-#pragma unroll
-      for (int i = 0; i < D; ++i) idx[i] = index_step(idx[i], P.gstep[i], n);
+      walk.step(P);
       if (!kPackFold && (st & fold_mask<TR>()) == fold_mask<TR>()) {
 #pragma unroll
         for (int s = 0; s < SC; ++s) {
