@@ -278,7 +278,7 @@ __device__ __forceinline__ uint32_t dither32(uint64_t j, int i) {
 // 4x(1-x), weight 3 is z = 1/2 + v (16 + 8u + 6u^2 + 5u^3) / 32: seven
 // operations for z and the weight's factor u, against nine and three integer
 // ones for the form on min(x, 1-x), which has to put z on its half of the cube.
-// d = 8, n = 16777213, m = 16: 1.25 -> KORT ms.  z carries an absolute error of
+// d = 8, n = 16777213, m = 16: 1.25 -> 0.91 ms.  z carries an absolute error of
 // 2^-25 where the other form's is relative to z, which matters when U or F
 // comes near zero at the cube's corner: korobov_form() keeps such integrands
 // on the other form.  w then collects 4x(1-x), and 140/64 per dimension is
