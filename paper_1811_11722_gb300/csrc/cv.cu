@@ -272,7 +272,9 @@ int qmc_cv_train(int32_t d, uint64_t n_pilot, const uint64_t* g_pilot, const dou
   qmc_transform tnone{QMC_TRANSFORM_NONE, 0};  // g approximates f itself on the cube
   (void)t;
   Plan pilot;
-  rc = plan_build(&pilot, d, n_pilot, 2, g_pilot, sh2.data(), tnone, &f64, TuneChoice{});
+  TuneChoice tc;
+  tc.no_fx = true;  // a fit amplifies its inputs' last bits: the pilot keeps the double kernels' values
+  rc = plan_build(&pilot, d, n_pilot, 2, g_pilot, sh2.data(), tnone, &f64, tc);
   if (rc) return rc;
   const int P = (int)n_pilot;
   CvFit F;

@@ -11,11 +11,11 @@ namespace qmc {
 
 namespace {
 
-// c 2^k as (high word, low word / 8), rounded to the nearest multiple of 8
+// c 2^k as (high word, low word / 16), rounded to the nearest multiple of 16
 void fx_split(double c, int k, uint32_t* h, uint32_t* l) {
-  const uint64_t q = (uint64_t)std::llrint(std::ldexp(c, k - 3));
-  *h = (uint32_t)(q >> 29);
-  *l = (uint32_t)(q & 0x1FFFFFFFu);
+  const uint64_t q = (uint64_t)std::llrint(std::ldexp(c, k - 4));
+  *h = (uint32_t)(q >> 28);
+  *l = (uint32_t)(q & 0x0FFFFFFFu);
 }
 
 uint64_t fx_fixed(double c, int k) { return (uint64_t)std::llrint(std::ldexp(c, k)); }
@@ -71,7 +71,7 @@ int fx_grid(int occ, uint64_t n, int pairs, int max_ctas, int* nblk, int* L, uin
   return QMC_OK;
 }
 
-int fx_pairs(int m) { return (std::min(m, kMcMax) + 1) / 2; }
+int fx_pairs(int m) { return (std::min(m, kMcMax) + kFxRows - 1) / kFxRows; }
 
 const void* fx_kernel(int d, int tr) {
   switch (d) {
@@ -92,7 +92,7 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
   // U^-2 F^-1, deg U <= 1, deg F <= 2, d <= 8, no negative coefficient, the
   // constant terms within kFxRange of the coefficient sums
   if (f->kind != QMC_F_SECTOR || f->precision != QMC_FP64 || f->aU != -2 || f->aF != -1 || d > kDFast ||
-      tune.force_general || tune.L > 0 || (t.kind == QMC_TRANSFORM_KOROBOV && t.alpha != 3) ||
+      tune.force_general || tune.no_fx || tune.L > 0 || (t.kind == QMC_TRANSFORM_KOROBOV && t.alpha != 3) ||
       poly_degree(f->U, d) > 1 || poly_degree(f->F, d) > 2 || !poly_positive(f->U, d) || !poly_positive(f->F, d))
     return QMC_EUNSUPPORTED;
   const std::vector<double> cu = pack_dense(f->U, d, 1), cf = pack_dense(f->F, d, 2);
@@ -107,23 +107,32 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
   base.d = d;
   base.tr = tr;
   fx_lattice(base, n, g);
-  // recentring constants of the dot products: both floors, and the mean of the
-  // dropped low-word products (low words of the coordinates uniform)
-  base.u0 = fx_fixed(cu[0], ku - 1);
-  base.uk = 1ull << 32;
+  // What the sums drop on average, in their own units: a dot product the
+  // fraction of its cross sum (1/2), per term the last four bits of the
+  // coordinate (7.5 of 16 against the coefficient's high word) and the low words'
+  // product; F per row half of that (z_i is 1/2 on average) and 1.25 of its product.
+  const auto dropped = [](uint32_t ch, uint32_t cl) {
+    return 7.5 * std::ldexp((double)ch, -32) + 0.5 * std::ldexp((double)cl, -28);
+  };
+  double lost = 0.5;
   for (int i = 0; i < d; ++i) {
     fx_split(cu[1 + i], ku, &base.uh[i], &base.ul[i]);
-    base.uk += 4ull * base.ul[i];
+    lost += dropped(base.uh[i], base.ul[i]);
   }
-  base.f0 = fx_fixed(cf[0], kf - 2);
+  base.u0 = fx_fixed(cu[0], ku - 1) + (uint64_t)std::llrint(lost);
+  lost = 0.0;
   for (int i = 0, off = 1, o = 0; i < d; ++i) {
     base.fl[i] = fx_fixed(cf[off++], kf - 1);
-    base.fk[i] = 1ull << 32;
+    base.fmask[i] = base.fl[i] ? 1u : 0u;
+    double row = 0.5;
     for (int j = i; j < d; ++j, ++o) {
       fx_split(cf[off++], kf, &base.fh[o], &base.fq[o]);
-      base.fk[i] += 4ull * base.fq[o];
+      if (base.fh[o] | base.fq[o]) base.fmask[i] |= 2u << (j - i);
+      row += dropped(base.fh[o], base.fq[o]);
     }
+    if (base.fmask[i]) lost += 0.25 * row + 0.75;
   }
+  base.f0 = fx_fixed(cf[0], kf - 2) + (uint64_t)std::llrint(lost);
   // value = v 2^(2 su + sf) 2^(2 ku + kf - 252), the smallest shift 2 su + sf
   // taken out; Korobov: v carries 4 more bits, and its weights are (4x(1-x))^3
   // against Eq. (5)'s 140 (x(1-x))^3
@@ -132,7 +141,8 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
 
   int occ = 0, nblk = 0, L = 0;
   uint64_t tiles = 0;
-  int rc = grid_occupancy(func, 0, tune.occupancy, occ);
+  // three CTAs of 8 warps saturate an SM's issue slots
+  int rc = grid_occupancy(func, 0, tune.occupancy > 0 ? std::min(tune.occupancy, 3) : 3, occ);
   if (rc) return rc;
   rc = fx_grid(occ, n, fx_pairs(m), tune.max_ctas, &nblk, &L, &tiles);
   if (rc) return rc;
@@ -153,7 +163,7 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
     fx_shifts(P, shifts);
     Launch ln;
     ln.func = func;
-    ln.grid = dim3(nblk, (P.m_launch + 1) / 2);
+    ln.grid = dim3(nblk, fx_pairs(P.m_launch));
     ln.params.resize(sizeof(P));
     std::memcpy(ln.params.data(), &P, sizeof(P));
     pl->launches.push_back(std::move(ln));

@@ -3,8 +3,8 @@
 // What bounds it.  This part issues 2 FP64 operations per SM and clock, and a
 // sector value under FP64 takes 39 (d = 6, baker) to 170 (d = 8, Korobov 3) of
 // them: the double kernels sat on that pipe.  A 32x32 -> 64-bit multiply-add
-// runs at 62 per SM and clock, three of them make a 64-bit high product, so the
-// whole value is evaluated in integers: coordinates, U, F, the reciprocal, the
+// runs at 32 per SM and clock (four issue slots of 128), three of them make a
+// 64-bit high product, so the whole value is evaluated in integers: coordinates, U, F, the reciprocal, the
 // transform weight and the sum.  No FP64 instruction is left in the loop.
 //
 // Formats (unsigned fractions; Qk holds x 2^k).  Coordinates z are Q63.  The
@@ -20,13 +20,17 @@
 // coefficient sums, so the host admits polynomials whose constant term is at
 // least 1/1000 of that sum (kFxRange): the relative error then stays at or
 // below the double chains' 2^-53 per operation, and coordinates (63 bits
-// against 52) and sums (exact) are finer.  Truncated products are recentred: a
-// constant worth the mean of the dropped part enters each, so errors do not
-// add up in one direction.
+// against 52) and sums (exact) are finer.  Products drop their fractions; the
+// mean of what U and F lose goes into their constant terms.
 //
-// Measured (GB300): d = 6, baker, n = 1000003, m = 32: 2.82 -> 0.59 ms; d = 8,
-// Korobov 3, n = 4194301, m = 16: 20.4 -> 3.20 ms; per-shift values within
+// Measured (GB300): d = 6, baker, n = 1000003, m = 32: 2.82 -> 0.55 ms; d = 8,
+// Korobov 3, n = 4194301, m = 16: 20.4 -> 2.96 ms; per-shift values within
 // 2e-16 of a 64-bit evaluation on both sides.
+//
+// What bounds it now: issue slots, 78 multiply-adds of four and 295 others a value
+// at d = 6.  Tried: one row per CTA (d = 8: 4.47 ms), three CTAs per SM at 80
+// registers (no gain), every slot of F without the mask (d = 8: 3.03 against
+// 3.08 ms, but batches of sparse sectors 4.31 against 4.16 ms).
 //
 // Rows of two shifts are evaluated side by side (independent chains); a CTA
 // takes one pair of shift rows, so few shifts on a small lattice still spread
@@ -40,21 +44,38 @@ namespace qmc {
 constexpr int kFxShiftMin = 7;        // 2 su + sf of the largest U < 2^62 and F < 2^61 (leading zeros 2 and 3)
 constexpr double kFxRange = 1000.0;   // largest (coefficient sum) / (constant term) of U and of F
 
-// a b / 2^64 + c; the truncation (the dropped low words' product and the two
-// floors, 1.25 units on average) is recentred
-__host__ __device__ __forceinline__ uint64_t fx_mulhi_add(uint64_t a, uint64_t b, uint64_t c) {
+// a b + c, one multiply-add (spelled out: as a plain expression the compiler
+// splits sums of such products into products and adds)
+__host__ __device__ __forceinline__ uint64_t fx_mad(uint32_t a, uint32_t b, uint64_t c) {
+#ifdef __CUDA_ARCH__
+  uint64_t r;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
+  return (uint64_t)a * b + c;
+#endif
+}
+
+// a b / 2^64 + c, the low words' product and the fractions of the cross products
+// dropped (1.25 units on average, which k = 1.25 2^32 puts back)
+__host__ __device__ __forceinline__ uint64_t fx_mulhi_add(uint64_t a, uint64_t b, uint64_t c, uint64_t k = 0) {
   const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
-  const uint64_t t1 = (uint64_t)al * bh + 0x140000000ull;
+  const uint64_t t1 = k ? fx_mad(al, bh, k) : (uint64_t)al * bh;
   const uint64_t t2 = (uint64_t)ah * bl;
-  const uint64_t r = (uint64_t)ah * bh + c;
-  return r + (t1 >> 32) + (t2 >> 32);
+  return fx_mad(ah, bh, c) + (t1 >> 32) + (t2 >> 32);
+}
+
+// the same for a, b < 2^63 with a + b < 2^64: the cross products' sum fits 64 bits
+__host__ __device__ __forceinline__ uint64_t fx_mulhi63_add(uint64_t a, uint64_t b, uint64_t c) {
+  const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32), bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
+  const uint64_t t = fx_mad(ah, bl, (uint64_t)al * bh);
+  return fx_mad(ah, bh, c) + (t >> 32);
 }
 
 // a^2 / 2^64
 __host__ __device__ __forceinline__ uint64_t fx_sqr(uint64_t a) {
   const uint32_t al = (uint32_t)a, ah = (uint32_t)(a >> 32);
-  const uint64_t t = (uint64_t)al * ah + 0x60000000ull;  // half the cross term, recentred
-  return (uint64_t)ah * ah + (t >> 31);
+  return (uint64_t)ah * ah + (((uint64_t)al * ah) >> 31);
 }
 
 __host__ __device__ __forceinline__ int fx_clz(uint64_t a) {  // leading zeros, a >= 2^32
@@ -96,6 +117,11 @@ __host__ __device__ __forceinline__ uint64_t fx_recip(uint64_t y) {
   return (uint64_t)r0 * ((1u << 28) - (1u << 8)) + q1;
 }
 
+// a with all bits flipped where the 32-bit mask m is all ones
+__host__ __device__ __forceinline__ uint64_t fx_flip(uint64_t a, uint32_t m) {
+  return ((uint64_t)((uint32_t)(a >> 32) ^ m) << 32) | ((uint32_t)a ^ m);
+}
+
 // Transformed coordinate (Q63) of the 64-bit fraction X; under Korobov 3 the
 // factor 4x(1-x) (Q64) goes to u.  With v = |2x - 1|, u = 1 - v^2, Eq. (5)'s
 // polynomial for weight 3 is z = 1/2 +- v (16 + 8u + 6u^2 + 5u^3) / 32, all
@@ -105,39 +131,34 @@ __host__ __device__ __forceinline__ uint64_t fx_coord(uint64_t X, uint64_t& u) {
   if constexpr (TR == TR_NONE) {
     return X >> 1;
   } else if constexpr (TR == TR_BAKER) {
-    return X ^ (uint64_t)((int64_t)X >> 63);  // min(X, 2^64 - 1 - X) = 2^63 z
+    return fx_flip(X, (uint32_t)((int64_t)X >> 63));  // min(X, 2^64 - 1 - X) = 2^63 z
   } else {
-    const uint64_t low = ~(uint64_t)((int64_t)X >> 63);  // all ones on the lower half
-    const uint64_t v = (X + X) ^ low;
+    const uint32_t low = ~(uint32_t)((int64_t)X >> 63);  // all ones on the lower half
+    const uint64_t v = fx_flip(X + X, low);
     u = ~fx_sqr(v);
-    // (5u + 6) / 64 in Q64; the constants end in zero words
-    const uint32_t ul = (uint32_t)u, uh = (uint32_t)(u >> 32);
-    uint64_t h = (uint64_t)uh * 0x14000000u + 0x1800000000000000ull + (((uint64_t)ul * 0x14000000u) >> 32);
-    h = fx_mulhi_add(u, h, 0x2000000000000000ull);
-    // 16/64 less 2^-59, so that rounding cannot push z past 0 or 1
-    h = fx_mulhi_add(u, h, 0x4000000000000000ull - 32);
+    // (16 + 6u^2) / 64 + u (8 + 5u^2) / 64: one square and one product; the
+    // constant is two units low, so that u's last bit cannot push z past 0 or 1
+    const uint64_t q = fx_sqr(u) >> 6;
+    const uint64_t h = fx_mulhi_add(u, q * 4 + q + 0x2000000000000000ull,
+                                    (q * 2 + q) * 2 + (0x4000000000000000ull - 2));
     const uint64_t zv = fx_mulhi_add(v, h, 0);
-    return (zv ^ low) + 0x4000000000000000ull;
+    return fx_flip(zv, low) + 0x4000000000000000ull;
   }
 }
 
-// sum_j c_j z_j / 2^64 + c for constants c_j = (high word, low word / 8).  The
-// two cross-product sums stay below 2^64 because sum_j c_j < 2^63 and the low
-// words are 29 bits: no carry handling between terms, 3 multiply-adds each.
+// sum_j c_j z_j / 2^64 for constants c_j = (high word, low word / 16) with
+// sum_j c_j < 2^63 and z_j < 2^63: with 28-bit low words the cross products of
+// up to eight terms share one 64-bit sum, so a term is three multiply-adds and
+// nothing else.
 struct FxDot {
-  uint64_t hi, ta, tb;
-  __host__ __device__ __forceinline__ void start(uint64_t c, uint64_t k) {
-    hi = c;
-    ta = k;
-    tb = 0;
-  }
+  uint64_t hi, t;
   __host__ __device__ __forceinline__ void add(uint64_t z, uint32_t ch, uint32_t cl) {
-    const uint32_t zl = (uint32_t)z, zh = (uint32_t)(z >> 32);
-    hi += (uint64_t)zh * ch;
-    ta += (uint64_t)zl * ch;
-    tb += (uint64_t)zh * cl;
+    const uint32_t zl = (uint32_t)z >> 4, zh = (uint32_t)(z >> 32);
+    hi = fx_mad(zh, ch, hi);
+    t = fx_mad(zl, ch, t);
+    t = fx_mad(zh, cl, t);
   }
-  __host__ __device__ __forceinline__ uint64_t value() const { return hi + (ta >> 32) + (tb >> 29); }
+  __host__ __device__ __forceinline__ uint64_t value() const { return hi + (t >> 28); }
 };
 
 // NS weighted values at one point: v[s] 2^t[s] in units of value_scale.  TERM
@@ -146,7 +167,7 @@ struct FxDot {
 // precision; in the rule's sums the weight's 2^-64 absolute steps are below
 // the rounding of the sum's final conversion.
 template <int D, int TR, int NS, bool TERM = false>
-__host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint64_t* base, const int* rows,
+__host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint64_t* base, const uint64_t (*shift)[D],
                                                    uint64_t* v, int* t) {
   uint64_t z[NS][D], W[NS];
   int ew = 0;
@@ -155,7 +176,7 @@ __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
       uint64_t u = 0;
-      z[s][i] = fx_coord<TR>(base[i] + P.shift[rows[s]][i], u);
+      z[s][i] = fx_coord<TR>(base[i] + shift[s][i], u);
       if constexpr (TR == TR_KOROBOV) {
         if constexpr (TERM) {
           static_assert(NS == 1, "one term at a time");
@@ -172,7 +193,7 @@ __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint
   uint64_t U[NS], F[NS];
   FxDot dot[NS];
 #pragma unroll
-  for (int s = 0; s < NS; ++s) dot[s].start(P.u0, P.uk);
+  for (int s = 0; s < NS; ++s) dot[s] = FxDot{P.u0, 0};
 #pragma unroll
   for (int i = 0; i < D; ++i)
 #pragma unroll
@@ -182,17 +203,26 @@ __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint
     U[s] = dot[s].value();
     F[s] = P.f0;
   }
+  // F row by row; a bit per slot (the row's linear term first) tells which
+  // terms exist: a test and a branch (2 slots a pair of shifts) against 24
   int off = 0;
 #pragma unroll
   for (int i = 0; i < D; ++i) {
+    const uint32_t row = P.fmask[i];
+    if (row) {
 #pragma unroll
-    for (int s = 0; s < NS; ++s) dot[s].start(P.fl[i], P.fk[i]);
+      for (int s = 0; s < NS; ++s) dot[s] = FxDot{0, 0};
+      if (row & 1u)
 #pragma unroll
-    for (int j = i; j < D; ++j)
+        for (int s = 0; s < NS; ++s) dot[s].hi = P.fl[i];
 #pragma unroll
-      for (int s = 0; s < NS; ++s) dot[s].add(z[s][j], P.fh[off + j - i], P.fq[off + j - i]);
+      for (int j = i; j < D; ++j)
+        if (row & (2u << (j - i)))
 #pragma unroll
-    for (int s = 0; s < NS; ++s) F[s] = fx_mulhi_add(z[s][i], dot[s].value(), F[s]);
+          for (int s = 0; s < NS; ++s) dot[s].add(z[s][j], P.fh[off + j - i], P.fq[off + j - i]);
+#pragma unroll
+      for (int s = 0; s < NS; ++s) F[s] = fx_mulhi63_add(z[s][i], dot[s].value(), F[s]);
+    }
     off += D - i;
   }
 #pragma unroll
@@ -200,7 +230,7 @@ __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint
     const int su = fx_clz(U[s]), sf = fx_clz(F[s]);
     uint64_t r = fx_recip(fx_mulhi_add(fx_sqr(U[s] << su), F[s] << sf, 0));
     // the reciprocal is below 2^59: 4 more bits before the weight (0.2% on average at d = 8) takes them away
-    if constexpr (TR == TR_KOROBOV) r = fx_mulhi_add(r << 4, fx_mulhi_add(fx_sqr(W[s]), W[s], 0), 0);
+    if constexpr (TR == TR_KOROBOV) r = fx_mulhi_add(r << 4, fx_mulhi_add(fx_sqr(W[s]), W[s], 0), 0, 0x140000000ull);
     v[s] = r;
     t[s] = 2 * su + sf - kFxShiftMin - (TERM ? 3 * ew : 0);
   }
@@ -209,9 +239,8 @@ __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint
 // 128-bit sum
 struct FxSum {
   uint64_t lo, hi;
-  __host__ __device__ __forceinline__ void add(uint64_t l, uint64_t h) {
-    lo += l;
-    hi += h + (lo < l ? 1u : 0u);
+  __device__ __forceinline__ void add(uint64_t l, uint64_t h) {
+    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(lo), "+l"(hi) : "l"(l), "l"(h));
   }
 };
 
@@ -226,31 +255,34 @@ template <int D, int TR>
 __global__ void __launch_bounds__(kThreads)
     sector_fx_kernel(const __grid_constant__ FxParams P, double* __restrict__ partial,
                      unsigned long long* __restrict__ counters, const SampleIO sio) {
-  constexpr int NS = 2;
+  constexpr int NS = kFxRows;
   if (sio.count > 0) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= sio.count) return;
     const uint64_t j = sio.j[s];
     const int k = sio.k[s];
-    uint64_t base[D];
+    uint64_t base[D], sh[1][D];
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       const uint32_t idx = lattice_index(j, P.g[i], P.n);
       base[i] = frac64(idx, P.rc);
+      sh[0][i] = P.shift[k][i];
       if (sio.idx) sio.idx[(size_t)s * D + i] = idx;
       if (sio.coord) sio.coord[(size_t)s * D + i] = coord_used<double>(base[i] + P.shift[k][i]);
     }
     uint64_t v;
     int t;
-    fx_values<D, TR, 1, true>(P, base, &k, &v, &t);
+    fx_values<D, TR, 1, true>(P, base, sh, &v, &t);
     sio.values[2 * (size_t)s] = ldexp(__ull2double_rn(v), t) * P.value_scale;
     sio.values[2 * (size_t)s + 1] = 0.0;
     return;
   }
   const int r0 = blockIdx.y * NS;
-  int rows[NS];
+  uint64_t sh[NS][D];
 #pragma unroll
-  for (int s = 0; s < NS; ++s) rows[s] = r0 + s;
+  for (int s = 0; s < NS; ++s)
+#pragma unroll
+    for (int i = 0; i < D; ++i) sh[s][i] = P.shift[r0 + s][i];
   FxSum acc[NS];
 #pragma unroll
   for (int s = 0; s < NS; ++s) acc[s].lo = acc[s].hi = 0;
@@ -268,7 +300,7 @@ __global__ void __launch_bounds__(kThreads)
     for (int s = 0; s < steps; ++s) {
       uint64_t v[NS];
       int t[NS];
-      fx_values<D, TR, NS>(P, base, rows, v, t);
+      fx_values<D, TR, NS>(P, base, sh, v, t);
 #pragma unroll
       for (int q = 0; q < NS; ++q) acc[q].add(v[q] << t[q], __funnelshift_l((uint32_t)(v[q] >> 32), 0u, t[q]));
 #pragma unroll

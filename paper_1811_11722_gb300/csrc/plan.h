@@ -30,6 +30,7 @@ struct TuneChoice {
   bool no_jit = false; // keep the template kernel (no run-time specialisation)
   int max_ctas = 0;    // cap on CTAs of each launch (batched sectors run side by side)
   bool force_general = false;
+  bool no_fx = false;  // keep FP64 sectors on the double kernels
   int smacc = -1;      // specialised kernel: accumulator pairs in shared memory (1), registers (0),
                        // -1: the QMC_JIT_SMACC default
   int minb = 0;        // specialised kernel: minimum resident CTAs per SM in its launch bounds (0: none)
@@ -80,6 +81,7 @@ struct Plan {
                             // GeneralParams<float> (3), GeneralParams<double> (4), FxParams (5);
                             // 0: fixed lattice
   int grid_occ = 1;         // CTAs per SM the launch shape assumes
+  int grid_rows = 1;        // CTA rows of the largest launch, one per shift row (separable FP64), else 1
   bool grid_capped = true;  // the launch shape honours a cap on CTAs (rule plans; not deformed ones)
 };
 

@@ -146,6 +146,7 @@ __host__ __device__ inline void fill_pairs(RuleParams<R>& P, int d) {
     P.cp[nu + s] = make_float2(-(float)P.cF[s], -(float)P.cF[s]);
 }
 
+constexpr int kFxRows = 2;  // shift rows of a CTA of the fixed-point kernel
 // FP64 sectors in fixed point (fixed64.cuh): parameters of one launch, up to
 // kMcMax shift rows, two per CTA row.  Offsets of n, tiles and L as in RuleParams.
 struct FxParams {
@@ -162,10 +163,11 @@ struct FxParams {
   uint32_t g[kDFast];
   uint32_t step[kDFast][3];     // fraction (kThreads g_i mod n) / n to 96 bits, low word first
   uint64_t shift[kMcMax][kDFast];
-  uint64_t u0, uk;              // U: constant term in Q(k-1), recentring constant of its cross terms
-  uint32_t uh[kDFast], ul[kDFast];  // linear coefficients: high word; low word / 8
+  uint64_t u0;                  // U: constant term in Q(k-1)
+  uint32_t uh[kDFast], ul[kDFast];  // linear coefficients: high word; low word / 16
   uint64_t f0;                  // F: constant term in Q(k-2)
-  uint64_t fl[kDFast], fk[kDFast];  // rows: linear coefficient in Q(k-1), recentring constant
+  uint64_t fl[kDFast];          // rows: linear coefficient in Q(k-1)
+  uint32_t fmask[kDFast];       // rows: bit 0 linear term, bit 1 + j - i the term q_ij
   uint32_t fh[kDFast * (kDFast + 1) / 2], fq[kDFast * (kDFast + 1) / 2];  // q_ij, row by row
 };
 
