@@ -381,6 +381,14 @@ int grid_shape(int occ, uint64_t n, int max_ctas, int fixed_L, int& nblk, int& L
   return QMC_OK;
 }
 
+// The cap on a launch's CTA columns: with one CTA row per shift row, the rows
+// share the resident wave (a caller's cap stays one per row).
+static int rows_cap(const Plan* pl, int occ, int max_ctas) {
+  if (pl->grid_rows <= 1) return max_ctas;
+  const int cap = std::max(1, device_sm_count() * std::max(occ, 1) / pl->grid_rows);
+  return max_ctas > 0 ? std::min(max_ctas, cap) : cap;
+}
+
 int choose_grid(const void* func, size_t smem, uint64_t n, int& nblk, int& L, uint64_t& tiles,
                 int occupancy_override) {
   int occ = 0;
@@ -540,8 +548,20 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
     return fail(QMC_EUNSUPPORTED, "deformed sector integrands are served by the complex kernels");
   } else {
     int fk = f->kind == QMC_F_CONST ? FK_CONST : (f->kind == QMC_F_SEPARABLE_EXP ? FK_SEPEXP : FK_TRIG);
-    mc = 8;
-    func = separable_ptr(fp32, base.tr, fk);
+    func = separable_ptr(fp32, base.tr, base.alpha, fk);
+    if (fp32) {
+      mc = 8;
+    } else {  // one shift row per CTA row, up to kMcMax rows a launch
+      mc = kMcMax;
+      pl->grid_rows = std::min(m, kMcMax);
+      if (base.tr != TR_KOROBOV || base.alpha == 3) {  // fixed-point coordinates 2^63 z
+        for (int i = 0; i < d; ++i) {
+          base.sep_c[i] = std::ldexp((double)base.sep_c[i], -63);
+          base.sep_b[i] = std::ldexp((double)base.sep_b[i], -63);
+        }
+        if (base.tr == TR_KOROBOV) base.value_scale = korobov_scale(kKorCentred, d);
+      }
+    }
     if (!func) return fail(QMC_EUNSUPPORTED, "no separable kernel for this transform");
   }
 
@@ -575,7 +595,7 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
                                  : tune.occupancy,
                           occ);
   if (rc) return rc;
-  rc = grid_shape(occ, n, tune.max_ctas, tune.L, nblk, L, tiles);
+  rc = grid_shape(occ, n, rows_cap(pl, occ, tune.max_ctas), tune.L, nblk, L, tiles);
   if (rc) return rc;
   pl->param_kind = general ? (fp32 ? 3 : 4) : (fp32 ? 1 : 2);
   pl->grid_occ = occ;
@@ -604,7 +624,7 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
     ln.func = func;
     ln.cufunc = jit_fn;
     ln.smem = jit_fn ? jit_smem : 0;
-    ln.grid = dim3(nblk);
+    ln.grid = dim3(nblk, pl->grid_rows > 1 ? mk : 1);
     ln.params.resize(pbytes);
     if (general) {
       gp.base = P;
@@ -671,7 +691,7 @@ int plan_build(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, co
   } else if (f->precision == QMC_FP32EVAL) {
     rc = build_rule_plan<float>(pl, d, n, m, g, shifts, t, f, tune, eps);
   } else {
-    // sectors in fixed point where the integrand allows it (4.8-6.4x the double kernels)
+    // sectors in fixed point where the integrand allows it (5-7x the double kernels)
     rc = eps ? QMC_EUNSUPPORTED : build_fx_plan(pl, d, n, m, g, shifts, t, f, tune);
     if (rc == QMC_EUNSUPPORTED) rc = build_rule_plan<double>(pl, d, n, m, g, shifts, t, f, tune, eps);
   }
@@ -700,7 +720,8 @@ int plan_rebase(Plan* pl, uint64_t n, const uint64_t* g, int max_ctas) {
   if (pl->param_kind == 5) return fx_rebase(pl, n, g, max_ctas);
   int nblk = 0, L = 0;
   uint64_t tiles = 0;
-  int rc = grid_shape(pl->grid_occ, n, pl->grid_capped ? max_ctas : 0, pl->tune.L, nblk, L, tiles);
+  int rc = grid_shape(pl->grid_occ, n, rows_cap(pl, pl->grid_occ, pl->grid_capped ? max_ctas : 0), pl->tune.L, nblk, L,
+                      tiles);
   if (rc) return rc;
   for (Launch& ln : pl->launches) {
     uint8_t* p = ln.params.data();
@@ -710,7 +731,7 @@ int plan_rebase(Plan* pl, uint64_t n, const uint64_t* g, int max_ctas) {
       case 3: rebase_rule(reinterpret_cast<GeneralParams<float>*>(p)->base, pl->d, n, g, nblk, L, tiles); break;
       default: rebase_rule(reinterpret_cast<GeneralParams<double>*>(p)->base, pl->d, n, g, nblk, L, tiles); break;
     }
-    ln.grid = dim3(nblk);
+    ln.grid.x = nblk;
   }
   pl->n = n;
   pl->nblk = nblk;
@@ -1100,7 +1121,7 @@ int qmc_plan_describe(qmc_plan plan, char* buf, int32_t len) {
            "d=%d n=%llu m=%d complex=%d orders=%d shifts_per_launch=%d launches=%zu specialised=%d ctas=%d L=%d "
            "smem_acc=%d min_ctas=%d imm_shifts=%d",
            pl->d, (unsigned long long)pl->n, pl->m, pl->is_complex, pl->orders, pl->mc, pl->launches.size() + 1,
-           (ln && ln->cufunc) ? 1 : 0, pl->nblk, L, (ln && ln->smem) ? 1 : 0, pl->tune.minb,
+           (ln && ln->cufunc) ? 1 : 0, ln ? (int)(ln->grid.x * ln->grid.y) : pl->nblk, L, (ln && ln->smem) ? 1 : 0, pl->tune.minb,
            (ln && ln->cufunc) ? pl->imm : 0);
   return QMC_OK;
 }

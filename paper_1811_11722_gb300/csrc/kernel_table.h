@@ -59,14 +59,14 @@ QMC_DECL_DEF(double, 1) QMC_DECL_DEF(double, 2) QMC_DECL_DEF(double, 3) QMC_DECL
 QMC_DECL_DEF(double, 5) QMC_DECL_DEF(double, 6) QMC_DECL_DEF(double, 7) QMC_DECL_DEF(double, 8)
 #undef QMC_DECL_DEF
 
-// Separable integrands (const / separable exp / trig), runtime d and
-// Korobov weight (factors normalised, value scale 1).
+// Separable integrands (const / separable exp / trig), runtime d and Korobov
+// weight alpha.
 template <typename R>
-const void* separable_ptr_t(int tr, int fk);
-template <> const void* separable_ptr_t<float>(int tr, int fk);
-template <> const void* separable_ptr_t<double>(int tr, int fk);
-inline const void* separable_ptr(bool fp32, int tr, int fk) {
-  return fp32 ? separable_ptr_t<float>(tr, fk) : separable_ptr_t<double>(tr, fk);
+const void* separable_ptr_t(int tr, int alpha, int fk);
+template <> const void* separable_ptr_t<float>(int tr, int alpha, int fk);
+template <> const void* separable_ptr_t<double>(int tr, int alpha, int fk);
+inline const void* separable_ptr(bool fp32, int tr, int alpha, int fk) {
+  return fp32 ? separable_ptr_t<float>(tr, alpha, fk) : separable_ptr_t<double>(tr, alpha, fk);
 }
 
 // General sparse-polynomial sector kernel, runtime d, transform and powers.

@@ -1,4 +1,4 @@
-"""The fixed-point FP64 sector kernel against the oracle where it can go wrong:
+"""The fixed-point FP64 kernels (sectors, separable integrands) against the oracle where they can go wrong:
 every dimension and transform, ragged tiles and odd shift counts, coefficients
 that use all 53 bits, constant terms at both sides of the range the kernel
 takes, single terms with tiny weights.
@@ -95,3 +95,25 @@ def test_moves_with_the_walk(Q):
         q = dataclasses.replace(p, n=n, g=g[:p.d] % n)
         d, _ = Q.qmc_integrate(q.d, n, m, q.g, q.shifts, Q.transform("korobov", 3), Q.integrand_from_problem(q, "fp64"))
         assert abs(r.mean[0] - d.mean[0]) <= 1e-15 * abs(d.mean[0])
+
+
+@pytest.mark.parametrize("kind", ["const", "separable_exp", "trig"])
+@pytest.mark.parametrize("transform,alpha", [("none", 0), ("baker", 0), ("korobov", 3), ("korobov", 5)])
+@pytest.mark.parametrize("d,n,m", [(1, 2, 2), (3, 257, 33), (7, 10007, 5), (16, 65537, 40)])
+def test_separable(Q, oracle_lib, nthreads, kind, transform, alpha, d, n, m):
+    """Sums of both signs (trig) are held to the largest term: 1 without a
+    weight, Eq. (5)'s largest weight (35/16 at alpha = 3, 2.71 at 5) to the power d with one,
+    over sqrt(n) terms' worth of rounding and never below one."""
+    rng = I.SplitMix64(n + 7 * d)
+    p = I.Problem("sep", d, n, m, I.make_shifts(rng, m, d), transform, alpha=alpha, kind=kind,
+                  c=np.array([rng.uniform_in(-0.5, 1.0) for _ in range(d)]),
+                  b=np.array([rng.uniform_in(-0.5, 0.5) for _ in range(d)]),
+                  h=np.array([rng.randint(-3, 3) for _ in range(d)], dtype=np.int32),
+                  g=I.random_generating_vector(rng, d, n))
+    f = Q.integrand_from_problem(p, "fp64")
+    res, ps = Q.qmc_integrate(d, n, m, p.g, p.shifts, Q.transform(transform, alpha), f, want_per_shift=True)
+    ref = oracle_lib.integrate(p, p.g, nthreads=nthreads)
+    assert res.status == 0 and res.nonfinite == 0
+    top = {0: 1.0, 3: 35.0 / 16.0, 5: 2.71}[alpha] ** d / np.sqrt(n) if kind == "trig" else 0.0
+    tol = 20 * (d + 2) * 2.0 ** -53
+    assert np.all(np.abs(ps[:, 0] - ref["q"][:, 0]) <= tol * np.maximum(np.abs(ref["q"][:, 0]), max(top, 1.0) if kind == "trig" else 0.0))
