@@ -383,7 +383,7 @@ int grid_shape(int occ, uint64_t n, int max_ctas, int fixed_L, int& nblk, int& L
 
 // The cap on a launch's CTA columns: with one CTA row per shift row, the rows
 // share the resident wave (a caller's cap stays one per row).
-static int rows_cap(const Plan* pl, int occ, int max_ctas) {
+int rows_cap(const Plan* pl, int occ, int max_ctas) {
   if (pl->grid_rows <= 1) return max_ctas;
   const int cap = std::max(1, device_sm_count() * std::max(occ, 1) / pl->grid_rows);
   return max_ctas > 0 ? std::min(max_ctas, cap) : cap;

@@ -16,18 +16,52 @@ static bool deformed_packed_enabled() {
 }
 
 // The packed FP32 variant (two shifts per instruction), d <= kDef2DMax.
+template <int ALPHA>
 static const void* deformed2_ptr(int d) {
   switch (d) {
-    case 1: return (const void*)&deformed2_kernel<1>;
-    case 2: return (const void*)&deformed2_kernel<2>;
-    case 3: return (const void*)&deformed2_kernel<3>;
-    case 4: return (const void*)&deformed2_kernel<4>;
-    case 5: return (const void*)&deformed2_kernel<5>;
+    case 1: return (const void*)&deformed2_kernel<1, ALPHA>;
+    case 2: return (const void*)&deformed2_kernel<2, ALPHA>;
+    case 3: return (const void*)&deformed2_kernel<3, ALPHA>;
+    case 4: return (const void*)&deformed2_kernel<4, ALPHA>;
+    case 5: return (const void*)&deformed2_kernel<5, ALPHA>;
     default: return nullptr;
   }
 }
 
-constexpr int kMcDef = 8;  // shifts per launch (matches the kernel's shared accumulators)
+// Shifts per launch: the general kernel's shared accumulators; the FAST
+// kernels with a CTA row per shift row (FP64) or pair of rows (packed FP32).
+static_assert(kMcDeformed == 8, "shared accumulators");
+
+// det(H_off restricted to the bit set S) by expansion along its first row.
+static double minor_off(const std::vector<double>& H, int d, unsigned S, unsigned cols) {
+  if (!S) return 1.0;
+  int r = 0;
+  while (!(S >> r & 1u)) ++r;
+  double det = 0.0, sign = 1.0;
+  for (int c = 0; c < d; ++c) {
+    if (!(cols >> c & 1u)) continue;
+    if (c != r && H[(size_t)r * d + c] != 0.0)
+      det += sign * H[(size_t)r * d + c] * minor_off(H, d, S & ~(1u << r), cols & ~(1u << c));
+    sign = -sign;
+  }
+  return det;
+}
+
+// DefTab's constants.
+static std::vector<double> fast_table(const std::vector<double>& cf, int d, double lambda) {
+  std::vector<double> H((size_t)d * d, 0.0), t;
+  t.push_back(cf[0]);
+  for (int k = 0, off = 1; k < d; ++k) {
+    t.push_back(cf[off++]);
+    for (int l = k; l < d; ++l, ++off) H[(size_t)k * d + l] = H[(size_t)l * d + k] = (k == l ? 2.0 : 1.0) * cf[off];
+  }
+  for (int k = 0; k < d; ++k)
+    for (int l = k; l < d; ++l) t.push_back(H[(size_t)k * d + l]);
+  for (int k = 0; k < d; ++k) t.push_back(0.5 * H[(size_t)k * d + k]);
+  for (unsigned S = 0; S < (1u << d); ++S) t.push_back(minor_off(H, d, S, S));
+  for (double v : {lambda, -lambda, 2.0 * lambda, 0.5}) t.push_back(v);
+  return t;
+}
 
 // Offset of q_ij (i <= j) in the nested degree-2 layout (host copy of q_off).
 static int q_off_host(int D, int i, int j) {
@@ -72,43 +106,52 @@ static int build_def(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
 #undef QMC_D_CASE
     default: break;
   }
-  if (packed) func = deformed2_ptr(d);
+  // FP32 packed: the coordinate's form by the integrand's range, as for the sectors
+  const int form = packed ? korobov_form(d, pack_dense(f->U, d, 1), cf) : 3;
+  if (packed) func = form == kKorCentred ? deformed2_ptr<kKorCentred>(d) : deformed2_ptr<3>(d);
+  const bool tab = fast && d <= kDefFastMax;
+  const bool rows64 = tab && sizeof(R) == 8;  // a CTA row per shift row
   if (!func) return fail(QMC_EUNSUPPORTED, "no deformed kernel for d=%d", d);
   auto cu = pack_dense(f->U, d, u_linear ? 1 : 2);
   for (size_t i = 0; i < cu.size(); ++i) base.cU[i] = (R)cu[i];
-  for (size_t i = 0; i < cf.size(); ++i) base.cF[i] = (R)cf[i];
-  for (int k = 0; k < d; ++k)  // -lambda d2F/dy_k dy_l (constant: F has degree 2)
-    for (int l = 0; l < d; ++l) {
-      const int a = k < l ? k : l, b = k < l ? l : k;
-      const double h = (k == l ? 2.0 : 1.0) * cf[q_off_host(d, a, b)];
-      base.cF[kDefHessOff + k * d + l] = (R)(-f->lambda * h);
+  if (tab) {
+    const std::vector<double> t = fast_table(cf, d, f->lambda);
+    static_assert(DefTab<kDefFastMax>::END <= kPolyCoefMax && DefTab<kDef2DMax>::END + 1 + kDef2DMax <= kPairCoefMax,
+                  "deformed constants");
+    if (packed) {
+      int o = 0;
+      for (double v : t) base.cp[o++] = make_float2((float)v, (float)v);
+      for (double v : cu) base.cp[o++] = make_float2((float)v, (float)v);
+    } else {
+      for (size_t i = 0; i < t.size(); ++i) base.cF[i] = (R)t[i];
     }
-  if (packed) {  // (c, c) pairs: U's linear slots, F's slots, then the Hessian of F, k-major
-    int o = 0;
-    for (size_t i = 0; i < cu.size(); ++i, ++o) base.cp[o] = make_float2((float)cu[i], (float)cu[i]);
-    for (size_t i = 0; i < cf.size(); ++i, ++o) base.cp[o] = make_float2((float)cf[i], (float)cf[i]);
-    for (int k = 0; k < d; ++k)
-      for (int l = 0; l < d; ++l, ++o) {
+  } else {
+    for (size_t i = 0; i < cf.size(); ++i) base.cF[i] = (R)cf[i];
+    for (int k = 0; k < d; ++k)  // -lambda d2F/dy_k dy_l (constant: F has degree 2)
+      for (int l = 0; l < d; ++l) {
         const int a = k < l ? k : l, b = k < l ? l : k;
-        const float h = (float)((k == l ? 2.0 : 1.0) * cf[q_off_host(d, a, b)]);
-        base.cp[o] = make_float2(h, h);
+        const double h = (k == l ? 2.0 : 1.0) * cf[q_off_host(d, a, b)];
+        base.cF[kDefHessOff + k * d + l] = (R)(-f->lambda * h);
       }
-    if (o > kPairCoefMax) return fail(QMC_EUNSUPPORTED, "deformed: %d coefficient pairs", o);
   }
-  // Transform weight constants.  FP64 normalises each factor in the kernel.
-  // FP32 FAST multiplies the factors u and cubes the product: (2a+1)!/(a!)^2
-  // = 140 per dimension remains; other FP32 Korobov plans raise the product of
-  // the factors 4u to the power alpha: ((2a+1)!/(a!)^2 / 4^a) per dimension.
+  // Transform weight constants.  FP64 normalises each factor in the general
+  // kernel; its FAST kernel cubes the product of 4x(1-x) in units of 2^-64.
+  // FP32 FAST cubes the product of its form's factors; other FP32 Korobov plans
+  // raise the product of the factors 4u to the power alpha: ((2a+1)!/(a!)^2 /
+  // 4^a) per dimension.
   base.value_scale = 1.0;
-  if (sizeof(R) == 4 && base.tr == TR_KOROBOV)
-    base.value_scale = fast ? std::pow((double)base.kor[7], (double)d)
+  if (fast && sizeof(R) == 8) base.value_scale = korobov_scale(kKorCentred, d) * 0x1p-192;
+  else if (sizeof(R) == 4 && base.tr == TR_KOROBOV)
+    base.value_scale = fast ? korobov_scale(form, d)
                             : std::pow((double)base.kor[7] / std::pow(4.0, (double)base.alpha), (double)d);
   base.check_finite = 1;
   int nblk = 0, L = 0, occ = 0;
   uint64_t tiles = 0;
   int rc = grid_occupancy(func, 0, tune.occupancy, occ);
   if (rc) return rc;
-  rc = grid_shape(occ, n, 0, tune.L, nblk, L, tiles);
+  const int mc = packed || rows64 ? kMcMax : kMcDeformed;
+  pl->grid_rows = packed ? (std::min(m, kMcMax) + 1) / 2 : (rows64 ? std::min(m, kMcMax) : 1);
+  rc = grid_shape(occ, n, rows_cap(pl, occ, 0), tune.L, nblk, L, tiles);
   if (rc) return rc;
   pl->param_kind = sizeof(R) == 4 ? 1 : 2;
   pl->grid_occ = occ;
@@ -118,22 +161,20 @@ static int build_def(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
   base.nblk = nblk;
   pl->nblk = nblk;
   pl->func = func;
-  pl->mc = kMcDef;
+  pl->mc = mc;
   pl->final_scale = base.value_scale;
   pl->is_complex = 1;
-  for (int k0 = 0; k0 < m; k0 += kMcDef) {
-    const int mk = std::min(kMcDef, m - k0);
+  for (int k0 = 0; k0 < m; k0 += mc) {
+    const int mk = std::min(mc, m - k0);
     RuleParams<R> P = base;
     P.m_launch = mk;
     P.k_base = k0;
-    for (int kk = 0; kk < mk; ++kk)
-      for (int i = 0; i < d; ++i) {
-        uint64_t s64 = shift_fixed64(shifts[(size_t)(k0 + kk) * d + i]);
-        set_shift(P, kk, i, s64);
-      }
+    for (int kk = 0; kk < mc; ++kk)  // rows mk.. repeat row k0 (evaluated at most, never written back)
+      for (int i = 0; i < d; ++i)
+        set_shift(P, kk, i, shift_fixed64(shifts[(size_t)(kk < mk ? k0 + kk : k0) * d + i]));
     Launch ln;
     ln.func = func;
-    ln.grid = dim3(nblk);
+    ln.grid = dim3(nblk, packed ? (mk + 1) / 2 : (rows64 ? mk : 1));
     ln.params.resize(sizeof(P));
     std::memcpy(ln.params.data(), &P, sizeof(P));
     pl->launches.push_back(std::move(ln));

@@ -26,6 +26,12 @@ __device__ __forceinline__ uint64_t frac64(uint32_t idx, const Recip& rc) {
   return (uint64_t)idx * rc.rhi + __umul64hi((uint64_t)idx, rc.rlo);
 }
 
+// The fraction of j g / n in 64 bits, within 2 units: j times the fraction of
+// g / n held to 128 bits (within 2^-97), so no 64-bit division by n.
+__device__ __forceinline__ uint64_t point_frac64(uint32_t j, uint32_t g, const Recip& rc) {
+  return frac64(j, Recip{(uint64_t)g * rc.rhi + __umul64hi((uint64_t)g, rc.rlo), (uint64_t)g * rc.rlo});
+}
+
 // Round the 64-bit fraction to 32 bits.
 __device__ __forceinline__ uint32_t frac32(uint64_t p64) {
   return (uint32_t)((p64 + 0x80000000ull) >> 32);
@@ -326,7 +332,7 @@ __device__ __forceinline__ float coord_fx(uint32_t X, const float* kor, float& w
 // coord_fx for two shifts at once: the same operations per lane (so the same
 // values bit for bit) in packed f32x2 arithmetic; w holds the two products
 // of the Korobov factors.
-template <int TR, int ALPHA>
+template <int TR, int ALPHA, bool CLAMP = false>
 __device__ __forceinline__ float2 coord_fx2(uint32_t Xa, uint32_t Xb, const float* kor, float2& w) {
   if constexpr (TR == TR_NONE) {
     return make_float2(__uint2float_rn(Xa), __uint2float_rn(Xb));
@@ -337,7 +343,9 @@ __device__ __forceinline__ float2 coord_fx2(uint32_t Xa, uint32_t Xb, const floa
     q = fma2(q, u, make_float2(8 * 0x1p-36f, 8 * 0x1p-36f));
     q = fma2(q, u, make_float2(16 * 0x1p-36f, 16 * 0x1p-36f));
     w = mul2(w, u);
-    return fma2(T, q, make_float2(0.5f, 0.5f));
+    if constexpr (CLAMP)
+      return make_float2(__saturatef(__fmaf_rn(T.x, q.x, 0.5f)), __saturatef(__fmaf_rn(T.y, q.y, 0.5f)));
+    else return fma2(T, q, make_float2(0.5f, 0.5f));
   } else {
     const float2 a = make_float2(fabsf(__int2float_rn((int32_t)Xa)), fabsf(__int2float_rn((int32_t)Xb)));
     if constexpr (TR == TR_BAKER) {

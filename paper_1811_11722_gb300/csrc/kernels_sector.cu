@@ -64,10 +64,15 @@ const void* eps_ptr<QMC_REAL, QMC_D>(int ne, int tr) {
 
 template <>
 const void* deformed_ptr<QMC_REAL, QMC_D>(bool fast, bool u_linear) {
+  if constexpr (sizeof(QMC_REAL) == 8 && QMC_D <= kDefFastMax) {  // FP64: its own kernel
+    if (fast)
+      return u_linear ? (const void*)&deformed64_kernel<QMC_D, 1> : (const void*)&deformed64_kernel<QMC_D, 2>;
+  }
+  constexpr bool kFast = sizeof(QMC_REAL) == 4 || QMC_D > kDefFastMax;
   if (u_linear)
-    return fast ? (const void*)&deformed_kernel<QMC_REAL, QMC_D, true, 1>
+    return fast ? (const void*)&deformed_kernel<QMC_REAL, QMC_D, kFast, 1>
                 : (const void*)&deformed_kernel<QMC_REAL, QMC_D, false, 1>;
-  return fast ? (const void*)&deformed_kernel<QMC_REAL, QMC_D, true, 2>
+  return fast ? (const void*)&deformed_kernel<QMC_REAL, QMC_D, kFast, 2>
               : (const void*)&deformed_kernel<QMC_REAL, QMC_D, false, 2>;
 }
 

@@ -81,7 +81,8 @@ struct Plan {
                             // GeneralParams<float> (3), GeneralParams<double> (4), FxParams (5);
                             // 0: fixed lattice
   int grid_occ = 1;         // CTAs per SM the launch shape assumes
-  int grid_rows = 1;        // CTA rows of the largest launch, one per shift row (separable FP64), else 1
+  int grid_rows = 1;        // CTA rows of the largest launch, one per shift row or pair (separable FP64,
+                            // deformed FAST kernels), else 1
   bool grid_capped = true;  // the launch shape honours a cap on CTAs (rule plans; not deformed ones)
 };
 
@@ -101,6 +102,7 @@ uint64_t shift_fixed64(double delta);
 int choose_grid(const void* func, size_t smem, uint64_t n, int& nblk, int& L, uint64_t& tiles,
                 int occupancy_override);
 int grid_occupancy(const void* func, size_t smem, int occupancy_override, int& occ);
+int rows_cap(const Plan* pl, int occ, int max_ctas);
 int grid_shape(int occ, uint64_t n, int max_ctas, int fixed_L, int& nblk, int& L, uint64_t& tiles);
 // Move a built plan to the lattice (n, g) of the same dimension: lattice
 // fields and launch shape of every launch (max_ctas as TuneChoice::max_ctas);
