@@ -856,12 +856,23 @@ int plan_execute(Plan* pl, qmc_result* out, double* per_shift, cudaStream_t stre
                        (per_shift && ps_dev) ? per_shift : (per_shift ? pl->ws.per_shift : nullptr), stream);
   if (rc) return rc;
   const size_t G = (size_t)pl->orders;
-  if (!out_dev) QMC_CUDA(cudaMemcpyAsync(out, pl->ws.result, G * sizeof(qmc_result), cudaMemcpyDeviceToHost, stream));
-  if (per_shift && !ps_dev)
-    QMC_CUDA(cudaMemcpyAsync(per_shift, pl->ws.per_shift, G * pl->m * 2 * sizeof(double),
-                             cudaMemcpyDeviceToHost, stream));
-  if (!out_dev || (per_shift && !ps_dev)) {
-    QMC_CUDA(cudaStreamSynchronize(stream));
+  const size_t res_bytes = G * sizeof(qmc_result), ps_bytes = G * pl->m * 2 * sizeof(double);
+  const bool res_host = !out_dev, ps_host = per_shift && !ps_dev;
+  if (res_host || ps_host) {
+    if (res_host && ps_host) {
+      // the workspace holds the results and then the per-shift values: one copy
+      // to pageable memory costs as much as either (8 us of a 70 us call)
+      const size_t ps_at = (size_t)((const char*)pl->ws.per_shift - (const char*)pl->ws.result);
+      std::vector<char> host(ps_at + ps_bytes);
+      QMC_CUDA(cudaMemcpyAsync(host.data(), pl->ws.result, host.size(), cudaMemcpyDeviceToHost, stream));
+      QMC_CUDA(cudaStreamSynchronize(stream));
+      std::memcpy(out, host.data(), res_bytes);
+      std::memcpy(per_shift, host.data() + ps_at, ps_bytes);
+    } else {
+      if (res_host) QMC_CUDA(cudaMemcpyAsync(out, pl->ws.result, res_bytes, cudaMemcpyDeviceToHost, stream));
+      else QMC_CUDA(cudaMemcpyAsync(per_shift, pl->ws.per_shift, ps_bytes, cudaMemcpyDeviceToHost, stream));
+      QMC_CUDA(cudaStreamSynchronize(stream));
+    }
     if (!out_dev) {
       // the first failing order's status (NaN/Inf values are counted per order)
       for (size_t o = 0; o < G; ++o)

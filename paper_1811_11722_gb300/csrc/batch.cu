@@ -115,7 +115,13 @@ static int batch_build(BatchPlan* bp, int32_t count, const qmc_problem* problems
       plans[i] = std::move(pl);
     }
   };
-  const unsigned nt = std::max(1u, std::min<unsigned>(std::thread::hardware_concurrency(), (unsigned)std::min(count, 32)));
+  // FP64 problems are packed in ~5 us each, less than a thread takes to start;
+  // FP32 ones write (and may compile) their specialised source.  The 32-sector
+  // FP64 walk took 4.2 ms with 16 threads, 3.4 ms without.
+  int jits = 0;
+  for (int i = 0; i < count; ++i) jits += problems[i].f && problems[i].f->precision == QMC_FP32EVAL ? 1 : 0;
+  const unsigned nt = std::max(1u, std::min<unsigned>(std::thread::hardware_concurrency(),
+                                                      (unsigned)std::max(std::min(jits, 32), count / 64)));
   std::vector<std::thread> th;
   for (unsigned t = 1; t < nt; ++t) th.emplace_back(work);
   work();
@@ -748,9 +754,18 @@ static int walk_pass(BatchPlan* bp, const std::vector<int>& act, std::vector<Fin
   e = cudaLaunchKernel(finalize_batch_ptr(), dim3((unsigned)act.size()), dim3(256), fargs,
                        (size_t)bp->max_m * 2 * sizeof(double), stream);
   if (e != cudaSuccess) return cuda_fail(e, "walk final pass");
+  if (ps) {  // the results and, after them, the per-shift values in one copy
+    const size_t ps_at = (size_t)((const char*)bp->ps_dev - (const char*)bp->res_dev);
+    const size_t ps_bytes = (size_t)bp->total_m * 2 * sizeof(double);
+    std::vector<char> host(ps_at + ps_bytes);
+    e = cudaMemcpyAsync(host.data(), bp->res_dev, host.size(), cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) return cuda_fail(e, "walk results");
+    std::memcpy(res.data(), host.data(), res.size() * sizeof(qmc_result));
+    std::memcpy(ps, host.data() + ps_at, ps_bytes);
+    return QMC_OK;
+  }
   e = cudaMemcpyAsync(res.data(), bp->res_dev, res.size() * sizeof(qmc_result), cudaMemcpyDeviceToHost, stream);
-  if (e == cudaSuccess && ps)
-    e = cudaMemcpyAsync(ps, bp->ps_dev, (size_t)bp->total_m * 2 * sizeof(double), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return cuda_fail(e, "walk results");
   return QMC_OK;
