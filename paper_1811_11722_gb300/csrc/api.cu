@@ -827,8 +827,6 @@ int launch_finalize(const Plan* pl, const Workspace& ws, qmc_result* res_dev, do
   A.m = pl->m;
   A.is_complex = pl->is_complex;
   A.groups = pl->orders;
-  A.sum_last = pl->sum_last ? 1 : 0;
-  A.pad = 0;
   A.dn = (double)pl->n;
   A.value_scale = pl->final_scale;
   A.offset[0] = pl->offset[0];
@@ -838,7 +836,7 @@ int launch_finalize(const Plan* pl, const Workspace& ws, qmc_result* res_dev, do
   A.per_shift = per_shift_dev;
   void* args[1] = {&A};
   size_t smem = (size_t)pl->m * 2 * sizeof(double);
-  QMC_CUDA(cudaLaunchKernel(finalize_ptr(), dim3(pl->orders), dim3(256), args, smem, stream));
+  QMC_CUDA(cudaLaunchKernel(finalize_ptr(), dim3(pl->orders), dim3(kFinThreads), args, smem, stream));
   return QMC_OK;
 }
 

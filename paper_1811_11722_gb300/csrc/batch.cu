@@ -218,7 +218,7 @@ static int batch_graph(BatchPlan* bp) {
   std::memset(&kp, 0, sizeof(kp));
   kp.func = (void*)finalize_batch_ptr();
   kp.gridDim = dim3(bp->count);
-  kp.blockDim = dim3(256);
+  kp.blockDim = dim3(kFinThreads);
   kp.sharedMemBytes = (unsigned)((size_t)bp->max_m * 2 * sizeof(double));
   kp.kernelParams = fargs;
   cudaGraphNode_t fnode;
@@ -441,7 +441,7 @@ static int persist_graph(BatchPlan* bp) {
   std::memset(&fp, 0, sizeof(fp));
   fp.func = (void*)finalize_batch_ptr();
   fp.gridDim = dim3(bp->count);
-  fp.blockDim = dim3(256);
+  fp.blockDim = dim3(kFinThreads);
   fp.sharedMemBytes = (unsigned)((size_t)bp->max_m * 2 * sizeof(double));
   fp.kernelParams = fargs;
   cudaGraphNode_t fnode;
@@ -699,7 +699,7 @@ static int oneshot_run(BatchPlan* bp, cudaStream_t stream) {
   if (rc) return rc;
   FinalizeArgs* fin = bp->fin_dev;
   void* fargs[1] = {&fin};
-  e = cudaLaunchKernel(finalize_batch_ptr(), dim3(bp->count), dim3(256), fargs, (size_t)bp->max_m * 2 * sizeof(double),
+  e = cudaLaunchKernel(finalize_batch_ptr(), dim3(bp->count), dim3(kFinThreads), fargs, (size_t)bp->max_m * 2 * sizeof(double),
                        stream);
   if (e != cudaSuccess) return cuda_fail(e, "batch final pass");
   return QMC_OK;
@@ -751,7 +751,7 @@ static int walk_pass(BatchPlan* bp, const std::vector<int>& act, std::vector<Fin
   if (rc) return rc;
   FinalizeArgs* fd = bp->fin_dev;
   void* fargs[1] = {&fd};
-  e = cudaLaunchKernel(finalize_batch_ptr(), dim3((unsigned)act.size()), dim3(256), fargs,
+  e = cudaLaunchKernel(finalize_batch_ptr(), dim3((unsigned)act.size()), dim3(kFinThreads), fargs,
                        (size_t)bp->max_m * 2 * sizeof(double), stream);
   if (e != cudaSuccess) return cuda_fail(e, "walk final pass");
   if (ps) {  // the results and, after them, the per-shift values in one copy
@@ -899,7 +899,7 @@ static int walk_pass_persistent(BatchPlan* bp, WalkPersist* W, const std::vector
   if (rc) return rc;
   FinalizeArgs* fd = bp->fin_dev;
   void* fargs[1] = {&fd};
-  e = cudaLaunchKernel(finalize_batch_ptr(), dim3((unsigned)act.size()), dim3(256), fargs,
+  e = cudaLaunchKernel(finalize_batch_ptr(), dim3((unsigned)act.size()), dim3(kFinThreads), fargs,
                        (size_t)bp->max_m * 2 * sizeof(double), stream);
   if (e != cudaSuccess) return cuda_fail(e, "walk final pass");
   e = cudaMemcpyAsync(res.data(), bp->res_dev, res.size() * sizeof(qmc_result), cudaMemcpyDeviceToHost, stream);

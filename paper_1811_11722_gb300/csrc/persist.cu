@@ -76,11 +76,7 @@ __device__ __noinline__ void persist_item(const RuleParams<float>& P, uint64_t j
     unpack_runs<MC>(run2, acc);
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int kk = 0; kk < MC; ++kk) {
-    const double t = acc[kk].warp_total();
-    if (lane == 0) red[warp][kk] = t;
-  }
+  warp_totals<float, MC>(acc, red[warp]);
   if constexpr (CHECK) {
     const unsigned long long bad = warp_sum_u64((unsigned long long)nbad);
     if (lane == 0 && bad) atomicAdd(&counters[0], bad);

@@ -122,11 +122,7 @@ __device__ __forceinline__ void pj_sweep(uint64_t j0, uint64_t chunk, uint32_t i
     unpack_runs<MC>(run2, acc);
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int kk = 0; kk < MC; ++kk) {
-    const double t = acc[kk].warp_total();
-    if (lane == 0) red[warp][kk] = t;
-  }
+  warp_totals<float, MC>(acc, red[warp]);
   if constexpr (SP::CHECK) {
     const unsigned long long bad = warp_sum_u64((unsigned long long)nbad);
     if (lane == 0 && bad) atomicAdd(&counters[0], bad);

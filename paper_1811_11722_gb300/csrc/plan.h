@@ -60,7 +60,6 @@ struct Plan {
   int m = 0;
   int is_complex = 0;
   int orders = 1;  // result groups: epsilon orders f_0..f_{orders-1}, or integrands + their sum
-  bool sum_last = false;  // the last group is the sum of the others (shared-lattice plans)
   int nblk = 0;
   int mc = 0;
   int imm = 0;     // the specialised kernel takes its shifts as immediate operands

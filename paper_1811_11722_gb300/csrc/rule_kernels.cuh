@@ -72,6 +72,27 @@ struct Acc<double> {
   __device__ __forceinline__ double thread_total() { return run; }
 };
 
+// The warp totals of N accumulators into out[0..N).
+template <typename R, int N>
+__device__ __forceinline__ void warp_totals(Acc<R>* acc, double* out) {
+  if constexpr (sizeof(R) == 4) {
+    float h[N], l[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      acc[k].fold();
+      h[k] = acc[k].hi;
+      l[k] = acc[k].lo;
+    }
+    warp_totals_ff<N>(h, l, out);
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const double t = acc[k].warp_total();
+      if ((threadIdx.x & 31) == 0) out[k] = t;
+    }
+  }
+}
+
 // Fixed-point base of a coordinate for the precision at hand.
 template <typename R>
 struct FixT;
@@ -290,11 +311,7 @@ __device__ __forceinline__ void block_epilogue(Acc<R>* acc, int mk, unsigned nba
                                                unsigned long long* __restrict__ counters) {
   __shared__ double red[kThreads / 32][MC];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int kk = 0; kk < MC; ++kk) {
-    double t = acc[kk].warp_total();
-    if (lane == 0) red[warp][kk] = t;
-  }
+  warp_totals<R, MC>(acc, red[warp]);
   unsigned long long bad = warp_sum_u64((unsigned long long)nbad);
   if (lane == 0 && bad) atomicAdd(&counters[0], bad);
   __syncthreads();
@@ -711,11 +728,7 @@ __device__ __forceinline__ void eps_epilogue(Acc<R> (&acc)[NE][MC], const unsign
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 0; o < NE; ++o) {
-#pragma unroll
-    for (int kk = 0; kk < MC; ++kk) {
-      double t = acc[o][kk].warp_total();
-      if (lane == 0) red[warp][o * MC + kk] = t;
-    }
+    warp_totals<R, MC>(acc[o], red[warp] + o * MC);
     unsigned long long bad = warp_sum_u64((unsigned long long)nbad[o]);
     if (lane == 0 && bad && o < P.eps_orders) atomicAdd(&counters[2 * o], bad);
   }
@@ -1080,11 +1093,6 @@ __device__ __forceinline__ void multi_body(const MultiParams& M, double* __restr
     } else {
       unpack_runs<MC>(run2[s], acc[s]);
     }
-#pragma unroll
-    for (int kk = 0; kk < MC; ++kk) {
-      double t = acc[s][kk].warp_total();
-      if (lane == 0) red[warp][s * MC + kk] = t;
-    }
     if constexpr (CHECK) {
       unsigned long long bad = warp_sum_u64((unsigned long long)nbad[s]);
       bad_all += bad;
@@ -1094,16 +1102,30 @@ __device__ __forceinline__ void multi_body(const MultiParams& M, double* __restr
   if constexpr (CHECK) {
     if (lane == 0 && bad_all) atomicAdd(&counters[2 * M.count], bad_all);
   }
+  static_assert(SC * MC <= 32, "one warp writes the slots");
+  warp_totals<float, SC * MC>(&acc[0][0], red[warp]);
   __syncthreads();
-  for (int t = threadIdx.x; t < SC * MC; t += kThreads) {
-    const int s = t / MC, kk = t % MC;
-    if (kk >= P.m_launch) continue;
+  if (threadIdx.x < SC * MC) {
+    const int s = threadIdx.x / MC, kk = threadIdx.x % MC;
     double acc_s = 0.0;
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) acc_s += red[w][t];
-    const size_t slot = (((size_t)(M.s_base + s) * P.m_total + P.k_base + kk) * P.nblk + blockIdx.x) * 2;
-    partial[slot] = acc_s;
-    partial[slot + 1] = 0.0;
+    for (int w = 0; w < kThreads / 32; ++w) acc_s += red[w][threadIdx.x];
+    const auto slot = [&](int grp) { return (((size_t)grp * P.m_total + P.k_base + kk) * P.nblk + blockIdx.x) * 2; };
+    if (kk < P.m_launch) {
+      partial[slot(M.s_base + s)] = acc_s;
+      partial[slot(M.s_base + s) + 1] = 0.0;
+    }
+    // the sum group's slot: this chunk's integrands in order, on top of the
+    // earlier chunks' launches
+    red[0][threadIdx.x] = acc_s;
+    __syncwarp(__activemask());
+    if (s == 0 && kk < P.m_launch) {
+      double tot = M.s_base == 0 ? 0.0 : partial[slot(M.count)];
+#pragma unroll
+      for (int q = 0; q < SC; ++q) tot += red[0][q * MC + kk];
+      partial[slot(M.count)] = tot;
+      partial[slot(M.count) + 1] = 0.0;
+    }
   }
 }
 
