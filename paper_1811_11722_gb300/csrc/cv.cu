@@ -18,7 +18,7 @@
 // Training kernels.  The two contractions of the fit run on tensor cores
 // (warp-level BF16 MMA, FP32 accumulation); the loss is summed in FP64:
 //   cv_basis     B[i][j][k] = cos(F pi k x_ji) for the pilot points, rounded to
-//                BF16, Bf[i][j][k], once per fit; padding points j >= P are zero rows
+//                BF16, Bf[i][j][cv_swz(j, k)], once per fit; padding points j >= P are zero rows
 //   cv_fit       per tile of 16 points: C_ri(x_j) = sum_k B a, g_j,
 //                e_j = 2 (g_j - h_j)/P, the factor D[i][j][r] = e_j prod_{i'!=i} C_ri'
 //                and grad_part[c][i][r][k] += sum_j D[i][j][r] B[i][j][k], all in
@@ -82,24 +82,45 @@ __global__ void cv_basis_kernel(const double* __restrict__ x, int P, int Ppad, i
   uint16_t* out = Bf + ((size_t)i * Ppad + j) * kCvK;
 #pragma unroll 4
   for (int k = 0; k < kCvK; ++k)
-    out[k] = j < P ? bf16_bits((float)cospi((double)freq * (double)k * xv)) : (uint16_t)0;
+    out[cv_swz(j, k)] = j < P ? bf16_bits((float)cospi((double)freq * (double)k * xv)) : (uint16_t)0;
+}
+
+// (double)f by integer operations: the conversion instruction holds the FP64 pipe
+// for 16 clocks a warp, as long as the addition that needs it.
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t u = __float_as_uint(f), e = (u >> 23) & 255u;
+  if (e == 0 || e == 255) return (double)f;  // zero, denormal, infinity, NaN
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(u << 29));
 }
 
 // Adam step.  A CTA takes 32 parameters: warp w adds the CTAs' partial
-// gradients c = w, w + 8, ... in FP64 (coalesced rows of 32), the eight warp
-// sums are added in warp order, and warp 0 applies the update.  The order of
-// every addition is fixed, so the fit is reproducible.
+// gradients c = w, w + 8, ... in FP64 (coalesced rows of 32, eight loads in
+// flight), the eight warp sums are added in warp order, and warp 0 applies the
+// update.  The order of every addition is fixed, so the fit is reproducible.
+// The step's bias corrections are computed before the wait for the gradient.
 constexpr int kAdamWarps = 8;
 __global__ void __launch_bounds__(kAdamWarps * 32)
     cv_adam_kernel(const float* __restrict__ grad_part, int nchunk, int npar, float* __restrict__ a,
                    float* __restrict__ m1, float* __restrict__ m2, int step, float lr, int band) {
   __shared__ double part[kAdamWarps][32];
+  __shared__ float corr[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * 32 + lane;
+  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  grid_launch_next();
+  if (warp == 1 && lane < 2) corr[lane] = 1.0f - powf(lane ? b2 : b1, (float)step);
+  grid_wait();
   double g = 0.0;
   if (q < npar)
-#pragma unroll 4
-    for (int c = warp; c < nchunk; c += kAdamWarps) g += (double)grad_part[(size_t)c * npar + q];
+    for (int c = warp; c < nchunk; c += 8 * kAdamWarps) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        v[u] = c + kAdamWarps * u < nchunk ? grad_part[(size_t)(c + kAdamWarps * u) * npar + q] : 0.0f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (c + kAdamWarps * u < nchunk) g += widen(v[u]);
+    }
   part[warp][lane] = g;
   __syncthreads();
   if (warp != 0 || q >= npar) return;
@@ -110,27 +131,26 @@ __global__ void __launch_bounds__(kAdamWarps * 32)
   double tot = 0.0;
 #pragma unroll
   for (int w = 0; w < kAdamWarps; ++w) tot += part[w][lane];
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float gf = (float)tot;
   const float mm = b1 * m1[q] + (1.0f - b1) * gf;
   const float vv = b2 * m2[q] + (1.0f - b2) * gf * gf;
   m1[q] = mm;
   m2[q] = vv;
-  const float mh = mm / (1.0f - powf(b1, (float)step));
-  const float vh = vv / (1.0f - powf(b2, (float)step));
+  const float mh = mm / corr[0];
+  const float vh = vv / corr[1];
   a[q] -= lr * mh / (sqrtf(vh) + eps);
 }
 
-static const void* cv_fit_for(int d) {
+static const void* cv_fit_for(int d, size_t* smem) {
   switch (d) {
-    case 1: return cv_fit_ptr<1>();
-    case 2: return cv_fit_ptr<2>();
-    case 3: return cv_fit_ptr<3>();
-    case 4: return cv_fit_ptr<4>();
-    case 5: return cv_fit_ptr<5>();
-    case 6: return cv_fit_ptr<6>();
-    case 7: return cv_fit_ptr<7>();
-    default: return cv_fit_ptr<8>();
+    case 1: return cv_fit_ptr<1>(smem);
+    case 2: return cv_fit_ptr<2>(smem);
+    case 3: return cv_fit_ptr<3>(smem);
+    case 4: return cv_fit_ptr<4>(smem);
+    case 5: return cv_fit_ptr<5>(smem);
+    case 6: return cv_fit_ptr<6>(smem);
+    case 7: return cv_fit_ptr<7>(smem);
+    default: return cv_fit_ptr<8>(smem);
   }
 }
 
@@ -142,11 +162,36 @@ static int cv_fit_grid(int Ppad) {
   return std::max(1, std::min(batches, 2 * std::max(sms, 1)));
 }
 
+// A kernel of the fit; overlap: its prologue may run while the one before it
+// finishes (it waits itself for that one's results).
+static cudaError_t cv_launch(const void* func, int grid, int block, size_t smem, void** args, bool overlap,
+                             cudaStream_t st) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, func, args);
+}
+
 // Loss partials into lp[0 .. nchunk) and gradient partials into grad_part[nchunk][npar].
-static void cv_fit_step(int d, int P, int Ppad, int nchunk, const uint16_t* Bf, const double* hv, const float* a,
-                        float* grad_part, double* lp, cudaStream_t st) {
+// overlap: the kernel before it in the stream is an Adam step (the basis is long in place).
+static cudaError_t cv_fit_step(int d, int P, int Ppad, int nchunk, const uint16_t* Bf, const double* hv, const float* a,
+                               float* grad_part, double* lp, bool overlap, cudaStream_t st) {
   void* args[7] = {(void*)&Bf, (void*)&hv, (void*)&a, (void*)&P, (void*)&Ppad, (void*)&grad_part, (void*)&lp};
-  cudaLaunchKernel(cv_fit_for(d), dim3(nchunk), dim3(kCvFitWarps * 32), args, 0, st);
+  size_t smem = 0;
+  const void* func = cv_fit_for(d, &smem);
+  if (!overlap) {  // a fit's first step
+    cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  return cv_launch(func, nchunk, kCvFitWarps * 32, smem, args, overlap, st);
 }
 
 static float bf16_round(float v) {
@@ -170,11 +215,13 @@ struct CvFit {
   float* m2 = nullptr;
   float* grad_part = nullptr;
   double* loss_part = nullptr;
-  void* block = nullptr;
+  void* block = nullptr;     // stream-ordered: two calls of cudaMalloc and cudaFree cost 0.4 ms
+  cudaStream_t st = nullptr;
   ~CvFit() {
-    if (block) cudaFree(block);
+    if (block) cudaFreeAsync(block, st);
   }
-  int alloc(int d_, int P_) {
+  int alloc(int d_, int P_, cudaStream_t st_) {
+    st = st_;
     d = d_;
     P = P_;
     Ppad = (P + kCvTile - 1) / kCvTile * kCvTile;
@@ -185,8 +232,9 @@ struct CvFit {
                    (size_t)nchunk * npar * 4, (size_t)nchunk * 8};
     size_t total = 0;
     for (size_t s : sz) total += (s + 255) & ~(size_t)255;
-    if (cudaMalloc(&block, total) != cudaSuccess) {
+    if (cudaMallocAsync(&block, total, st) != cudaSuccess) {
       cudaGetLastError();
+      block = nullptr;
       return fail(QMC_ENOMEM, "control-variate fit buffers (%zu bytes)", total);
     }
     char* p = (char*)block;
@@ -233,7 +281,7 @@ int qmc_cv_loss_grad(int32_t d, const qmc_cv_config* cfg, int32_t P, const doubl
   if (P < 1 || !x || !h || !a || !loss_out || !grad_out) return fail(QMC_EINVAL, "bad loss/gradient arguments");
   cudaStream_t st = (cudaStream_t)stream;
   CvFit F;
-  rc = F.alloc(d, P);
+  rc = F.alloc(d, P, st);
   if (rc) return rc;
   std::vector<double> hv(2 * (size_t)P, 0.0);
   for (int j = 0; j < P; ++j) hv[2 * (size_t)j] = h[j];
@@ -241,11 +289,12 @@ int qmc_cv_loss_grad(int32_t d, const qmc_cv_config* cfg, int32_t P, const doubl
   cudaMemcpyAsync(F.hv, hv.data(), hv.size() * 8, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(F.a, a, (size_t)F.npar * 4, cudaMemcpyHostToDevice, st);
   cv_basis_kernel<<<(F.Ppad * d + 255) / 256, 256, 0, st>>>(F.x, P, F.Ppad, d, (float)cfg->freq_step, F.Bf);
-  cv_fit_step(d, P, F.Ppad, F.nchunk, F.Bf, F.hv, F.a, F.grad_part, F.loss_part, st);
+  cudaError_t e = cv_fit_step(d, P, F.Ppad, F.nchunk, F.Bf, F.hv, F.a, F.grad_part, F.loss_part, false, st);
+  if (e != cudaSuccess) return cuda_fail(e, "control-variate gradient");
   std::vector<float> gp((size_t)F.nchunk * F.npar);
   cudaMemcpyAsync(gp.data(), F.grad_part, gp.size() * 4, cudaMemcpyDeviceToHost, st);
   *loss_out = cv_loss_host(F, st);
-  cudaError_t e = cudaStreamSynchronize(st);
+  e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "control-variate gradient");
   for (int q = 0; q < F.npar; ++q) {
     double s = 0.0;
@@ -278,17 +327,11 @@ int qmc_cv_train(int32_t d, uint64_t n_pilot, const uint64_t* g_pilot, const dou
   if (rc) return rc;
   const int P = (int)n_pilot;
   CvFit F;
-  rc = F.alloc(d, P);
+  rc = F.alloc(d, P, st);
   if (rc) return rc;
-  uint64_t* dj = nullptr;
-  int32_t* dk = nullptr;
-  if (cudaMalloc(&dj, (size_t)P * 8) != cudaSuccess || cudaMalloc(&dk, (size_t)P * 4) != cudaSuccess) {
-    cudaGetLastError();
-    if (dj) cudaFree(dj);
-    return fail(QMC_ENOMEM, "pilot index buffers");
-  }
-  std::unique_ptr<void, void (*)(void*)> g1(dj, [](void* p) { cudaFree(p); });
-  std::unique_ptr<void, void (*)(void*)> g2(dk, [](void* p) { cudaFree(p); });
+  // the pilot's point and shift lists: 12 bytes a point in the basis's 64 d, which is written after they are read
+  uint64_t* dj = (uint64_t*)F.Bf;
+  int32_t* dk = (int32_t*)(dj + P);
   cv_iota_kernel<<<(P + 255) / 256, 256, 0, st>>>(dj, P);
   cudaMemsetAsync(dk, 0, (size_t)P * 4, st);
   SampleIO sio;
@@ -343,13 +386,17 @@ int qmc_cv_train(int32_t d, uint64_t n_pilot, const uint64_t* g_pilot, const dou
   cudaMemsetAsync(F.m2, 0, (size_t)F.npar * 4, st);
   double first = 0.0, last = 0.0;
   for (int step = 1; step <= cfg->steps; ++step) {
-    cv_fit_step(d, P, F.Ppad, F.nchunk, F.Bf, F.hv, F.a, F.grad_part, F.loss_part, st);
+    e = cv_fit_step(d, P, F.Ppad, F.nchunk, F.Bf, F.hv, F.a, F.grad_part, F.loss_part, step > 1, st);
+    if (e != cudaSuccess) return cuda_fail(e, "control-variate training");
     if (step == 1) first = cv_loss_host(F, st);
-    const float lr = (float)(0.5 * cfg->lr * (1.0 + std::cos(M_PI * (double)(step - 1) / (double)cfg->steps)));
-    cv_adam_kernel<<<(F.npar + 31) / 32, kAdamWarps * 32, 0, st>>>(F.grad_part, F.nchunk, F.npar, F.a, F.m1, F.m2,
-                                                                  step, lr, cfg->band);
+    float lr = (float)(0.5 * cfg->lr * (1.0 + std::cos(M_PI * (double)(step - 1) / (double)cfg->steps)));
+    int band = cfg->band;
+    void* args[9] = {&F.grad_part, &F.nchunk, &F.npar, &F.a, &F.m1, &F.m2, &step, &lr, &band};
+    e = cv_launch((const void*)&cv_adam_kernel, (F.npar + 31) / 32, kAdamWarps * 32, 0, args, true, st);
+    if (e != cudaSuccess) return cuda_fail(e, "control-variate training");
   }
-  cv_fit_step(d, P, F.Ppad, F.nchunk, F.Bf, F.hv, F.a, F.grad_part, F.loss_part, st);
+  e = cv_fit_step(d, P, F.Ppad, F.nchunk, F.Bf, F.hv, F.a, F.grad_part, F.loss_part, true, st);
+  if (e != cudaSuccess) return cuda_fail(e, "control-variate training");
   last = cv_loss_host(F, st);
   std::vector<float> af(F.npar);
   cudaMemcpyAsync(af.data(), F.a, (size_t)F.npar * 4, cudaMemcpyDeviceToHost, st);

@@ -25,7 +25,8 @@ const void* cv_estimator5_ptr<QMC_D>(int tr, int alpha) {
 }
 
 template <>
-const void* cv_fit_ptr<QMC_D>() {
+const void* cv_fit_ptr<QMC_D>(size_t* smem) {
+  *smem = sizeof(CvFitSmem<QMC_D>);
   return (const void*)&cv_fit_kernel<QMC_D>;
 }
 
