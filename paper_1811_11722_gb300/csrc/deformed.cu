@@ -110,6 +110,11 @@ static int build_def(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
   const int form = packed ? korobov_form(d, pack_dense(f->U, d, 1), cf) : 3;
   if (packed) func = form == kKorCentred ? deformed2_ptr<kKorCentred>(d) : deformed2_ptr<3>(d);
   const bool tab = fast && d <= kDefFastMax;
+  if (sizeof(R) == 8 && tab && u_linear && f->aU == -2 && f->aF == -1) {
+    int rc = build_deformed_fx_plan(pl, d, n, m, g, shifts, fast_table(cf, d, f->lambda), pack_dense(f->U, d, 1),
+                                    f->lambda, tune);
+    if (rc != QMC_EUNSUPPORTED) return rc;
+  }
   const bool rows64 = tab && sizeof(R) == 8;  // a CTA row per shift row
   if (!func) return fail(QMC_EUNSUPPORTED, "no deformed kernel for d=%d", d);
   auto cu = pack_dense(f->U, d, u_linear ? 1 : 2);

@@ -646,12 +646,36 @@ __global__ void __launch_bounds__(kThreads, 2)
   }
 }
 
+// The CTA's sums of both parts in a fixed order to out[0..1] (a lane of warps 0 and
+// 1 adds eight threads' parts, then the warp tree), and its counts.
+__device__ __forceinline__ void block_sum2(double re, double im, unsigned nbad, unsigned ndef,
+                                           unsigned long long* __restrict__ counters, double* __restrict__ out) {
+  __shared__ double red[2][kThreads];
+  red[0][threadIdx.x] = re;
+  red[1][threadIdx.x] = im;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned long long b1 = warp_sum_u64((unsigned long long)nbad);
+  const unsigned long long b2 = warp_sum_u64((unsigned long long)ndef);
+  if (lane == 0 && b1) atomicAdd(&counters[0], b1);
+  if (lane == 0 && b2) atomicAdd(&counters[1], b2);
+  __syncthreads();
+  if (warp < 2) {
+    double t = red[warp][lane];
+#pragma unroll
+    for (int w = 1; w < kThreads / 32; ++w) t += red[warp][lane + 32 * w];
+    t = warp_sum_d(t);
+    if (lane == 0) out[warp] = t;
+  }
+}
+
 // ------------------------------------------------------- FP64, FAST --
 
 // One shift row per CTA row, a thread's points kThreads apart; the FP64 pipe
 // (2 operations per SM and clock) bounds it, so fractions and coordinates
 // stay in integers.  At d = 5: 225 FP64 operations a value, against 630 with LU and
-// the double transform.  n = 262139, m = 20: 5.28 -> 2.25 ms.
+// the double transform.  n = 262139, m = 20: 5.28 -> 2.25 ms.  It serves what the
+// fixed-point form (deformed_fx.cuh) leaves: d = 7, U of degree 2, other powers,
+// scales out of its range.
 template <int D, int KU>
 __global__ void __launch_bounds__(kThreads)
     deformed64_kernel(const __grid_constant__ RuleParams<double> P, double* __restrict__ partial,
@@ -698,23 +722,7 @@ __global__ void __launch_bounds__(kThreads)
       im += ok ? v.im : 0.0;
     }
   }
-  // fixed-order sums: a lane of warps 0 and 1 adds eight threads' parts, then the warp tree
-  __shared__ double red[2][kThreads];
-  red[0][threadIdx.x] = re;
-  red[1][threadIdx.x] = im;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned long long b1 = warp_sum_u64((unsigned long long)nbad);
-  const unsigned long long b2 = warp_sum_u64((unsigned long long)ndef);
-  if (lane == 0 && b1) atomicAdd(&counters[0], b1);
-  if (lane == 0 && b2) atomicAdd(&counters[1], b2);
-  __syncthreads();
-  if (warp < 2) {
-    double t = red[warp][lane];
-#pragma unroll
-    for (int w = 1; w < kThreads / 32; ++w) t += red[warp][lane + 32 * w];
-    t = warp_sum_d(t);
-    if (lane == 0) partial[((size_t)(P.k_base + k) * P.nblk + blockIdx.x) * 2 + warp] = t;
-  }
+  block_sum2(re, im, nbad, ndef, counters, partial + ((size_t)(P.k_base + k) * P.nblk + blockIdx.x) * 2);
 }
 
 }  // namespace qmc

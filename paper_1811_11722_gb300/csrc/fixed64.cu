@@ -1,5 +1,6 @@
-// Plans of FP64 sector integrands on the fixed-point kernel (fixed64.cuh):
-// which integrands it takes, their coefficients in fixed point, the launches.
+// Plans of FP64 integrands on the fixed-point kernels (sectors: fixed64.cuh,
+// deformed: deformed_fx.cuh): which integrands they take, the coefficients in
+// fixed point, the launches.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -32,7 +33,7 @@ bool fx_scale(const std::vector<double>& c, int* k) {
   return std::abs(*k) <= 200;
 }
 
-void fx_lattice(FxParams& P, uint64_t n, const uint64_t* g) {
+void fx_lattice(FxBase& P, uint64_t n, const uint64_t* g) {
   P.n = n;
   P.rc = reciprocal(n);
   for (int i = 0; i < P.d; ++i) {
@@ -48,7 +49,7 @@ void fx_lattice(FxParams& P, uint64_t n, const uint64_t* g) {
 
 // rows m_launch.. of the last pair repeat the launch's first row (evaluated,
 // never written back)
-void fx_shifts(FxParams& P, const double* shifts) {
+void fx_shifts(FxBase& P, const double* shifts) {
   for (int kk = 0; kk < kMcMax; ++kk)
     for (int i = 0; i < P.d; ++i) {
       const int src = kk < P.m_launch ? P.k_base + kk : P.k_base;
@@ -56,13 +57,12 @@ void fx_shifts(FxParams& P, const double* shifts) {
     }
 }
 
-// Launch shape: one resident wave over (point tiles, pairs of shift rows),
-// `pairs` pairs in the largest launch.  max_ctas (> 0) caps the CTAs of one
-// pair of rows.
-int fx_grid(int occ, uint64_t n, int pairs, int max_ctas, int* nblk, int* L, uint64_t* tiles) {
+// Launch shape: one resident wave over (point tiles, CTA rows), `rows` rows in the
+// largest launch.  max_ctas (> 0) caps the CTAs of one row.
+int fx_grid(int occ, uint64_t n, int rows, int max_ctas, int* nblk, int* L, uint64_t* tiles) {
   const int sms = device_sms();
   if (sms <= 0) return fail(QMC_ECUDA, "no CUDA device");
-  uint64_t want = std::max<uint64_t>(1, (uint64_t)sms * (uint64_t)std::max(occ, 1) / (uint64_t)pairs);
+  uint64_t want = std::max<uint64_t>(1, (uint64_t)sms * (uint64_t)std::max(occ, 1) / (uint64_t)rows);
   if (max_ctas > 0) want = std::min<uint64_t>(want, (uint64_t)max_ctas);
   const uint64_t per = (n + want * kThreads - 1) / (want * kThreads);
   *L = (int)std::max<uint64_t>(1, std::min<uint64_t>(per, 512));
@@ -144,7 +144,8 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
   // three CTAs of 8 warps saturate an SM's issue slots
   int rc = grid_occupancy(func, 0, tune.occupancy > 0 ? std::min(tune.occupancy, 3) : 3, occ);
   if (rc) return rc;
-  rc = fx_grid(occ, n, fx_pairs(m), tune.max_ctas, &nblk, &L, &tiles);
+  pl->grid_rows = fx_pairs(m);
+  rc = fx_grid(occ, n, pl->grid_rows, tune.max_ctas, &nblk, &L, &tiles);
   if (rc) return rc;
   pl->param_kind = 5;
   pl->grid_occ = occ;
@@ -171,13 +172,147 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
   return QMC_OK;
 }
 
+constexpr double kDefFxMin = 1.0 / 32.0;  // smallest sum of |lambda dF| over the cube
+
+// The deformed FAST integrand in fixed point (deformed_fx.cuh) from DefTab's
+// constants t (F(0), dF(0), Hessian, half diagonal, minors) and U's cu.
+// QMC_EUNSUPPORTED, nothing written, where the scales leave the range in which
+// the fixed-point errors stay below the double kernel's.
+int build_deformed_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
+                           const std::vector<double>& t, const std::vector<double>& cu, double lambda,
+                           const TuneChoice& tune) {
+  if (d > kDefFxMax || !(lambda > 0.0) || tune.L > 0 || tune.no_fx) return QMC_EUNSUPPORTED;
+  const void* func = nullptr;
+  switch (d) {
+    case 1: func = deformed_fx_ptr<1>(); break;
+    case 2: func = deformed_fx_ptr<2>(); break;
+    case 3: func = deformed_fx_ptr<3>(); break;
+    case 4: func = deformed_fx_ptr<4>(); break;
+    case 5: func = deformed_fx_ptr<5>(); break;
+    case 6: func = deformed_fx_ptr<6>(); break;
+  }
+  const double* lin = t.data() + 1;
+  const double* Hu = lin + d;
+  const double* minors = Hu + d * (d + 1) / 2 + d;
+  const auto at = [&](int k, int l) {
+    const int i = std::min(k, l), j = std::max(k, l);
+    return i * d - i * (i - 1) / 2 + (j - i);
+  };
+  // bounds over the cube: |g'_k|, their sum (y.g'), |m_k|, the recursion's nodes
+  double gmax = 0.0, gsum = 0.0, lsum = 0.0, usum = 0.0;
+  std::vector<double> growth(d);
+  for (int k = 0; k < d; ++k) {
+    double gk = std::fabs(lin[k]);
+    for (int l = 0; l < d; ++l) gk += std::fabs(Hu[at(k, l)]);
+    gk *= lambda;
+    gmax = std::max(gmax, gk);
+    gsum += gk;
+    lsum += std::fabs(lin[k]);
+    usum += std::fabs(cu[1 + k]);
+    growth[k] = std::hypot(1.0, gk + 0.25 * lambda * std::fabs(Hu[at(k, k)]));
+  }
+  std::vector<double> node((size_t)1 << d);
+  double top = 1.0;
+  for (unsigned S = 0; S < (1u << d); ++S) {
+    node[S] = std::fabs(minors[S]) * std::pow(lambda, (double)__builtin_popcount(S));
+    top = std::max(top, node[S]);
+  }
+  for (int J = d - 1; J >= 0; --J)
+    for (unsigned S = 0; S < (1u << J); ++S) {
+      node[S] = growth[J] * node[S] + 0.25 * node[S | (1u << J)];
+      top = std::max(top, node[S]);
+    }
+  // near the origin F and U are their constants, against which the sums' absolute
+  // errors count; y.g' gives F in units of lambda
+  if (!(std::fabs(t[0]) * kFxRange >= lsum + gsum / lambda) || !(std::fabs(cu[0]) * kFxRange >= usum) ||
+      !(gsum >= kDefFxMin))
+    return QMC_EUNSUPPORTED;
+  // the largest scale that keeps `most` below 2^bits
+  const auto scale = [](double most, double bits) { return (int)std::floor(bits - std::log2(std::max(most, 1e-300))); };
+  const int cg = std::min({62, scale(gmax, 60.5), scale(gsum, 61.5)});
+  const int x = std::min(cg, scale(top, 60.5));
+  const int cl = std::min(62, scale(lsum, 60.5)), cuq = std::min(62, scale(usum, 60.5));
+  if (gmax > 4.0 || 62 - cg > 8 || x < 54 || cg - x > 8 || cl < 40 || cuq < 40 || !std::isfinite(top) ||
+      !std::isfinite(gsum))
+    return QMC_EUNSUPPORTED;
+
+  DefFxParams base;
+  std::memset(&base, 0, sizeof(base));
+  base.d = d;
+  base.tr = TR_KOROBOV;
+  fx_lattice(base, n, g);
+  const auto fixed = [](double c, int q) { return (int64_t)std::llrint(std::ldexp(c, q)); };
+  const auto times = [&](double a, double b, int q) {  // a b without the product's rounding
+    const double hi = a * b;
+    return fixed(hi, q) + fixed(std::fma(a, b, -hi), q);
+  };
+  const auto limb = [](int64_t v) {  // to the nearest, the last three bits are dropped
+    return FxLimb{(int32_t)((v + 4) >> 31), (int32_t)(((uint32_t)(v + 4) >> 3) & 0x0FFFFFFFu)};
+  };
+  for (int k = 0; k < d; ++k) {
+    for (int l = k; l < d; ++l) base.H[at(k, l)] = limb(times(-lambda, Hu[at(k, l)], cg));
+    base.Q[k] = limb(times(-0.5 * lambda, Hu[at(k, k)], cg));
+    base.gl[k] = times(-lambda, lin[k], cg);
+    base.fl[k] = limb(fixed(lin[k], cl));
+    base.u[k] = limb(fixed(cu[1 + k], cuq));
+  }
+  for (unsigned S = 0; S < (1u << d); ++S) {
+    const double h = minors[S] * std::pow(-lambda, (double)__builtin_popcount(S));
+    base.hs[S] = fixed(h, x);
+    base.hl[S] = limb(base.hs[S]);
+  }
+  base.sh = 62 - cg;
+  base.mx = cg - x;
+  base.has_lin = lsum > 0.0;
+  base.u0 = cu[0];
+  base.su = std::ldexp(1.0, -cuq);
+  base.f0 = t[0];
+  base.c1 = std::ldexp(0.5, -cl);
+  base.c2 = -std::ldexp(0.5, -cg) / lambda;
+  base.c3 = std::ldexp(1.0, -cg) / lambda;
+  base.sd = std::ldexp(1.0, -x);
+  base.value_scale = korobov_scale(kKorCentred, d) * 0x1p-192;
+
+  int occ = 0, nblk = 0, L = 0;
+  uint64_t tiles = 0;
+  int rc = grid_occupancy(func, 0, tune.occupancy, occ);
+  if (rc) return rc;
+  pl->grid_rows = std::min(m, kMcMax);
+  rc = fx_grid(occ, n, pl->grid_rows, 0, &nblk, &L, &tiles);
+  if (rc) return rc;
+  pl->param_kind = 5;
+  pl->grid_occ = occ;
+  pl->grid_capped = false;  // as the other deformed plans
+  base.L = L;
+  base.tiles = tiles;
+  base.nblk = nblk;
+  pl->nblk = nblk;
+  pl->func = func;
+  pl->mc = kMcMax;
+  pl->final_scale = base.value_scale;
+  pl->is_complex = 1;
+  for (int k0 = 0; k0 < m; k0 += kMcMax) {
+    DefFxParams P = base;
+    P.m_launch = std::min(kMcMax, m - k0);
+    P.k_base = k0;
+    fx_shifts(P, shifts);
+    Launch ln;
+    ln.func = func;
+    ln.grid = dim3(nblk, P.m_launch);
+    ln.params.resize(sizeof(P));
+    std::memcpy(ln.params.data(), &P, sizeof(P));
+    pl->launches.push_back(std::move(ln));
+  }
+  return QMC_OK;
+}
+
 int fx_rebase(Plan* pl, uint64_t n, const uint64_t* g, int max_ctas) {
   int nblk = 0, L = 0;
   uint64_t tiles = 0;
-  int rc = fx_grid(pl->grid_occ, n, fx_pairs(pl->m), max_ctas, &nblk, &L, &tiles);
+  int rc = fx_grid(pl->grid_occ, n, pl->grid_rows, pl->grid_capped ? max_ctas : 0, &nblk, &L, &tiles);
   if (rc) return rc;
   for (Launch& ln : pl->launches) {
-    FxParams& P = *reinterpret_cast<FxParams*>(ln.params.data());
+    FxBase& P = *reinterpret_cast<FxBase*>(ln.params.data());
     fx_lattice(P, n, g);
     P.L = L;
     P.tiles = tiles;
@@ -191,7 +326,7 @@ int fx_rebase(Plan* pl, uint64_t n, const uint64_t* g, int max_ctas) {
 }
 
 void fx_reshift(Plan* pl, const double* shifts) {
-  for (Launch& ln : pl->launches) fx_shifts(*reinterpret_cast<FxParams*>(ln.params.data()), shifts);
+  for (Launch& ln : pl->launches) fx_shifts(*reinterpret_cast<FxBase*>(ln.params.data()), shifts);
 }
 
 }  // namespace qmc

@@ -251,6 +251,28 @@ __device__ __forceinline__ uint64_t fx_frac96(uint32_t idx, const Recip& rc, uin
   return frac64(idx, rc);
 }
 
+// A thread's successive points, kThreads apart: the fractions advance by a 96-bit
+// add modulo 1.
+template <int D>
+struct FxWalk96 {
+  uint64_t base[D];
+  uint32_t lo[D];
+  __device__ __forceinline__ void start(const FxBase& P, uint64_t j) {
+#pragma unroll
+    for (int i = 0; i < D; ++i) base[i] = fx_frac96(lattice_index(j, P.g[i], P.n), P.rc, lo[i]);
+  }
+  __device__ __forceinline__ void step(const FxBase& P) {
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      uint32_t mid = (uint32_t)base[i], top = (uint32_t)(base[i] >> 32);
+      asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+          : "+r"(lo[i]), "+r"(mid), "+r"(top)
+          : "r"(P.step[i][0]), "r"(P.step[i][1]), "r"(P.step[i][2]));
+      base[i] = ((uint64_t)top << 32) | mid;
+    }
+  }
+};
+
 template <int D, int TR>
 __global__ void __launch_bounds__(kThreads)
     sector_fx_kernel(const __grid_constant__ FxParams P, double* __restrict__ partial,
@@ -292,25 +314,16 @@ __global__ void __launch_bounds__(kThreads)
     if (j0 >= P.n) continue;
     const uint64_t left = (P.n - j0 + kThreads - 1) / kThreads;
     const int steps = left < (uint64_t)P.L ? (int)left : P.L;
-    uint64_t base[D];
-    uint32_t blo[D];
-#pragma unroll
-    for (int i = 0; i < D; ++i) base[i] = fx_frac96(lattice_index(j0, P.g[i], P.n), P.rc, blo[i]);
+    FxWalk96<D> walk;
+    walk.start(P, j0);
 #pragma unroll 1
     for (int s = 0; s < steps; ++s) {
       uint64_t v[NS];
       int t[NS];
-      fx_values<D, TR, NS>(P, base, sh, v, t);
+      fx_values<D, TR, NS>(P, walk.base, sh, v, t);
 #pragma unroll
       for (int q = 0; q < NS; ++q) acc[q].add(v[q] << t[q], __funnelshift_l((uint32_t)(v[q] >> 32), 0u, t[q]));
-#pragma unroll
-      for (int i = 0; i < D; ++i) {  // the next point's fractions: a 96-bit add modulo 1
-        uint32_t mid = (uint32_t)base[i], top = (uint32_t)(base[i] >> 32);
-        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
-            : "+r"(blo[i]), "+r"(mid), "+r"(top)
-            : "r"(P.step[i][0]), "r"(P.step[i][1]), "r"(P.step[i][2]));
-        base[i] = ((uint64_t)top << 32) | mid;
-      }
+      walk.step(P);
     }
   }
   // exact integer sums over the CTA, one conversion per slot

@@ -25,7 +25,12 @@ QMC_DECL_SECTOR(double, 5) QMC_DECL_SECTOR(double, 6) QMC_DECL_SECTOR(double, 7)
 // any of the three transforms (Korobov weight 3); null for other codes.
 template <int D>
 const void* sector_fx_ptr(int tr);
-#define QMC_DECL_FX(D) template <> const void* sector_fx_ptr<D>(int);
+// The deformed FAST integrand in fixed point (deformed_fx.cuh), null above kDefFxMax.
+template <int D>
+const void* deformed_fx_ptr();
+#define QMC_DECL_FX(D)                              \
+  template <> const void* sector_fx_ptr<D>(int); \
+  template <> const void* deformed_fx_ptr<D>();
 QMC_DECL_FX(1) QMC_DECL_FX(2) QMC_DECL_FX(3) QMC_DECL_FX(4)
 QMC_DECL_FX(5) QMC_DECL_FX(6) QMC_DECL_FX(7) QMC_DECL_FX(8)
 #undef QMC_DECL_FX
@@ -43,8 +48,8 @@ QMC_DECL_EPS(double, 5) QMC_DECL_EPS(double, 6) QMC_DECL_EPS(double, 7) QMC_DECL
 #undef QMC_DECL_EPS
 
 // Contour-deformed complex sector kernel, d = D <= kDFast: fast = Korobov 3
-// and unpivoted LU (host-checked dominance); otherwise runtime transform and
-// pivoted LU.
+// and host-checked dominance (principal minors up to kDefFastMax, unpivoted LU
+// above); otherwise runtime transform and pivoted LU.
 template <typename R, int D>
 const void* deformed_ptr(bool fast, bool u_linear);
 // Deformed sector kernels: the Hessian of F times -lambda, [k][l] with row

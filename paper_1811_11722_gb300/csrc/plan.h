@@ -77,7 +77,7 @@ struct Plan {
   SavedProblem saved;
   // what plan_rebase needs to move the plan to another lattice
   int param_kind = 0;       // launches hold RuleParams<float> (1), RuleParams<double> (2),
-                            // GeneralParams<float> (3), GeneralParams<double> (4), FxParams (5);
+                            // GeneralParams<float> (3), GeneralParams<double> (4), FxBase and more (5);
                             // 0: fixed lattice
   int grid_occ = 1;         // CTAs per SM the launch shape assumes
   int grid_rows = 1;        // CTA rows of the largest launch, one per shift row or pair (separable FP64,
@@ -131,6 +131,9 @@ double korobov_scale(int form, int d);
 // or QMC_EUNSUPPORTED (nothing written) for integrands outside its range.
 int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
                   const qmc_transform& t, const qmc_integrand* f, const TuneChoice& tune);
+int build_deformed_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
+                           const std::vector<double>& t, const std::vector<double>& cu, double lambda,
+                           const TuneChoice& tune);
 int fx_rebase(Plan* pl, uint64_t n, const uint64_t* g, int max_ctas);
 void fx_reshift(Plan* pl, const double* shifts);
 int plan_alloc(Plan* pl, cudaStream_t stream, bool async);

@@ -8,6 +8,7 @@
 #ifdef __CUDACC_RTC__
 // run-time compilation (NVRTC): no host headers
 typedef unsigned long long uint64_t;
+typedef long long int64_t;
 typedef unsigned int uint32_t;
 typedef int int32_t;
 typedef unsigned char uint8_t;
@@ -150,7 +151,7 @@ __host__ __device__ inline void fill_pairs(RuleParams<R>& P, int d) {
 constexpr int kFxRows = 2;  // shift rows of a CTA of the fixed-point kernel
 // FP64 sectors in fixed point (fixed64.cuh): parameters of one launch, up to
 // kMcMax shift rows, two per CTA row.  Offsets of n, tiles and L as in RuleParams.
-struct FxParams {
+struct FxBase {
   uint64_t n;
   uint64_t tiles;
   int32_t L;
@@ -164,12 +165,34 @@ struct FxParams {
   uint32_t g[kDFast];
   uint32_t step[kDFast][3];     // fraction (kThreads g_i mod n) / n to 96 bits, low word first
   uint64_t shift[kMcMax][kDFast];
+};
+struct FxParams : FxBase {
   uint64_t u0;                  // U: constant term in Q(k-1)
   uint32_t uh[kDFast], ul[kDFast];  // linear coefficients: high word; low word / 16
   uint64_t f0;                  // F: constant term in Q(k-2)
   uint64_t fl[kDFast];          // rows: linear coefficient in Q(k-1)
   uint32_t fmask[kDFast];       // rows: bit 0 linear term, bit 1 + j - i the term q_ij
   uint32_t fh[kDFast * (kDFast + 1) / 2], fq[kDFast * (kDFast + 1) / 2];  // q_ij, row by row
+};
+
+// The deformed FAST integrand in signed fixed point (deformed_fx.cuh): a
+// constant's limbs (high 31 bits signed, the next 28 bits), and the tables.
+constexpr int kDefFxMax = 6;
+struct FxLimb {
+  int32_t h, l;
+};
+struct DefFxParams : FxBase {
+  FxLimb H[kDefFxMax * (kDefFxMax + 1) / 2];  // -lambda times F's Hessian, upper triangle, Q(cg)
+  FxLimb Q[kDefFxMax];                        // half its diagonal
+  int64_t gl[kDefFxMax];                      // -lambda times F's linear coefficients, Q(cg)
+  FxLimb fl[kDefFxMax];                       // F's linear coefficients, Q(cl)
+  FxLimb u[kDefFxMax];                        // U's linear coefficients, Q(cu)
+  int64_t hs[1 << kDefFxMax];                 // (-lambda)^|S| det(H_off restricted to S), Q(x)
+  FxLimb hl[1 << kDefFxMax];
+  int32_t sh, mx, has_lin;                    // 62 - cg, cg - x
+  double u0, su;                              // U: constant, unit of its sums
+  double f0, c1, c2, c3;                      // F: constant, units of y.l, y.g, v.H v and -v.g
+  double sd;                                  // 2^-x
 };
 
 // Several integrands on one lattice (shared-lattice sweep): the rule's

@@ -59,3 +59,23 @@ def test_both_coordinate_forms(Q, oracle_lib, nthreads, c0):
 @pytest.mark.parametrize("quad_u,powers", [(2, (-2, -1)), (0, (-1, -2)), (2, (1, -1))])
 def test_quadratic_u_and_powers(Q, oracle_lib, nthreads, precision, tol, quad_u, powers):
     run(Q, oracle_lib, nthreads, 4, 20021, 9, precision, tol, quad_u=quad_u, powers=powers)
+
+
+@pytest.mark.parametrize("d,c0,lam,linear", [(1, 2.0, 0.3, True), (3, 2.0, 0.3, False), (5, 0.5, 0.1, False),
+                                             (6, 1.0, 0.02, True), (6, 0.01, 0.05, True), (4, 1.0, 1e-4, True),
+                                             (5, 2.0, 0.45, True), (6, 2.0, 1.5, False)])
+def test_fixed_point_ranges(Q, oracle_lib, nthreads, d, c0, lam, linear):
+    """The fixed-point FP64 form at the ends of its scales, and integrands just
+    outside of it (a small constant, a small or a large lambda)."""
+    rng = I.SplitMix64(977 * d + int(1000 * lam))
+    U = I.random_poly(rng, d, d, 0)
+    F = I.random_poly(rng, d, d if linear else 0, d * (d + 1) // 2, neg_quad=0)
+    U.coef[0], F.coef[0] = 1.0, float(np.float32(c0))
+    n, m = 30011, 7
+    p = I.Problem("def", d, n, m, I.make_shifts(rng, m, d), "korobov", alpha=3, kind="sector_deformed", U=U, F=F,
+                  aU=-2, aF=-1, lam=lam, g=I.random_generating_vector(rng, d, n))
+    f = Q.integrand_from_problem(p, "fp64")
+    _, ps = Q.qmc_integrate(d, n, m, p.g, p.shifts, Q.transform("korobov", 3), f, want_per_shift=True)
+    ref = oracle_lib.integrate(p, p.g, nthreads=nthreads)
+    a, b = ps[:, 0] + 1j * ps[:, 1], ref["q"][:, 0] + 1j * ref["q"][:, 1]
+    assert np.all(np.abs(a - b) <= 1e-12 * np.abs(b)), np.abs(a / b - 1).max()
