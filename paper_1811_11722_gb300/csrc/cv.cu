@@ -38,6 +38,7 @@
 // (cv_tc5.cuh) with tcgen05.mma and the basis in tensor memory, or
 // cv_tc_kernel (cv_device.cuh) with warp-level mma.sync.
 #include <cuda_runtime.h>
+#include <math_constants.h>
 
 #include <algorithm>
 #include <chrono>
@@ -85,20 +86,23 @@ __global__ void cv_basis_kernel(const double* __restrict__ x, int P, int Ppad, i
     out[cv_swz(j, k)] = j < P ? bf16_bits((float)cospi((double)freq * (double)k * xv)) : (uint16_t)0;
 }
 
-// (double)f by integer operations: the conversion instruction holds the FP64 pipe
-// for 16 clocks a warp, as long as the addition that needs it.
+// (double)f of a zero or normal number by integer operations: the conversion
+// instruction holds the FP64 pipe for 16 clocks a warp, as long as the addition that
+// needs it.
+__device__ __forceinline__ bool widens(float f) { return f == 0.0f || (fabsf(f) >= 0x1p-126f && fabsf(f) < CUDART_INF_F); }
 __device__ __forceinline__ double widen(float f) {
-  const uint32_t u = __float_as_uint(f), e = (u >> 23) & 255u;
-  if (e == 0 || e == 255) return (double)f;  // zero, denormal, infinity, NaN
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(u << 29));
+  const uint32_t u = __float_as_uint(f), a = u & 0x7FFFFFFFu;
+  return __hiloint2double((int)((u & 0x80000000u) | (a ? (a >> 3) + (896u << 20) : 0u)), (int)(u << 29));
 }
 
 // Adam step.  A CTA takes 32 parameters: warp w adds the CTAs' partial
-// gradients c = w, w + 8, ... in FP64 (coalesced rows of 32, eight loads in
-// flight), the eight warp sums are added in warp order, and warp 0 applies the
+// gradients c = w, w + 8, ... in FP64 (coalesced rows of 32, sixteen loads
+// in flight), the eight warp sums are added in warp order, and warp 0 applies the
 // update.  The order of every addition is fixed, so the fit is reproducible.
+// A branch per value in the widening cost 1.9 us of a step's 15.5, so one test
+// covers the sixteen.
 // The step's bias corrections are computed before the wait for the gradient.
-constexpr int kAdamWarps = 8;
+constexpr int kAdamWarps = 8, kAdamLoads = 16;
 __global__ void __launch_bounds__(kAdamWarps * 32)
     cv_adam_kernel(const float* __restrict__ grad_part, int nchunk, int npar, float* __restrict__ a,
                    float* __restrict__ m1, float* __restrict__ m2, int step, float lr, int band) {
@@ -112,14 +116,22 @@ __global__ void __launch_bounds__(kAdamWarps * 32)
   grid_wait();
   double g = 0.0;
   if (q < npar)
-    for (int c = warp; c < nchunk; c += 8 * kAdamWarps) {
-      float v[8];
+    for (int c = warp; c < nchunk; c += kAdamLoads * kAdamWarps) {
+      float v[kAdamLoads];
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
+      for (int u = 0; u < kAdamLoads; ++u)
         v[u] = c + kAdamWarps * u < nchunk ? grad_part[(size_t)(c + kAdamWarps * u) * npar + q] : 0.0f;
+      bool plain = true;
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (c + kAdamWarps * u < nchunk) g += widen(v[u]);
+      for (int u = 0; u < kAdamLoads; ++u) plain &= widens(v[u]);
+      if (plain && c + kAdamWarps * (kAdamLoads - 1) < nchunk) {
+#pragma unroll
+        for (int u = 0; u < kAdamLoads; ++u) g += widen(v[u]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < kAdamLoads; ++u)
+          if (c + kAdamWarps * u < nchunk) g += (double)v[u];
+      }
     }
   part[warp][lane] = g;
   __syncthreads();
@@ -386,7 +398,8 @@ int qmc_cv_train(int32_t d, uint64_t n_pilot, const uint64_t* g_pilot, const dou
   cudaMemsetAsync(F.m2, 0, (size_t)F.npar * 4, st);
   double first = 0.0, last = 0.0;
   for (int step = 1; step <= cfg->steps; ++step) {
-    e = cv_fit_step(d, P, F.Ppad, F.nchunk, F.Bf, F.hv, F.a, F.grad_part, F.loss_part, step > 1, st);
+    e = cv_fit_step(d, P, F.Ppad, F.nchunk, F.Bf, F.hv, F.a, F.grad_part, step == 1 ? F.loss_part : nullptr,
+                    step > 1, st);
     if (e != cudaSuccess) return cuda_fail(e, "control-variate training");
     if (step == 1) first = cv_loss_host(F, st);
     float lr = (float)(0.5 * cfg->lr * (1.0 + std::cos(M_PI * (double)(step - 1) / (double)cfg->steps)));

@@ -347,7 +347,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // there.  Rows of 32 BF16 values (basis and parameters) keep their four 16-byte
 // quarters permuted by bits 1 and 2 of the row number (cv_swz), so that the eight
 // rows of a fragment load touch distinct banks; the parameter rows before collided
-// eightfold at d = 8.  16381 pilot points, d = 8, 200 steps: 5.08 -> 3.96 ms.
+// eightfold at d = 8.  The residuals' FP64 operations, 16 clocks a warp each, are
+// split over the quads' lanes, and the loss is summed in the steps whose loss is
+// read (loss_part not null): 2 us of a step.  16381 pilot points, d = 8, 200 steps:
+// 5.08 -> 3.18 ms.
 __host__ __device__ __forceinline__ int cv_swz(int row, int k) {  // position of degree k in its row
   return ((((k >> 3) ^ (row >> 1)) & 3) << 3) | (k & 7);
 }
@@ -397,13 +400,26 @@ __global__ void __launch_bounds__(kCvFitWarps * 32)
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   stage(blockIdx.x * W);  // the grid has no CTA without a batch
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  // the FP64 pipe (16 clocks a warp instruction) takes one of a lane's two points: the
+  // quad's even lanes point g, its odd ones g + 8
+  const int row = g + 8 * (t & 1);
+  const auto pilot = [&](int j) { return j < P ? hv[2 * (size_t)j] : 0.0; };
+  double h = pilot((blockIdx.x * W + warp) * 16 + row);
   grid_wait();
   grid_launch_next();
-  for (int q = threadIdx.x; q < kCvR * D * kCvK; q += blockDim.x) {
-    const int k = q % kCvK, i = (q / kCvK) % D, r = q / (kCvK * D);
-    S.as[i][r * kCvK + cv_swz(r, k)] = bf16_bits(a[q]);
+#pragma unroll
+  for (int u = 0; u < kCvR * D * kCvK / (W * 32 * 4) + 1; ++u) {
+    const int q = 4 * (u * W * 32 + (int)threadIdx.x);
+    if (q < kCvR * D * kCvK) {
+      const float4 v = *reinterpret_cast<const float4*>(a + q);
+      const int k = q % kCvK, i = (q / kCvK) % D, r = q / (kCvK * D);
+      uint2 w;
+      w.x = bf16_bits(v.x) | (uint32_t)bf16_bits(v.y) << 16;
+      w.y = bf16_bits(v.z) | (uint32_t)bf16_bits(v.w) << 16;
+      *reinterpret_cast<uint2*>(&S.as[i][r * kCvK + cv_swz(r, k)]) = w;
+    }
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   // fragment words of row g (and g + 8, the same permutation) at degrees 16 ks + 2t and + 8
   int pos[2][2];
 #pragma unroll
@@ -416,16 +432,15 @@ __global__ void __launch_bounds__(kCvFitWarps * 32)
 #pragma unroll
     for (int v = 0; v < 4; ++v) acc[n][v] = 0.0f;
   double l2 = 0.0;
-  const double dP = (double)P, rP = 1.0 / dP;
+  const double hP = 0.5 * (double)P, rP = 1.0 / hP;
   for (int b0 = blockIdx.x * W; b0 < ntiles; b0 += gridDim.x * W) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();  // this batch's basis and as[] in place; fs[] free
     // ---- forward, warp w on tile b0 + w
     const int tile = b0 + warp;
     if (tile < ntiles) {
-      const int j0 = tile * 16;
-      const int jA = j0 + g, jB = j0 + g + 8;
-      const double hA = jA < P ? hv[2 * (size_t)jA] : 0.0, hB = jB < P ? hv[2 * (size_t)jB] : 0.0;
+      const int j = tile * 16 + row;
+      if (b0 != (int)blockIdx.x * W) h = pilot(j);
       float C[D][2][4];  // [dimension][r-tile][fragment]
 #pragma unroll
       for (int i = 0; i < D; ++i) {
@@ -450,7 +465,7 @@ __global__ void __launch_bounds__(kCvFitWarps * 32)
           }
         }
       }
-      // g for rows j0 + g (fragments 0, 1) and j0 + g + 8 (fragments 2, 3)
+      // g for the tile's rows g (fragments 0, 1) and g + 8 (fragments 2, 3)
       float gA = 0.0f, gB = 0.0f;
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt)
@@ -466,10 +481,13 @@ __global__ void __launch_bounds__(kCvFitWarps * 32)
       gA += __shfl_xor_sync(0xffffffffu, gA, 2);
       gB += __shfl_xor_sync(0xffffffffu, gB, 1);
       gB += __shfl_xor_sync(0xffffffffu, gB, 2);
-      const double errA = jA < P ? (double)gA - hA : 0.0;
-      const double errB = jB < P ? (double)gB - hB : 0.0;
-      if (t == 0) l2 += errA * errA + errB * errB;
-      const float eA = (float)div_by(2.0 * errA, dP, rP), eB = (float)div_by(2.0 * errB, dP, rP);
+      const double err = j < P ? (double)(t & 1 ? gB : gA) - h : 0.0;
+      if (loss_part) {
+        const double errB = __shfl_xor_sync(0xffffffffu, err, 1);
+        if (t == 0) l2 += err * err + errB * errB;
+      }
+      const float e2 = (float)div_by(err, hP, rP);  // 2 err / P
+      const float eA = __shfl_sync(0xffffffffu, e2, lane & ~1), eB = __shfl_sync(0xffffffffu, e2, lane | 1);
       // D_i in the accumulator layout as BF16 pairs (rows = points g, g + 8;
       // columns = ranks 8 nt + 2t, +1), transposed block by block into
       // D_i^T[r][j]: lane (g, t) then holds ranks 8 nt + g at points 2t, 2t + 1
@@ -531,6 +549,7 @@ __global__ void __launch_bounds__(kCvFitWarps * 32)
       *reinterpret_cast<float2*>(out + ((g + 8) * D + warp) * kCvK + 8 * n + 2 * t) = make_float2(acc[n][2], acc[n][3]);
     }
   }
+  if (!loss_part) return;
   l2 = warp_sum_d(l2);
   if (lane == 0) S.red[warp] = l2;
   __syncthreads();
