@@ -92,7 +92,10 @@ enum {
 
 /* Arithmetic of the per-point evaluation.  Per-shift sums, Q^(k), Qbar and
  * sigma^2 are FP64 on the device in both modes.
- * FP64: coordinates, transform and f in double.
+ * FP64: coordinates, transform and f in double, or, where the integrand's
+ *   coefficients bound the error below double's, in 64-bit fixed point (U^-2
+ *   F^-1 sectors of degree 1 and 2 with none, baker or Korobov 3; deformed ones
+ *   under Korobov 3 with d <= 6).
  * FP32EVAL: coordinates from 32-bit fixed point, transform and f in float,
  *   compensated float run sums promoted to double per thread.  Under the
  *   Korobov transform every value enters the compensated sum on its own (its
@@ -221,10 +224,10 @@ typedef struct {
 
 /* Many independent rules (e.g. the sectors of one integral: uneven d, n,
  * integrand) evaluated together.  Every problem keeps the kernel it would get
- * from qmc_integrate, with at most ceil(n m / 2^16) CTAs (at most 4 per SM);
- * the problems' launches go round-robin to internal streams forked from
- * `stream` (the GPU runs the sectors side by side), followed by one
- * final-pass launch for all problems.  The workspace comes from the
+ * from qmc_integrate, with at most ceil(n m / 2^16) CTAs (at most 4 per SM; FP64
+ * sectors in fixed point: for each pair of shift rows); the problems' launches
+ * go round-robin to internal streams forked from `stream` (the GPU runs the
+ * sectors side by side), followed by one final-pass launch for all problems.  The workspace comes from the
  * stream-ordered allocator (cudaMallocAsync / cudaFreeAsync on `stream`).
  *   count      number of problems (1..65536)
  *   problems   [count] descriptors (host); each as for qmc_integrate

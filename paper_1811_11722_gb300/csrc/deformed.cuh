@@ -276,8 +276,8 @@ __device__ __forceinline__ void def_fast(const V* c, const V* y, Cx<V>* z, Cx<V>
   dm1 = def_root<D, 0, V>(c + T::M, m, b);
 }
 
-// det(I + i M) - 1 by LU without pivoting, for d above kDefFastMax (J = I + i M strictly diagonally dominant
-// on the cube, shown by the host).  The elimination runs on B = J - I with the
+// det(I + i M) - 1 by LU without pivoting, for d above kDefFastMax (J = I + i M
+// strictly diagonally dominant on the cube, shown by the host).  The elimination runs on B = J - I with the
 // identity implicit: the pivot of column c is 1 + b_cc, the updates
 // b_rq -= f b_cq never touch it (c < q), and the determinant is carried as
 // Delta = det - 1 through (1 + Delta)(1 + b) = 1 + (Delta + b + Delta b).
