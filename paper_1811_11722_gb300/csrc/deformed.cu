@@ -16,21 +16,16 @@ static bool deformed_packed_enabled() {
 }
 
 // The packed FP32 variant (two shifts per instruction), d <= kDef2DMax.
-template <int ALPHA>
 static const void* deformed2_ptr(int d) {
   switch (d) {
-    case 1: return (const void*)&deformed2_kernel<1, ALPHA>;
-    case 2: return (const void*)&deformed2_kernel<2, ALPHA>;
-    case 3: return (const void*)&deformed2_kernel<3, ALPHA>;
-    case 4: return (const void*)&deformed2_kernel<4, ALPHA>;
-    case 5: return (const void*)&deformed2_kernel<5, ALPHA>;
+    case 1: return (const void*)&deformed2_kernel<1>;
+    case 2: return (const void*)&deformed2_kernel<2>;
+    case 3: return (const void*)&deformed2_kernel<3>;
+    case 4: return (const void*)&deformed2_kernel<4>;
+    case 5: return (const void*)&deformed2_kernel<5>;
     default: return nullptr;
   }
 }
-
-// Shifts per launch: the general kernel's shared accumulators; the FAST
-// kernels with a CTA row per shift row (FP64) or pair of rows (packed FP32).
-static_assert(kMcDeformed == 8, "shared accumulators");
 
 // det(H_off restricted to rows S and columns cols) by expansion along its first row.
 // seen (2^2d) keeps the minors found for the other subsets of one table: d = 7, all
@@ -111,30 +106,21 @@ static int build_def(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
 #undef QMC_D_CASE
     default: break;
   }
-  // FP32 packed: the coordinate's form by the integrand's range, as for the sectors
-  const int form = packed ? korobov_form(d, pack_dense(f->U, d, 1), cf) : 3;
-  if (packed) func = form == kKorCentred ? deformed2_ptr<kKorCentred>(d) : deformed2_ptr<3>(d);
-  const bool tab = fast && d <= kDefFastMax;
-  if (sizeof(R) == 8 && tab && u_linear && f->aU == -2 && f->aF == -1) {
+  if (packed) func = deformed2_ptr(d);
+  // FP64 FAST: a CTA row per shift row, det J from the minors' table
+  const bool rows64 = sizeof(R) == 8 && fast && d <= kDefFastMax;
+  if (rows64 && u_linear && f->aU == -2 && f->aF == -1) {
     int rc = build_deformed_fx_plan(pl, d, n, m, g, shifts, fast_table(cf, d, f->lambda), pack_dense(f->U, d, 1),
                                     f->lambda, tune);
     if (rc != QMC_EUNSUPPORTED) return rc;
   }
-  const bool rows64 = tab && sizeof(R) == 8;  // a CTA row per shift row
   if (!func) return fail(QMC_EUNSUPPORTED, "no deformed kernel for d=%d", d);
   auto cu = pack_dense(f->U, d, u_linear ? 1 : 2);
   for (size_t i = 0; i < cu.size(); ++i) base.cU[i] = (R)cu[i];
-  if (tab) {
+  if (rows64) {
     const std::vector<double> t = fast_table(cf, d, f->lambda);
-    static_assert(DefTab<kDefFastMax>::END <= kPolyCoefMax && DefTab<kDef2DMax>::END + 1 + kDef2DMax <= kPairCoefMax,
-                  "deformed constants");
-    if (packed) {
-      int o = 0;
-      for (double v : t) base.cp[o++] = make_float2((float)v, (float)v);
-      for (double v : cu) base.cp[o++] = make_float2((float)v, (float)v);
-    } else {
-      for (size_t i = 0; i < t.size(); ++i) base.cF[i] = (R)t[i];
-    }
+    static_assert(DefTab<kDefFastMax>::END <= kPolyCoefMax, "deformed constants");
+    for (size_t i = 0; i < t.size(); ++i) base.cF[i] = (R)t[i];
   } else {
     for (size_t i = 0; i < cf.size(); ++i) base.cF[i] = (R)cf[i];
     for (int k = 0; k < d; ++k)  // -lambda d2F/dy_k dy_l (constant: F has degree 2)
@@ -144,23 +130,34 @@ static int build_def(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
         base.cF[kDefHessOff + k * d + l] = (R)(-f->lambda * h);
       }
   }
+  if (packed) {  // (c, c) pairs: U's linear slots, F's slots, then the Hessian of F, k-major
+    int o = 0;
+    for (double v : cu) base.cp[o++] = make_float2((float)v, (float)v);
+    for (double v : cf) base.cp[o++] = make_float2((float)v, (float)v);
+    for (int k = 0; k < d; ++k)
+      for (int l = 0; l < d; ++l) {
+        const float h = (float)((k == l ? 2.0 : 1.0) * cf[q_off_host(d, std::min(k, l), std::max(k, l))]);
+        base.cp[o++] = make_float2(h, h);
+      }
+    static_assert(1 + kDef2DMax + poly_slots(kDef2DMax, 2) + kDef2DMax * kDef2DMax <= kPairCoefMax, "coefficient pairs");
+  }
   // Transform weight constants.  FP64 normalises each factor in the general
   // kernel; its FAST kernel cubes the product of 4x(1-x) in units of 2^-64.
-  // FP32 FAST cubes the product of its form's factors; other FP32 Korobov plans
-  // raise the product of the factors 4u to the power alpha: ((2a+1)!/(a!)^2 /
-  // 4^a) per dimension.
+  // FP32 FAST multiplies the factors u and cubes the product: (2a+1)!/(a!)^2
+  // = 140 per dimension remains; other FP32 Korobov plans raise the product of
+  // the factors 4u to the power alpha: ((2a+1)!/(a!)^2 / 4^a) per dimension.
   base.value_scale = 1.0;
   if (fast && sizeof(R) == 8) base.value_scale = korobov_scale(kKorCentred, d) * 0x1p-192;
   else if (sizeof(R) == 4 && base.tr == TR_KOROBOV)
-    base.value_scale = fast ? korobov_scale(form, d)
+    base.value_scale = fast ? korobov_scale(3, d)
                             : std::pow((double)base.kor[7] / std::pow(4.0, (double)base.alpha), (double)d);
   base.check_finite = 1;
   int nblk = 0, L = 0, occ = 0;
   uint64_t tiles = 0;
   int rc = grid_occupancy(func, 0, tune.occupancy, occ);
   if (rc) return rc;
-  const int mc = packed || rows64 ? kMcMax : kMcDeformed;
-  pl->grid_rows = packed ? (std::min(m, kMcMax) + 1) / 2 : (rows64 ? std::min(m, kMcMax) : 1);
+  const int mc = rows64 ? kMcMax : kMcDeformed;  // the others: as many as they have shared accumulators
+  pl->grid_rows = rows64 ? std::min(m, kMcMax) : 1;
   rc = grid_shape(occ, n, rows_cap(pl, occ, 0), tune.L, nblk, L, tiles);
   if (rc) return rc;
   pl->param_kind = sizeof(R) == 4 ? 1 : 2;
@@ -184,7 +181,7 @@ static int build_def(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t*
         set_shift(P, kk, i, shift_fixed64(shifts[(size_t)(kk < mk ? k0 + kk : k0) * d + i]));
     Launch ln;
     ln.func = func;
-    ln.grid = dim3(nblk, packed ? (mk + 1) / 2 : (rows64 ? mk : 1));
+    ln.grid = dim3(nblk, rows64 ? mk : 1);
     ln.params.resize(sizeof(P));
     std::memcpy(ln.params.data(), &P, sizeof(P));
     pl->launches.push_back(std::move(ln));

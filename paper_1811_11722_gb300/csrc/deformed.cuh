@@ -7,14 +7,20 @@
 //   J_kl = dw_k/dy_l = delta_kl - i lambda [delta_kl (1 - 2 y_k) dF/dy_k
 //                                           + y_k (1 - y_k) d2F/dy_k dy_l]
 //   f    = U(w)^aU F(w)^aF det J,   value = f * prod_i (transform weight)
-// F (and U) are dense polynomials of degree <= 2.  Two evaluations:
+// F (and U) are dense polynomials of degree <= 2.  Three evaluations:
 //
 // General.  dF/dy is a linear form read from F's nested-Horner coefficients,
 // -lambda d2F a constant matrix the host tabulates after them, and det J of J =
 // I + i M (M real) comes from LU factorisation with partial pivoting done by
 // conditional row swaps in registers (no dynamic register indexing).
 //
-// FAST (Korobov 3, J diagonally dominant on the cube, d <= kDefFastMax).  With
+// FAST FP32 (Korobov 3, J diagonally dominant on the cube).  The same without
+// pivoting, det J - 1 carried with the identity implicit (det_ipm_minus1).  The
+// minors below do not serve FP32: with F formed from its gradient, y.(dF(0) + g)
+// rounds with a bias, and estimates over 8e7 values lie up to 4e-9 from FP64
+// instead of 1.4e-9 (24 integrands, d = 5; 0.95 ms against 1.42).
+//
+// FAST FP64 (the same integrands, d <= kDefFastMax).  With
 // H the Hessian of F, b_k = -lambda y_k (1 - y_k) and m_k the diagonal of M,
 // J = diag(1 + i m) + i diag(b) H_off, so det J is multi-affine in the pairs
 // (1 + i m_k, i b_k):
@@ -33,24 +39,6 @@
 #include "rule_kernels.cuh"
 
 namespace qmc {
-
-// Operations of the FAST evaluation, scalar or packed.
-__device__ __forceinline__ float2 fma_(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
-template <class V>
-__device__ __forceinline__ V mul_(V a, V b) {
-  return a * b;
-}
-__device__ __forceinline__ float2 mul_(float2 a, float2 b) { return mul2(a, b); }
-template <class V>
-__device__ __forceinline__ V add_(V a, V b) {
-  return a + b;
-}
-__device__ __forceinline__ float2 add_(float2 a, float2 b) { return add2(a, b); }
-template <class V>
-__device__ __forceinline__ V neg_(V a) {
-  return -a;
-}
-__device__ __forceinline__ float2 neg_(float2 a) { return make_float2(-a.x, -a.y); }
 
 template <typename R>
 struct Cx {
@@ -115,7 +103,7 @@ __device__ __forceinline__ Cx<R> poly2_complex(const R* c, const Cx<R>* z) {
 // (nested layout c0, l_0 .. l_{D-1}).
 template <int D, typename R>
 __device__ __forceinline__ Cx<R> poly1_complex(const R* c, const Cx<R>* z) {
-  Cx<R> acc{c[0], R{}};
+  Cx<R> acc{c[0], R(0)};
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     acc.re = fma_(c[1 + i], z[i].re, acc.re);
@@ -198,7 +186,7 @@ __device__ __forceinline__ double def_coord_used(const RuleParams<R>& P, typenam
   else return coord_used<R>(b + shift_of(P, k, i));
 }
 
-// ---- FAST evaluation, for a scalar or a pair of shifts per register pair ----
+// ---- FAST evaluation in FP64 ----
 
 constexpr int kDefFastMax = 7;  // 2^d minors fit the coefficient table
 
@@ -216,64 +204,63 @@ struct DefTab {
 
 // The sum over the variables J..D-1 with S chosen among the first J: a
 // complex number.  Minors of single rows are zero (H_off has no diagonal).
-template <int D, int J, int S, class V>
-__device__ __forceinline__ Cx<V> def_node(const V* minors, const V* m, const V* b) {
+template <int D, int J, int S>
+__device__ __forceinline__ Cx<double> def_node(const double* minors, const double* m, const double* b) {
   if constexpr (J == D - 1) {
     if constexpr ((S & (S - 1)) == 0) {
-      return {V{}, mul_(b[J], minors[S | (1 << J)])};
+      return {0.0, b[J] * minors[S | (1 << J)]};
     } else {
-      return {minors[S], fma_(m[J], minors[S], mul_(b[J], minors[S | (1 << J)]))};
+      return {minors[S], fma_(m[J], minors[S], b[J] * minors[S | (1 << J)])};
     }
   } else {
-    const Cx<V> x = def_node<D, J + 1, S, V>(minors, m, b), y = def_node<D, J + 1, S | (1 << J), V>(minors, m, b);
-    return {fma_(neg_(b[J]), y.im, fma_(neg_(m[J]), x.im, x.re)), fma_(b[J], y.re, fma_(m[J], x.re, x.im))};
+    const Cx<double> x = def_node<D, J + 1, S>(minors, m, b), y = def_node<D, J + 1, S | (1 << J)>(minors, m, b);
+    return {fma_(-b[J], y.im, fma_(-m[J], x.im, x.re)), fma_(b[J], y.re, fma_(m[J], x.re, x.im))};
   }
 }
 
 // det J - 1: the empty set's branch carried without its 1, so that every
-// rounding is relative to a small quantity.  (Rounding values near 1 made the
-// FP32 configuration-4 integral 2e-8 too large.)
-template <int D, int J, class V>
-__device__ __forceinline__ Cx<V> def_root(const V* minors, const V* m, const V* b) {
+// rounding is relative to a small quantity.
+template <int D, int J>
+__device__ __forceinline__ Cx<double> def_root(const double* minors, const double* m, const double* b) {
   if constexpr (J == D - 1) {
-    return {V{}, m[J]};
+    return {0.0, m[J]};
   } else {
-    const Cx<V> x = def_root<D, J + 1, V>(minors, m, b), y = def_node<D, J + 1, 1 << J, V>(minors, m, b);
-    return {fma_(neg_(b[J]), y.im, fma_(neg_(m[J]), x.im, x.re)),
-            fma_(b[J], y.re, fma_(m[J], x.re, add_(m[J], x.im)))};
+    const Cx<double> x = def_root<D, J + 1>(minors, m, b), y = def_node<D, J + 1, 1 << J>(minors, m, b);
+    return {fma_(-b[J], y.im, fma_(-m[J], x.im, x.re)),
+            fma_(b[J], y.re, fma_(m[J], x.re, m[J] + x.im))};
   }
 }
 
 // The contour z = y + i v, F at it and det J - 1.
-template <int D, class V>
-__device__ __forceinline__ void def_fast(const V* c, const V* y, Cx<V>* z, Cx<V>& F, Cx<V>& dm1) {
+template <int D>
+__device__ __forceinline__ void def_fast(const double* c, const double* y, Cx<double>* z, Cx<double>& F, Cx<double>& dm1) {
   using T = DefTab<D>;
-  const V lam = c[T::LAM], nlam = c[T::LAM + 1], lam2 = c[T::LAM + 2];
-  V b[D], m[D], v[D];
-  V fy{}, fi{};  // y.(dF(0) + g), v.g
+  const double lam = c[T::LAM], nlam = c[T::LAM + 1], lam2 = c[T::LAM + 2];
+  double b[D], m[D], v[D];
+  double fy = 0.0, fi = 0.0;  // y.(dF(0) + g), v.g
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    V g = c[T::L + k];
+    double g = c[T::L + k];
 #pragma unroll
     for (int l = 0; l < D; ++l) g = fma_(c[T::h(k, l)], y[l], g);
-    b[k] = mul_(y[k], fma_(lam, y[k], nlam));  // -lambda y (1 - y)
-    v[k] = mul_(b[k], g);
-    m[k] = fma_(fma_(lam2, y[k], nlam), g, mul_(b[k], c[T::h(k, k)]));
-    const V s = add_(g, c[T::L + k]);
-    fy = k == 0 ? mul_(y[k], s) : fma_(y[k], s, fy);
-    fi = k == 0 ? mul_(v[k], g) : fma_(v[k], g, fi);
+    b[k] = y[k] * fma_(lam, y[k], nlam);  // -lambda y (1 - y)
+    v[k] = b[k] * g;
+    m[k] = fma_(fma_(lam2, y[k], nlam), g, b[k] * c[T::h(k, k)]);
+    const double s = g + c[T::L + k];
+    fy = k == 0 ? y[k] * s : fma_(y[k], s, fy);
+    fi = k == 0 ? v[k] * g : fma_(v[k], g, fi);
     z[k] = {y[k], v[k]};
   }
-  V fr = fma_(c[T::LAM + 3], fy, c[0]);
+  double fr = fma_(c[T::LAM + 3], fy, c[0]);
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    V r = mul_(c[T::Q + k], v[k]);
+    double r = c[T::Q + k] * v[k];
 #pragma unroll
     for (int l = k + 1; l < D; ++l) r = fma_(c[T::h(k, l)], v[l], r);
-    fr = fma_(neg_(v[k]), r, fr);
+    fr = fma_(-v[k], r, fr);
   }
   F = {fr, fi};
-  dm1 = def_root<D, 0, V>(c + T::M, m, b);
+  dm1 = def_root<D, 0>(c + T::M, m, b);
 }
 
 // det(I + i M) - 1 by LU without pivoting, for d above kDefFastMax (J = I + i M
@@ -334,11 +321,6 @@ __device__ __forceinline__ double def_coord64(uint64_t X, int i, double& wt, uin
   const long long bits = __double_as_longlong(__ull2double_rn(z));
   return __longlong_as_double(z ? bits - (63ll << 52) : 0);  // z 2^-63
 }
-template <bool TERM>
-__device__ __forceinline__ float def_coord64(uint64_t, int, float&, uint64_t&) {
-  return 0.0f;  // not instantiated with a use: FP32 FAST takes coord_fx
-}
-
 // Weighted complex value at one point and shift; *bad set when Im F(w) > 0.
 // FAST: compile-time Korobov weight 3 and no pivoting (host-checked);
 // otherwise the runtime transform and pivoted LU.  KU: degree of U (1 or 2),
@@ -368,9 +350,9 @@ __device__ __forceinline__ Cx<R> deformed_value(const RuleParams<R>& P, const ty
     if constexpr (!TERM) wt = __ull2double_rn(wf);
     wt = wt * wt * wt;  // 2^192 (prod u)^3
   }
-  if constexpr (FAST && D <= kDefFastMax) {
+  if constexpr (FAST && D <= kDefFastMax && sizeof(R) == 8) {
     Cx<R> z[D], F, dm1;
-    def_fast<D, R>(P.cF, y, z, F, dm1);
+    def_fast<D>(P.cF, y, z, F, dm1);
     Cx<R> U;
     if constexpr (KU == 1) U = poly1_complex<D, R>(P.cU, z);
     else U = poly2_complex<D, R>(P.cU, z);
@@ -533,51 +515,124 @@ __global__ void __launch_bounds__(kThreads)
 
 // --------------------------------------------- packed FP32, two shifts --
 //
-// The FAST variant (U of degree 1) for FP32 with two shifts per instruction:
-// every real quantity of a (point, shift) is a float2 holding shifts 2p and
-// 2p + 1, and the arithmetic is f32x2.  The constants come as (c, c) pairs from
-// the launch parameters (cp): DefTab's, then U's 1 + d slots, which fits for
-// d <= kDef2DMax.
+// The FAST variant (Korobov 3, unpivoted LU, U of degree 1) for FP32 with
+// two shifts per instruction: every real quantity of a (point, shift) is a
+// float2 holding shifts 2p and 2p + 1, and the arithmetic is f32x2.  The
+// coefficients come as (c, c) pairs from the launch parameters (cp):
+// U's 1 + d linear slots, F's nested degree-2 slots, then the Hessian of F
+// (2 q_kk on the diagonal) k-major, which fits for d <= kDef2DMax.
 constexpr int kDef2DMax = 5;
 
-__device__ __forceinline__ Cx<float2> cmul(const Cx<float2>& a, const Cx<float2>& b) {
-  return {fma2(neg_(a.im), b.im, mul2(a.re, b.re)), fma2(a.re, b.im, mul2(a.im, b.re))};
+struct Cx2 {
+  float2 re, im;
+};
+
+__device__ __forceinline__ float2 neg2(float2 a) { return mul2(a, make_float2(-1.0f, -1.0f)); }
+
+__device__ __forceinline__ Cx2 cmul2(const Cx2& a, const Cx2& b) {
+  return {fma2(neg2(a.im), b.im, mul2(a.re, b.re)), fma2(a.re, b.im, mul2(a.im, b.re))};
 }
 
 // 1 / a: (re, -im) / |a|^2 with the correctly rounded packed reciprocal
-__device__ __forceinline__ Cx<float2> crecip(const Cx<float2>& a) {
-  const float2 rn = recip_neg2(neg_(fma2(a.re, a.re, mul2(a.im, a.im))));  // 1 / |a|^2
-  return {mul2(a.re, rn), mul2(neg_(a.im), rn)};
+__device__ __forceinline__ Cx2 crecip2(const Cx2& a) {
+  const float2 rn = recip_neg2(fma2(a.re, a.re, mul2(a.im, a.im)));  // -1 / |a|^2
+  return {mul2(a.re, neg2(rn)), mul2(a.im, rn)};
 }
 
-template <int D, int ALPHA>
-__device__ __forceinline__ Cx<float2> deformed_value2(const RuleParams<float>& P, const uint32_t* base, int k,
-                                                      bool& bad_a, bool& bad_b) {
+template <int D>
+__device__ __forceinline__ Cx2 deformed_value2(const RuleParams<float>& P, const uint32_t* base, int p, bool& bad_a,
+                                               bool& bad_b) {
   float2 y[D];
-  float2 w = make_float2(1.0f, 1.0f);
+  float wa = 1.0f, wb = 1.0f;
 #pragma unroll
   for (int i = 0; i < D; ++i)
-    y[i] = coord_fx2<TR_KOROBOV, ALPHA, true>(base[i] + P.shiftx[k][i], base[i] + P.shiftx[k + 1][i], P.kor, w);
-  Cx<float2> z[D], F, dm1;
-  def_fast<D, float2>(P.cp, y, z, F, dm1);
-  const Cx<float2> U = poly1_complex<D, float2>(P.cp + DefTab<D>::END, z);
+    y[i] = make_float2(coord_fx<TR_KOROBOV, 3>(base[i] + P.shiftx[2 * p][i], P.kor, wa),
+                       coord_fx<TR_KOROBOV, 3>(base[i] + P.shiftx[2 * p + 1][i], P.kor, wb));
+  const float2* cu = P.cp;
+  const float2* cf = P.cp + 1 + D;
+  const float2* H = cf + poly_slots(D, 2);
+  const float2 nlam = make_float2(-P.lam, -P.lam);
+  const float2 one = make_float2(1.0f, 1.0f), zero = make_float2(0.0f, 0.0f);
+  Cx2 z[D];
+  float2 ar[D][D], ai[D][D];  // B = J - I = i M (real parts zero)
+#pragma unroll
+  for (int kk = 0; kk < D; ++kk) {
+    float2 gr = cf[l_off(D, kk)];  // dF/dy_kk
+#pragma unroll
+    for (int j = 0; j < D; ++j) gr = fma2(H[kk * D + j], y[j], gr);
+    const float2 na = mul2(nlam, fma2(neg2(y[kk]), y[kk], y[kk]));  // -lambda y (1 - y)
+    z[kk] = {y[kk], mul2(na, gr)};
+#pragma unroll
+    for (int l = 0; l < D; ++l) {
+      ar[kk][l] = zero;
+      ai[kk][l] = mul2(na, H[kk * D + l]);
+    }
+    ai[kk][kk] = fma2(mul2(nlam, fma2(y[kk], make_float2(-2.0f, -2.0f), one)), gr, ai[kk][kk]);
+  }
+  // det J - 1 by LU without pivoting on B = J - I (J diagonally dominant,
+  // shown by the host; see det_ipm_minus1 for why the identity stays implicit)
+  Cx2 dm1{zero, zero};
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    const Cx2 b{ar[c][c], ai[c][c]};
+    const Cx2 t = cmul2(dm1, b);
+    dm1.re = add2(add2(dm1.re, b.re), t.re);
+    dm1.im = add2(add2(dm1.im, b.im), t.im);
+    if (c + 1 < D) {
+      const Cx2 inv = crecip2(Cx2{add2(one, b.re), b.im});
+#pragma unroll
+      for (int r = c + 1; r < D; ++r) {
+        const Cx2 f = cmul2(Cx2{ar[r][c], ai[r][c]}, inv);
+        const float2 frn = neg2(f.re), fin = neg2(f.im);
+#pragma unroll
+        for (int q = c + 1; q < D; ++q) {  // a_rq -= f a_cq, as four fused steps
+          ar[r][q] = fma2(frn, ar[c][q], ar[r][q]);
+          ar[r][q] = fma2(f.im, ai[c][q], ar[r][q]);
+          ai[r][q] = fma2(frn, ai[c][q], ai[r][q]);
+          ai[r][q] = fma2(fin, ar[c][q], ai[r][q]);
+        }
+      }
+    }
+  }
+  // U (degree 1) and F (degree 2) at w, real coefficients
+  Cx2 U{cu[0], zero};
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    U.re = fma2(cu[1 + i], z[i].re, U.re);
+    U.im = fma2(cu[1 + i], z[i].im, U.im);
+  }
+  Cx2 F{cf[0], zero};
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    Cx2 r{cf[l_off(D, i)], zero};
+#pragma unroll
+    for (int j = i; j < D; ++j) {
+      const float2 q = cf[q_off(D, i, j)];
+      r.re = fma2(q, z[j].re, r.re);
+      r.im = fma2(q, z[j].im, r.im);
+    }
+    const float2 nzi = neg2(z[i].im);
+    F.re = fma2(z[i].re, r.re, F.re);
+    F.re = fma2(nzi, r.im, F.re);
+    F.im = fma2(z[i].re, r.im, F.im);
+    F.im = fma2(z[i].im, r.re, F.im);
+  }
   bad_a = F.im.x > 0.0f;  // the contour left the allowed half-plane, Im F(w) > 0
   bad_b = F.im.y > 0.0f;
-  const Cx<float2> rv = crecip(cmul(cmul(U, U), F));
-  const Cx<float2> t = cmul(dm1, rv);
-  w = korobov_weight_fx2(w);  // the constant per dimension in FP64 by the final pass
-  return {mul2(add2(rv.re, t.re), w), mul2(add2(rv.im, t.im), w)};
+  const Cx2 rv = crecip2(cmul2(cmul2(U, U), F));
+  const Cx2 t = cmul2(dm1, rv);
+  Cx2 v{add2(rv.re, t.re), add2(rv.im, t.im)};
+  const float2 w = korobov_weight_fx2(make_float2(wa, wb));  // (prod u)^3; 140^d in FP64 by the final pass
+  v.re = mul2(v.re, w);
+  v.im = mul2(v.im, w);
+  return v;
 }
 
-// A pair of shift rows per CTA row: a pair's points stay in one thread's
-// registers from start to end, and few points still spread over the chip.
-// At d = 5: 322 issue slots a value (128 packed operations of two), against 680
-// with LU; the FP32 pipe is 83% busy.  n = 4194301, m = 20: 1.415 -> 0.957 ms.
-template <int D, int ALPHA>
-__global__ void __launch_bounds__(kThreads, 2)
+template <int D>
+__global__ void __launch_bounds__(kThreads, 2)  // two CTAs per SM: 128 registers, no spills at d = 5
     deformed2_kernel(const __grid_constant__ RuleParams<float> P, double* __restrict__ partial,
                      unsigned long long* __restrict__ counters, const SampleIO sio) {
-  if (sio.count > 0) {  // sampling: the same evaluation, one (point, shift) per thread in both halves
+  if (sio.count > 0) {  // sampling: the scalar path of the same variant, one (point, shift) per thread
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= sio.count) return;
     const uint64_t j = sio.j[s];
@@ -586,63 +641,95 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       uint32_t idx = lattice_index(j, P.g[i], P.n);
-      base[i] = sec_base<float, ALPHA>(idx, P.rc, j, i);
+      base[i] = def_base<float, true>(idx, P.rc, j, i);
       if (sio.idx) sio.idx[(size_t)s * D + i] = idx;
-      if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<float, ALPHA>(P, base[i], k, i);
+      if (sio.coord) sio.coord[(size_t)s * D + i] = def_coord_used<float, true>(P, base[i], k, i);
     }
-    bool bad_a, bad_b;
-    const Cx<float2> v = deformed_value2<D, ALPHA>(P, base, k & ~1, bad_a, bad_b);
-    sio.values[2 * (size_t)s] = (double)((k & 1) ? v.re.y : v.re.x) * P.value_scale;
-    sio.values[2 * (size_t)s + 1] = (double)((k & 1) ? v.im.y : v.im.x) * P.value_scale;
+    bool bad;
+    Cx<float> v = deformed_value<float, D, true, 1>(P, base, k, bad);
+    sio.values[2 * (size_t)s] = (double)v.re * P.value_scale;
+    sio.values[2 * (size_t)s + 1] = (double)v.im * P.value_scale;
     return;
   }
-  const int k = 2 * blockIdx.y;
-  const bool has_b = k + 1 < P.m_launch;  // an odd last shift: the pair's second row is evaluated, not kept
-  float2 zero = make_float2(0.0f, 0.0f);
-  float2 hr = zero, lr = zero, hi = zero, li = zero;  // compensated sums of both parts
+  __shared__ double accs[2][kMcDeformed][kThreads];
+  const uint32_t n = (uint32_t)P.n;
+  const int mk = P.m_launch;
+  for (int kk = 0; kk < kMcDeformed; ++kk) {
+    accs[0][kk][threadIdx.x] = 0.0;
+    accs[1][kk][threadIdx.x] = 0.0;
+  }
   unsigned nbad = 0, ndef = 0;
   const uint64_t tile_pts = (uint64_t)kThreads * (uint64_t)P.L;
   for (uint64_t tile = blockIdx.x; tile < P.tiles; tile += gridDim.x) {
     const uint64_t j0 = tile * tile_pts + threadIdx.x;
     if (j0 >= P.n) continue;
-    const uint64_t left = (P.n - j0 + kThreads - 1) / kThreads;
+    uint64_t left = (P.n - j0 + kThreads - 1) / kThreads;
     const int steps = left < (uint64_t)P.L ? (int)left : P.L;
-    FxWalk<D, ALPHA> walk;
-    walk.start(P, j0);
 #pragma unroll 1
-    for (int s = 0; s < steps; ++s) {
-      uint32_t base[D];
-      walk.bases(base);
-      bool bad_a, bad_b;
-      Cx<float2> v = deformed_value2<D, ALPHA>(P, base, k, bad_a, bad_b);
-      ndef += (bad_a ? 1u : 0u) + ((bad_b && has_b) ? 1u : 0u);
-      const bool ok_a = finite_(v.re.x) && finite_(v.im.x);
-      const bool ok_b = finite_(v.re.y) && finite_(v.im.y);
-      nbad += (ok_a ? 0u : 1u) + ((ok_b || !has_b) ? 0u : 1u);
-      // Korobov-weighted values: every value into the (hi, lo) pairs
-      fast2sum_add2(hr, lr, make_float2(ok_a ? v.re.x : 0.0f, ok_b ? v.re.y : 0.0f));
-      fast2sum_add2(hi, li, make_float2(ok_a ? v.im.x : 0.0f, ok_b ? v.im.y : 0.0f));
-      walk.step(P);
+    for (int kk = 0; kk < mk; kk += 2) {
+      const bool has_b = kk + 1 < mk;  // an odd last shift: the pair's second row is evaluated, not kept
+      uint32_t idx[D];
+#pragma unroll
+      for (int i = 0; i < D; ++i) idx[i] = lattice_index(j0, P.g[i], P.n);
+      Acc<float> are_a, aim_a, are_b, aim_b;
+      are_a.init();
+      aim_a.init();
+      are_b.init();
+      aim_b.init();
+#pragma unroll 1
+      for (int s = 0; s < steps; ++s) {
+        const uint64_t j = j0 + (uint64_t)s * kThreads;
+        uint32_t base[D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) base[i] = def_base<float, true>(idx[i], P.rc, j, i);
+        bool bad_a, bad_b;
+        Cx2 v = deformed_value2<D>(P, base, kk >> 1, bad_a, bad_b);
+        ndef += (bad_a ? 1u : 0u) + ((bad_b && has_b) ? 1u : 0u);
+        const bool ok_a = finite_(v.re.x) && finite_(v.im.x);
+        const bool ok_b = finite_(v.re.y) && finite_(v.im.y);
+        nbad += (ok_a ? 0u : 1u) + ((ok_b || !has_b) ? 0u : 1u);
+        are_a.add(ok_a ? v.re.x : 0.0f);
+        aim_a.add(ok_a ? v.im.x : 0.0f);
+        are_b.add(ok_b ? v.re.y : 0.0f);
+        aim_b.add(ok_b ? v.im.y : 0.0f);
+#pragma unroll
+        for (int i = 0; i < D; ++i) idx[i] = index_step(idx[i], P.gstep[i], n);
+        {  // Korobov-weighted values: every value into the (hi, lo) pairs
+          are_a.fold();
+          aim_a.fold();
+          are_b.fold();
+          aim_b.fold();
+        }
+      }
+      accs[0][kk][threadIdx.x] += are_a.thread_total();
+      accs[1][kk][threadIdx.x] += aim_a.thread_total();
+      if (has_b) {
+        accs[0][kk + 1][threadIdx.x] += are_b.thread_total();
+        accs[1][kk + 1][threadIdx.x] += aim_b.thread_total();
+      }
     }
   }
-  __shared__ double red[kThreads / 32][4];
+  __shared__ double red[kThreads / 32][kMcDeformed][2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float h4[4] = {hr.x, hi.x, hr.y, hi.y}, l4[4] = {lr.x, li.x, lr.y, li.y};
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    warp_sum_ff(h4[q], l4[q]);
-    if (lane == 0) red[warp][q] = (double)h4[q] + (double)l4[q];
+  for (int kk = 0; kk < mk; ++kk) {
+    const double tr = warp_sum_d(accs[0][kk][threadIdx.x]);
+    const double ti = warp_sum_d(accs[1][kk][threadIdx.x]);
+    if (lane == 0) {
+      red[warp][kk][0] = tr;
+      red[warp][kk][1] = ti;
+    }
   }
-  const unsigned long long b1 = warp_sum_u64((unsigned long long)nbad);
-  const unsigned long long b2 = warp_sum_u64((unsigned long long)ndef);
+  unsigned long long b1 = warp_sum_u64((unsigned long long)nbad);
+  unsigned long long b2 = warp_sum_u64((unsigned long long)ndef);
   if (lane == 0 && b1) atomicAdd(&counters[0], b1);
   if (lane == 0 && b2) atomicAdd(&counters[1], b2);
   __syncthreads();
-  if (threadIdx.x < (has_b ? 4 : 2)) {
+  if (threadIdx.x < 2 * mk) {
+    const int kk = threadIdx.x >> 1, part = threadIdx.x & 1;
     double s = 0.0;
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) s += red[w][threadIdx.x];
-    partial[((size_t)(P.k_base + k + (threadIdx.x >> 1)) * P.nblk + blockIdx.x) * 2 + (threadIdx.x & 1)] = s;
+    for (int w = 0; w < kThreads / 32; ++w) s += red[w][kk][part];
+    partial[((size_t)(P.k_base + kk) * P.nblk + blockIdx.x) * 2 + part] = s;
   }
 }
 

@@ -332,7 +332,7 @@ __device__ __forceinline__ float coord_fx(uint32_t X, const float* kor, float& w
 // coord_fx for two shifts at once: the same operations per lane (so the same
 // values bit for bit) in packed f32x2 arithmetic; w holds the two products
 // of the Korobov factors.
-template <int TR, int ALPHA, bool CLAMP = false>
+template <int TR, int ALPHA>
 __device__ __forceinline__ float2 coord_fx2(uint32_t Xa, uint32_t Xb, const float* kor, float2& w) {
   if constexpr (TR == TR_NONE) {
     return make_float2(__uint2float_rn(Xa), __uint2float_rn(Xb));
@@ -343,9 +343,7 @@ __device__ __forceinline__ float2 coord_fx2(uint32_t Xa, uint32_t Xb, const floa
     q = fma2(q, u, make_float2(8 * 0x1p-36f, 8 * 0x1p-36f));
     q = fma2(q, u, make_float2(16 * 0x1p-36f, 16 * 0x1p-36f));
     w = mul2(w, u);
-    if constexpr (CLAMP)
-      return make_float2(__saturatef(__fmaf_rn(T.x, q.x, 0.5f)), __saturatef(__fmaf_rn(T.y, q.y, 0.5f)));
-    else return fma2(T, q, make_float2(0.5f, 0.5f));
+    return fma2(T, q, make_float2(0.5f, 0.5f));
   } else {
     const float2 a = make_float2(fabsf(__int2float_rn((int32_t)Xa)), fabsf(__int2float_rn((int32_t)Xb)));
     if constexpr (TR == TR_BAKER) {

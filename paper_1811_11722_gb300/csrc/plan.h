@@ -81,7 +81,7 @@ struct Plan {
                             // 0: fixed lattice
   int grid_occ = 1;         // CTAs per SM the launch shape assumes
   int grid_rows = 1;        // CTA rows of the largest launch, one per shift row or pair (separable FP64,
-                            // deformed FAST kernels), else 1
+                            // deformed FP64 FAST, fixed-point kernels), else 1
   bool grid_capped = true;  // the launch shape honours a cap on CTAs (rule plans; not deformed ones)
 };
 

@@ -25,8 +25,7 @@ constexpr int kDFast = 8;       // largest d with a specialised sector kernel
 constexpr int kPolyCoefMax = 176;  // nested-Horner slots: d=8 degree 3 needs 165, deformed constants at d=7 need 174
 constexpr int kTermsMax = 64;   // sparse monomials per polynomial (general kernel)
 constexpr int kThreads = 256;   // threads per CTA of the rule kernels
-constexpr int kPairCoefMax = 72;  // packed FP32 path: U (deg 1) + F (deg 2) slots at d = 8 is 54, deformed
-                                  // constants and U at d = 5 are 67
+constexpr int kPairCoefMax = 56;  // packed FP32 path: U (deg 1) + F (deg 2) slots at d = 8 is 54
 constexpr int kEpsMax = QMC_EPS_MAX;  // epsilon orders of one pass (Eq. 7 expansion)
 constexpr int kEpsAcc = 24;     // shifts x orders accumulated by one epsilon launch
 
