@@ -1116,9 +1116,11 @@ __device__ __forceinline__ void multi_body(const MultiParams& M, double* __restr
       partial[slot(M.s_base + s) + 1] = 0.0;
     }
     // the sum group's slot: this chunk's integrands in order, on top of the
-    // earlier chunks' launches
+    // earlier chunks' launches.  The barrier names all the lanes that write: a
+    // launch without one of its shift rows has parted them above.
+    constexpr unsigned kLanes = SC * MC == 32 ? 0xffffffffu : (1u << (SC * MC % 32)) - 1;
     red[0][threadIdx.x] = acc_s;
-    __syncwarp(__activemask());
+    __syncwarp(kLanes);
     if (s == 0 && kk < P.m_launch) {
       double tot = M.s_base == 0 ? 0.0 : partial[slot(M.count)];
 #pragma unroll

@@ -1,0 +1,29 @@
+"""Results that depend on an order inside a kernel or between overlapped kernels."""
+import numpy as np
+import pytest
+
+from paper_1811_11722_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def Q():
+    from paper_1811_11722_gb300 import build, qmc
+    build.build_library()
+    return qmc
+
+
+@pytest.mark.parametrize("count", [9, 11, 16])
+@pytest.mark.parametrize("transform,alpha", [("baker", 0), ("korobov", 3)])
+def test_multi_sum_slots(Q, count, transform, alpha):
+    """The sum group with an odd shift count (the last launch of a chunk keeps one of its two rows) and a
+    short, an odd and a full last chunk: per shift, the integrands' values added.  The two differ in
+    the order of at most count + 600 additions of positive numbers: 700 * 2^-53 = 8e-14."""
+    probs = I.config3_shared(count=count, d=4, n=50021, m=5, transform=transform, alpha=alpha)
+    g = I.random_generating_vector(I.SplitMix64(63), 4, probs[0].n)
+    fs = [Q.integrand_from_problem(p, "fp32") for p in probs]
+    res, ps = Q.qmc_integrate_multi(4, probs[0].n, 5, g, probs[0].shifts, Q.transform(transform, alpha), fs,
+                                    want_per_shift=True)
+    assert np.allclose(ps[count, :, 0], ps[:count, :, 0].sum(axis=0), rtol=8e-14, atol=0)
+    assert abs(res[count].mean[0] - ps[count, :, 0].mean()) <= 8e-14 * abs(res[count].mean[0])
