@@ -104,8 +104,8 @@ __device__ __forceinline__ double widen(float f) {
 // The step's bias corrections are computed before the wait for the gradient.
 constexpr int kAdamWarps = 8, kAdamLoads = 16;
 __global__ void __launch_bounds__(kAdamWarps * 32)
-    cv_adam_kernel(const float* __restrict__ grad_part, int nchunk, int npar, float* __restrict__ a,
-                   float* __restrict__ m1, float* __restrict__ m2, int step, float lr, int band) {
+    cv_adam_kernel(float* grad_part, int nchunk, int npar, float* a, float* m1, float* m2, int step, float lr,
+                   int band) {
   __shared__ double part[kAdamWarps][32];
   __shared__ float corr[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -114,13 +114,16 @@ __global__ void __launch_bounds__(kAdamWarps * 32)
   grid_launch_next();
   if (warp == 1 && lane < 2) corr[lane] = 1.0f - powf(lane ? b2 : b1, (float)step);
   grid_wait();
+  const bool mine = warp == 0 && q < npar;
+  const float a0 = mine ? ld_fresh(a + q) : 0.0f, m10 = mine ? ld_fresh(m1 + q) : 0.0f;
+  const float m20 = mine ? ld_fresh(m2 + q) : 0.0f;
   double g = 0.0;
   if (q < npar)
     for (int c = warp; c < nchunk; c += kAdamLoads * kAdamWarps) {
       float v[kAdamLoads];
 #pragma unroll
       for (int u = 0; u < kAdamLoads; ++u)
-        v[u] = c + kAdamWarps * u < nchunk ? grad_part[(size_t)(c + kAdamWarps * u) * npar + q] : 0.0f;
+        v[u] = c + kAdamWarps * u < nchunk ? ld_fresh(grad_part + (size_t)(c + kAdamWarps * u) * npar + q) : 0.0f;
       bool plain = true;
 #pragma unroll
       for (int u = 0; u < kAdamLoads; ++u) plain &= widens(v[u]);
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(kAdamWarps * 32)
     }
   part[warp][lane] = g;
   __syncthreads();
-  if (warp != 0 || q >= npar) return;
+  if (!mine) return;
   if (band > 0 && q % kCvK >= band) {  // a band-limited fit holds the higher degrees at zero
     a[q] = 0.0f;
     return;
@@ -144,13 +147,13 @@ __global__ void __launch_bounds__(kAdamWarps * 32)
 #pragma unroll
   for (int w = 0; w < kAdamWarps; ++w) tot += part[w][lane];
   const float gf = (float)tot;
-  const float mm = b1 * m1[q] + (1.0f - b1) * gf;
-  const float vv = b2 * m2[q] + (1.0f - b2) * gf * gf;
+  const float mm = b1 * m10 + (1.0f - b1) * gf;
+  const float vv = b2 * m20 + (1.0f - b2) * gf * gf;
   m1[q] = mm;
   m2[q] = vv;
   const float mh = mm / corr[0];
   const float vh = vv / corr[1];
-  a[q] -= lr * mh / (sqrtf(vh) + eps);
+  a[q] = a0 - lr * mh / (sqrtf(vh) + eps);
 }
 
 static const void* cv_fit_for(int d, size_t* smem) {

@@ -374,12 +374,30 @@ struct CvFitSmem {
 // wait for the kernels this one depends on (a no-op unless launched with the
 // programmatic attribute); let the next one start its prologue
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Loads of what the kernel before wrote while this one was already resident: from L2
+// (this SM's first-level cache may hold the line from an earlier step) and where
+// they stand, after the wait.  Such memory is not read-only for the kernel's
+// lifetime, so its pointers carry neither const nor __restrict__.
+__device__ __forceinline__ float ld_fresh(float* p) {
+  float v;
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_fresh4(float* p) {
+  float4 v;
+  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p)
+               : "memory");
+  return v;
+}
 
 template <int D>
 __global__ void __launch_bounds__(kCvFitWarps * 32)
-    cv_fit_kernel(const uint16_t* __restrict__ Bf, const double* __restrict__ hv, const float* __restrict__ a, int P,
-                  int Ppad, float* __restrict__ grad_part, double* __restrict__ loss_part) {
+    cv_fit_kernel(const uint16_t* __restrict__ Bf, const double* __restrict__ hv, float* a, int P, int Ppad,
+                  float* grad_part, double* loss_part) {
   constexpr int W = kCvFitWarps;
   static_assert(D <= W, "one warp per dimension in the backward");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -407,12 +425,18 @@ __global__ void __launch_bounds__(kCvFitWarps * 32)
   const auto pilot = [&](int j) { return j < P ? hv[2 * (size_t)j] : 0.0; };
   double h = pilot((blockIdx.x * W + warp) * 16 + row);
   grid_wait();
-  grid_launch_next();
+  constexpr int kLoads = (kCvR * D * kCvK + W * 32 * 4 - 1) / (W * 32 * 4);
+  float4 av[kLoads];
 #pragma unroll
-  for (int u = 0; u < kCvR * D * kCvK / (W * 32 * 4) + 1; ++u) {
+  for (int u = 0; u < kLoads; ++u) {
+    const int q = 4 * (u * W * 32 + (int)threadIdx.x);
+    if (q < kCvR * D * kCvK) av[u] = ld_fresh4(a + q);
+  }
+#pragma unroll
+  for (int u = 0; u < kLoads; ++u) {
     const int q = 4 * (u * W * 32 + (int)threadIdx.x);
     if (q < kCvR * D * kCvK) {
-      const float4 v = *reinterpret_cast<const float4*>(a + q);
+      const float4 v = av[u];
       const int k = q % kCvK, i = (q / kCvK) % D, r = q / (kCvK * D);
       uint2 w;
       w.x = bf16_bits(v.x) | (uint32_t)bf16_bits(v.y) << 16;
@@ -420,6 +444,7 @@ __global__ void __launch_bounds__(kCvFitWarps * 32)
       *reinterpret_cast<uint2*>(&S.as[i][r * kCvK + cv_swz(r, k)]) = w;
     }
   }
+  grid_launch_next();  // the parameters are in: the next Adam step, which writes them, may come up
   // fragment words of row g (and g + 8, the same permutation) at degrees 16 ks + 2t and + 8
   int pos[2][2];
 #pragma unroll

@@ -27,3 +27,22 @@ def test_multi_sum_slots(Q, count, transform, alpha):
                                     want_per_shift=True)
     assert np.allclose(ps[count, :, 0], ps[:count, :, 0].sum(axis=0), rtol=8e-14, atol=0)
     assert abs(res[count].mean[0] - ps[count, :, 0].mean()) <= 8e-14 * abs(res[count].mean[0])
+
+
+@pytest.mark.parametrize("d,n_pilot", [(8, 16381), (3, 33013)])
+def test_fit_is_reproducible(Q, d, n_pilot):
+    """One fit many times: every addition has its place, so parameters and losses keep their bits.  Two sizes: one batch
+    of tiles per block of the fit kernel, and several."""
+    rng = I.SplitMix64(71 + d)
+    U, F = I.random_poly(rng, d, d, 0), I.random_poly(rng, d, 0, min(24, d * (d + 1) // 2))
+    f = Q.Integrand(Q.QMC_F_SECTOR, d, Q.QMC_FP32EVAL, (U.coef, U.expo), (F.coef, F.expo))
+    g = I.random_generating_vector(rng, d, n_pilot)
+    shift = np.array([rng.uniform() for _ in range(d)])
+    cfg = Q.qmc_cv_config(16, 32, 1, 60, 1e-2, 0, 5)
+    first = None
+    for _ in range(30):
+        a, losses = Q.qmc_cv_train(d, n_pilot, g, shift, Q.transform("none"), f, cfg)
+        got = np.concatenate([np.asarray(a, dtype=np.float64).ravel(), np.asarray(losses, dtype=np.float64).ravel()])
+        assert np.all(np.isfinite(got))
+        first = got if first is None else first
+        assert np.array_equal(got, first)
