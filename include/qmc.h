@@ -92,10 +92,11 @@ enum {
 
 /* Arithmetic of the per-point evaluation.  Per-shift sums, Q^(k), Qbar and
  * sigma^2 are FP64 on the device in both modes.
- * FP64: coordinates, transform and f in double, or, where the integrand's
- *   coefficients bound the error below double's, in 64-bit fixed point (U^-2
- *   F^-1 sectors of degree 1 and 2 with none, baker or Korobov 3; deformed ones
- *   under Korobov 3 with d <= 6).
+ * FP64: coordinates, transform and f in double, or, where the coefficients keep
+ *   the error of an estimate within 1.5 2^-53 of it (one rounding of the result),
+ *   in 64-bit fixed point: U^-2 F^-1 sectors of degree 1 and 2 with none, baker or
+ *   Korobov 3 whose coefficients add up to at most 1000 times the constant term,
+ *   and deformed ones under Korobov 3 with d <= 6.
  * FP32EVAL: coordinates from 32-bit fixed point, transform and f in float,
  *   compensated float run sums promoted to double per thread.  Under the
  *   Korobov transform every value enters the compensated sum on its own (its

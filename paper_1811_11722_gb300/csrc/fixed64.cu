@@ -19,17 +19,23 @@ void fx_split(double c, int k, uint32_t* h, uint32_t* l) {
   *l = (uint32_t)(q & 0x0FFFFFFFu);
 }
 
-uint64_t fx_fixed(double c, int k) { return (uint64_t)std::llrint(std::ldexp(c, k)); }
+// c 2^k + more, rounded once
+uint64_t fx_fixed(double c, int k, double more) {
+  const double q = std::ldexp(c, k), whole = std::floor(q);
+  return (uint64_t)whole + (uint64_t)std::llrint((q - whole) + more);
+}
 
-// k with sum(c) 2^k in [2^61, 2^63), kept clear of 2^63 by rounding; false when
-// the constant term is too small against the sum or the scale is extreme.
-bool fx_scale(const std::vector<double>& c, int* k) {
+// k with sum(c) 2^k in [2^62, 2^64), kept clear of 2^64 by rounding, and the ratio
+// of the sum to the constant term; false when that is too large or the scale is
+// extreme.
+bool fx_scale(const std::vector<double>& c, int* k, double* ratio) {
   double sum = 0.0;
   for (double v : c) sum += v;
   if (!(c[0] > 0.0) || !std::isfinite(sum) || c[0] * kFxRange < sum) return false;
   int x = 0;
   const double f = std::frexp(sum, &x);
-  *k = 63 - x - (f > 1.0 - 0x1p-30 ? 1 : 0);
+  *k = 64 - x - (f > 1.0 - 0x1p-30 ? 1 : 0);
+  *ratio = sum / c[0];
   return std::abs(*k) <= 200;
 }
 
@@ -97,7 +103,8 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
     return QMC_EUNSUPPORTED;
   const std::vector<double> cu = pack_dense(f->U, d, 1), cf = pack_dense(f->F, d, 2);
   int ku = 0, kf = 0;
-  if (!fx_scale(cu, &ku) || !fx_scale(cf, &kf)) return QMC_EUNSUPPORTED;
+  double ru = 0.0, rf = 0.0;
+  if (!fx_scale(cu, &ku, &ru) || !fx_scale(cf, &kf, &rf)) return QMC_EUNSUPPORTED;
   const int tr = t.kind == QMC_TRANSFORM_KOROBOV ? TR_KOROBOV : (t.kind == QMC_TRANSFORM_BAKER ? TR_BAKER : TR_NONE);
   const void* func = fx_kernel(d, tr);
   if (!func) return QMC_EUNSUPPORTED;
@@ -107,32 +114,41 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
   base.d = d;
   base.tr = tr;
   fx_lattice(base, n, g);
-  // What the sums drop on average, in their own units: a dot product the
-  // fraction of its cross sum (1/2), per term the last four bits of the
-  // coordinate (7.5 of 16 against the coefficient's high word) and the low words'
-  // product; F per row half of that (z_i is 1/2 on average) and 1.25 of its product.
-  const auto dropped = [](uint32_t ch, uint32_t cl) {
-    return 7.5 * std::ldexp((double)ch, -32) + 0.5 * std::ldexp((double)cl, -28);
+  base.peaked = tr == TR_KOROBOV && std::max(ru, rf) > kFxPeaked ? 1 : 0;
+  // What is added to the constants: what the sums lose on average at z = 0, in
+  // their own units.  A dot product drops the fraction of its cross sum (1/2) and per
+  // term the last four bits of the coordinate (7.5 of 16 against the coefficient's
+  // high word) and the low words' product; a row's product 3/4.  The coordinates are
+  // themselves too large by `high` 2^-63 there (truncated products; Korobov's measured
+  // on the CPU over s = 1e-6..0.07).
+  const double high = tr == TR_KOROBOV ? 6.5 : (tr == TR_BAKER ? -0.5 : -0.25);
+  const auto lost = [&](double c, int k, uint32_t ch, uint32_t cl) {
+    return 7.5 * std::ldexp((double)ch, -32) + 0.5 * std::ldexp((double)cl, -28) - high * std::ldexp(c, k - 64);
   };
-  double lost = 0.5;
+  double more = 0.5;
   for (int i = 0; i < d; ++i) {
     fx_split(cu[1 + i], ku, &base.uh[i], &base.ul[i]);
-    lost += dropped(base.uh[i], base.ul[i]);
+    more += lost(cu[1 + i], ku, base.uh[i], base.ul[i]);
   }
-  base.u0 = fx_fixed(cu[0], ku - 1) + (uint64_t)std::llrint(lost);
-  lost = 0.0;
+  base.u0 = fx_fixed(cu[0], ku - 1, more);
+  more = 0.0;
   for (int i = 0, off = 1, o = 0; i < d; ++i) {
-    base.fl[i] = fx_fixed(cf[off++], kf - 1);
-    base.fmask[i] = base.fl[i] ? 1u : 0u;
+    const double l = cf[off++];
     double row = 0.5;
-    for (int j = i; j < d; ++j, ++o) {
-      fx_split(cf[off++], kf, &base.fh[o], &base.fq[o]);
-      if (base.fh[o] | base.fq[o]) base.fmask[i] |= 2u << (j - i);
-      row += dropped(base.fh[o], base.fq[o]);
+    bool any = l != 0.0;
+    for (int j = i; j < d; ++j, ++o, ++off) {
+      fx_split(cf[off], kf, &base.fh[o], &base.fq[o]);
+      if (!(base.fh[o] | base.fq[o])) continue;
+      base.fmask[i] |= 2u << (j - i);
+      row += lost(cf[off], kf, base.fh[o], base.fq[o]);
+      any = true;
     }
-    if (base.fmask[i]) lost += 0.25 * row + 0.75;
+    if (!any) continue;
+    base.fmask[i] |= 1u;
+    base.fl[i] = (uint64_t)std::max<int64_t>(0, (int64_t)fx_fixed(l, kf - 1, row));
+    more += 0.75 - high * std::ldexp(l, kf - 65);
   }
-  base.f0 = fx_fixed(cf[0], kf - 2) + (uint64_t)std::llrint(lost);
+  base.f0 = fx_fixed(cf[0], kf - 2, more);
   // value = v 2^(2 su + sf) 2^(2 ku + kf - 252), the smallest shift 2 su + sf
   // taken out; Korobov: v carries 4 more bits, and its weights are (4x(1-x))^3
   // against Eq. (5)'s 140 (x(1-x))^3

@@ -9,23 +9,40 @@
 //
 // Formats (unsigned fractions; Qk holds x 2^k).  Coordinates z are Q63.  The
 // coefficients of U and F are scaled by 2^k so that their sum stays below
-// 2^63; every product takes the high 64 bits, so a chain of products steps down
-// by one bit: U's terms Qk -> U in Q(k-1) < 2^62, F's quadratic terms Qk -> rows
-// Q(k-1) -> F in Q(k-2) < 2^61.  U and F are then normalised to [2^63, 2^64) by
+// 2^64; every product takes the high 64 bits, so a chain of products steps down
+// by one bit: U's terms Qk -> U in Q(k-1) < 2^63, F's quadratic terms Qk -> rows
+// Q(k-1) -> F in Q(k-2) < 2^62.  U and F are then normalised to [2^63, 2^64) by
 // their leading zeros, which keeps U^2 F and its reciprocal to ~2^-56 relative.
 // The value re-enters fixed point as V 2^t (t <= 30) and is summed exactly in
 // 128 bits.
 //
-// Precision.  U and F carry an absolute error of a few 2^-62 of their
-// coefficient sums, so the host admits polynomials whose constant term is at
-// least 1/1000 of that sum (kFxRange): the relative error then stays at or
-// below the double chains' 2^-53 per operation, and coordinates (63 bits
-// against 52) and sums (exact) are finer.  Products drop their fractions; the
-// mean of what U and F lose goes into their constant terms.
+// Precision.  With R the larger (coefficient sum) / (constant term) of U and F, a
+// unit of U is R 2^-63 of its smallest value and one of F R 2^-62.  What the dropped
+// products and the coordinates' truncations take away is 4 to 10 units with a spread
+// of 2 to 3; its mean at the corner z = 0, where U and F are smallest and such
+// integrands peak, goes into the constants (fixed64.cu), so that the spread
+// averages out in a sum and half a unit of rounding is left.  The Korobov weight is a product of
+// factors in Q64, whose steps count where the integrand peaks where the weight is
+// small: from R = kFxPeaked on it is carried normalised.  The host admits R up to
+// kFxRange.  Evaluated on the CPU against 80-bit floats (8 integrands of 400000
+// points each per d, transform and R), relative error of the estimate and of a
+// value (root mean square):
+//             d   R      here              double chain
+//   Korobov   1   64     1.3e-17 1.3e-16   2.2e-18 1.3e-15
+//             1   1000   1.5e-16 2.9e-15   6.9e-18 3.7e-15
+//             8   64     3.0e-17 2.7e-15   7.5e-18 5.0e-15
+//             8   1000   1.4e-18 4.2e-17   5.7e-18 5.3e-15
+//   baker     1   64     4.2e-18 3.5e-16   9.9e-17 5.7e-14
+//             1   1000   1.1e-16 2.2e-14   4.2e-15 3.6e-12
+// (the double chain's baker and untransformed coordinates are multiples of 2^-53 and
+// 2^-52; its sums' own rounding is not in the figures).  With the mean taken over the
+// whole cube, one bit less and the weight never normalised, R = 1000 left 1.5e-15 of
+// the estimate at d = 1 and 1e-15 (6e-13 of a value) at d = 8.
 //
 // Measured (GB300): d = 6, baker, n = 1000003, m = 32: 2.82 -> 0.55 ms; d = 8,
-// Korobov 3, n = 4194301, m = 16: 20.4 -> 2.96 ms; per-shift values within
-// 2e-16 of a 64-bit evaluation on both sides.
+// Korobov 3, n = 4194301, m = 16: 20.4 -> 3.02 ms (2.98 without the peaked
+// integrands' branch); per-shift values within 2e-16 of a 64-bit evaluation on both
+// sides.
 //
 // What bounds it now: issue slots, 78 multiply-adds of four and 295 others a value
 // at d = 6.  Tried: one row per CTA (d = 8: 4.47 ms), three CTAs per SM at 80
@@ -41,8 +58,9 @@
 
 namespace qmc {
 
-constexpr int kFxShiftMin = 7;        // 2 su + sf of the largest U < 2^62 and F < 2^61 (leading zeros 2 and 3)
+constexpr int kFxShiftMin = 4;        // 2 su + sf of the largest U < 2^63 and F < 2^62 (leading zeros 1 and 2)
 constexpr double kFxRange = 1000.0;   // largest (coefficient sum) / (constant term) of U and of F
+constexpr double kFxPeaked = 64.0;    // the same, above which the Korobov weight is normalised
 
 // a b + c, one multiply-add (spelled out: as a plain expression the compiler
 // splits sums of such products into products and adds)
@@ -147,7 +165,7 @@ __host__ __device__ __forceinline__ uint64_t fx_coord(uint64_t X, uint64_t& u) {
 }
 
 // sum_j c_j z_j / 2^64 for constants c_j = (high word, low word / 16) with
-// sum_j c_j < 2^63 and z_j < 2^63: with 28-bit low words the cross products of
+// sum_j c_j < 2^64 and z_j < 2^63: with 28-bit low words the cross products of
 // up to eight terms share one 64-bit sum, so a term is three multiply-adds and
 // nothing else.
 struct FxDot {
@@ -164,13 +182,17 @@ struct FxDot {
 // NS weighted values at one point: v[s] 2^t[s] in units of value_scale.  TERM
 // (single terms listed by the caller): the weight keeps its leading zeros
 // apart, factor by factor, so a term of any size comes back to full relative
-// precision; in the rule's sums the weight's 2^-64 absolute steps are below
-// the rounding of the sum's final conversion.
+// precision.  In the rule's sums it does so for peaked integrands, after each half
+// of the factors; for the others the weight's 2^-64 absolute steps are below the
+// rounding of the sum's final conversion.  t[s] is negative only where the weight
+// is normalised.
 template <int D, int TR, int NS, bool TERM = false>
 __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint64_t* base, const uint64_t (*shift)[D],
                                                    uint64_t* v, int* t) {
-  uint64_t z[NS][D], W[NS];
-  int ew = 0;
+  // two products of factors, so that four at most multiply unnormalised
+  constexpr int H = D > 4 ? D / 2 : D;
+  uint64_t z[NS][D], W[NS], W2[NS];
+  int ew[NS];
 #pragma unroll
   for (int i = 0; i < D; ++i)
 #pragma unroll
@@ -179,17 +201,38 @@ __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint
       z[s][i] = fx_coord<TR>(base[i] + shift[s][i], u);
       if constexpr (TR == TR_KOROBOV) {
         if constexpr (TERM) {
-          static_assert(NS == 1, "one term at a time");
           const int su = fx_clz64(u);
-          W[s] = i == 0 ? u << su : fx_mulhi_add(W[s], u << su, 0);
+          u <<= su;
+          W[s] = i == 0 ? u : fx_mulhi_add(W[s], u, 0);
           const int sw = fx_clz64(W[s]);
           W[s] <<= sw;
-          ew += su + sw;
-        } else {
+          ew[s] = (i == 0 ? 0 : ew[s]) + su + sw;
+        } else if (i < H) {
           W[s] = i == 0 ? u : fx_mulhi_add(W[s], u, 0);
+        } else {
+          W2[s] = i == H ? u : fx_mulhi_add(W2[s], u, 0);
         }
       }
     }
+  if constexpr (TR == TR_KOROBOV && !TERM) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) ew[s] = 0;
+    const auto normalise = [&](uint64_t* w) {
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        const int sw = fx_clz64(w[s]);
+        w[s] <<= sw;
+        ew[s] += sw;
+      }
+    };
+    if (P.peaked) {
+      normalise(W);
+      if constexpr (H < D) normalise(W2);
+    }
+    if constexpr (H < D)
+#pragma unroll
+      for (int s = 0; s < NS; ++s) W[s] = fx_mulhi_add(W[s], W2[s], 0);
+  }
   uint64_t U[NS], F[NS];
   FxDot dot[NS];
 #pragma unroll
@@ -203,18 +246,15 @@ __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint
     U[s] = dot[s].value();
     F[s] = P.f0;
   }
-  // F row by row; a bit per slot (the row's linear term first) tells which
-  // terms exist: a test and a branch (2 slots a pair of shifts) against 24
+  // F row by row; a bit per slot (the row itself first) tells which terms
+  // exist: a test and a branch (2 slots a pair of shifts) against 24
   int off = 0;
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     const uint32_t row = P.fmask[i];
     if (row) {
 #pragma unroll
-      for (int s = 0; s < NS; ++s) dot[s] = FxDot{0, 0};
-      if (row & 1u)
-#pragma unroll
-        for (int s = 0; s < NS; ++s) dot[s].hi = P.fl[i];
+      for (int s = 0; s < NS; ++s) dot[s] = FxDot{P.fl[i], 0};
 #pragma unroll
       for (int j = i; j < D; ++j)
         if (row & (2u << (j - i)))
@@ -232,7 +272,7 @@ __host__ __device__ __forceinline__ void fx_values(const FxParams& P, const uint
     // the reciprocal is below 2^59: 4 more bits before the weight (0.2% on average at d = 8) takes them away
     if constexpr (TR == TR_KOROBOV) r = fx_mulhi_add(r << 4, fx_mulhi_add(fx_sqr(W[s]), W[s], 0), 0, 0x140000000ull);
     v[s] = r;
-    t[s] = 2 * su + sf - kFxShiftMin - (TERM ? 3 * ew : 0);
+    t[s] = 2 * su + sf - kFxShiftMin - (TR == TR_KOROBOV ? 3 * ew[s] : 0);
   }
 }
 
@@ -322,7 +362,10 @@ __global__ void __launch_bounds__(kThreads)
       int t[NS];
       fx_values<D, TR, NS>(P, walk.base, sh, v, t);
 #pragma unroll
-      for (int q = 0; q < NS; ++q) acc[q].add(v[q] << t[q], __funnelshift_l((uint32_t)(v[q] >> 32), 0u, t[q]));
+      for (int q = 0; q < NS; ++q) {
+        if (TR == TR_KOROBOV && P.peaked && t[q] < 0) acc[q].add(t[q] > -64 ? v[q] >> -t[q] : 0, 0);
+        else acc[q].add(v[q] << t[q], __funnelshift_l((uint32_t)(v[q] >> 32), 0u, t[q]));
+      }
       walk.step(P);
     }
   }

@@ -169,8 +169,9 @@ struct FxParams : FxBase {
   uint64_t u0;                  // U: constant term in Q(k-1)
   uint32_t uh[kDFast], ul[kDFast];  // linear coefficients: high word; low word / 16
   uint64_t f0;                  // F: constant term in Q(k-2)
-  uint64_t fl[kDFast];          // rows: linear coefficient in Q(k-1)
-  uint32_t fmask[kDFast];       // rows: bit 0 linear term, bit 1 + j - i the term q_ij
+  uint64_t fl[kDFast];          // rows: linear coefficient (and the mean of what is dropped) in Q(k-1)
+  uint32_t fmask[kDFast];       // rows: bit 0 the row has terms, bit 1 + j - i the term q_ij
+  int32_t peaked;               // the Korobov weight is carried normalised
   uint32_t fh[kDFast * (kDFast + 1) / 2], fq[kDFast * (kDFast + 1) / 2];  // q_ij, row by row
 };
 

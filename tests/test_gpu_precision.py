@@ -36,3 +36,54 @@ def test_fp32_deformed_estimates(Q, seed):
                       aU=-2, aF=-1, lam=0.1)
     a, b = (complex(*estimate(Q, p, prec).mean) for prec in ("fp32", "fp64"))
     assert abs(a - b) <= 2e-9 * abs(b)
+
+
+def exact_points(p):
+    """Untransformed points [n, m, d] of the rule in extended precision."""
+    j = np.arange(p.n, dtype=np.uint64)[:, None]
+    idx = (j * p.g[None, :].astype(np.uint64)) % np.uint64(p.n)
+    x = idx.astype(np.longdouble)[:, None, :] / np.longdouble(p.n) + p.shifts.astype(np.longdouble)[None, :, :]
+    return np.where(x >= 1, x - 1, x)
+
+
+def exact_transform(x, transform):
+    """z and the weight of one point, in extended precision."""
+    if transform == "none":
+        return x, np.longdouble(1)
+    s = np.minimum(x, 1 - x)
+    if transform == "baker":
+        return 2 * s, np.longdouble(1)
+    low = s ** 4 * (35 + s * (-84 + s * (70 - 20 * s)))
+    u = s * (1 - s)
+    return np.where(x > 0.5, 1 - low, low), np.prod(140 * u * u * u, axis=-1)
+
+
+def exact_poly(P, z):
+    tot = np.zeros(z.shape[:-1], dtype=np.longdouble)
+    for c, e in zip(P.coef, P.expo):
+        term = np.full_like(tot, np.longdouble(c))
+        for i in np.nonzero(e)[0]:
+            term = term * z[..., i] ** int(e[i])
+        tot += term
+    return tot
+
+
+@pytest.mark.parametrize("transform", ["none", "baker", "korobov"])
+@pytest.mark.parametrize("linear", [0, 2])
+@pytest.mark.parametrize("d", [1, 2, 3, 5, 8])
+def test_fp64_peaked_sectors(Q, d, transform, linear):
+    """FP64 sectors whose constant term is 1/990 of the coefficients' sum R, against extended precision:
+    the integrand peaks at the cube's corner, where U and F are a thousandth of their
+    range and (Korobov) the weight is small.  What may be left: half a unit of U's and F's constants, 2 R
+    2^-64 + R 2^-63 together 2.2e-16, and four roundings of the sum, the scale and the mean, 4.4e-16."""
+    rng = I.SplitMix64(500 + 10 * d + linear)
+    U, F = I.random_poly(rng, d, d, 0), I.random_poly(rng, d, min(linear, d), d * (d + 1) // 2)
+    for P in (U, F):
+        P.coef[0] = P.coef[1:].sum() / 989.0
+    n, m = 65537, 4
+    p = I.Problem("peak", d, n, m, I.make_shifts(rng, m, d), transform, alpha=3 if transform == "korobov" else 0, U=U,
+                  F=F, g=I.random_generating_vector(rng, d, n))
+    z, w = exact_transform(exact_points(p), transform)
+    ref = (w / (exact_poly(U, z) ** 2 * exact_poly(F, z))).mean()
+    got = estimate(Q, p, "fp64").mean[0]
+    assert abs(got - ref) <= 6.6e-16 * abs(ref), float(got / ref - 1)
