@@ -509,9 +509,14 @@ int qmc_integrate_noalloc(int32_t d, uint64_t n, int32_t m, const uint64_t* g, c
                           void* stream);
 #endif
 
-/* Single terms of Eq. (2), evaluated by the same device code the rule uses:
- * for each sample s, the weighted value f(z(x)) prod_i w(x_i) at point
- * j[s] (0-based, the paper's j-1) and shift k[s].
+/* Single terms of Eq. (2): for each sample s, the weighted value
+ * f(z(x)) prod_i w(x_i) at point j[s] (0-based, the paper's j-1) and shift k[s],
+ * from the kernel of the rule's plan, with its lattice index, fraction, shift and
+ * dither.  Where the rule's sums carry a Korobov weight to an absolute step
+ * (FP64 in fixed point, FP32EVAL in the form centred on x = 1/2), a single
+ * term's weight, and in FP32EVAL its coordinate, are evaluated to full relative
+ * precision instead: next to the cube's faces a term is more accurate than
+ * what the sum adds.
  *   values  [count * 2] (re, im), host
  *   idx     optional [count * d] lattice indices (j g_i) mod n, host
  *   coord   optional [count * d] the coordinate x the kernel used, as double, host
@@ -622,7 +627,8 @@ int qmc_integrate_eps(int32_t d, uint64_t n, int32_t m, const uint64_t* g, const
 int qmc_eps_plan_create(int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
                         qmc_transform t, const qmc_integrand* f, const qmc_eps* eps, qmc_plan* plan_out);
 /* Single terms: values [count][orders] (host), order o of the weighted value
- * at point j[s], shift k[s], by the device code of qmc_integrate_eps.
+ * at point j[s], shift k[s], from the kernel of qmc_integrate_eps (weights as for
+ * qmc_sample_points).
  * Synchronises `stream`. */
 int qmc_sample_points_eps(int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
                           qmc_transform t, const qmc_integrand* f, const qmc_eps* eps, int32_t count,

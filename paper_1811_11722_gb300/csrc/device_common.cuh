@@ -288,7 +288,11 @@ __device__ __forceinline__ uint32_t dither32(uint64_t j, int i) {
 // 2^-25 where the other form's is relative to z, which matters when U or F
 // comes near zero at the cube's corner: korobov_form() keeps such integrands
 // on the other form.  w then collects 4x(1-x), and 140/64 per dimension is
-// left to the final pass.
+// left to the final pass.  T's rounding (2^-26 in x near the faces) also costs the
+// factor its relative accuracy there: the weight of one dimension is off by up to
+// 5e-6 at x = 1e-2, 5e-4 at 1e-4 and 5e-2 at 1e-6 (plain form: 3e-7).  Such weights
+// are below 1e-4, 1e-10 and 1e-16 of the largest, so sums do not see it; single
+// listed terms take the plain form (sector_sample).
 template <int ALPHA>
 __host__ __device__ constexpr uint32_t fx_bias() {
   return ALPHA == kKorCentred ? 0x80000000u : 0u;

@@ -284,6 +284,17 @@ struct FxWalk {
   }
 };
 
+// Single terms of a plan in the centred Korobov form take the plain form: next to
+// the cube's faces the centred one loses the weight's relative accuracy (coord_fx),
+// which a sum does not see and a listed term does.  The plain form's weight lacks
+// 64 per dimension.
+template <int ALPHA>
+constexpr int kTermAlpha = ALPHA == kKorCentred ? 3 : ALPHA;
+template <int D, int ALPHA>
+__host__ __device__ constexpr double term_scale() {
+  return ALPHA == kKorCentred ? (double)(1ull << (6 * D)) : 1.0;
+}
+
 template <typename R, int D, int TR, int ALPHA, int KU, int KF, class POLY>
 __device__ void sector_sample(const RuleParams<R>& P, const SampleIO& sio) {
   using BT = typename SecBase<R>::T;
@@ -295,12 +306,12 @@ __device__ void sector_sample(const RuleParams<R>& P, const SampleIO& sio) {
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     uint32_t idx = lattice_index(j, P.g[i], P.n);
-    base[i] = sec_base<R, ALPHA>(idx, P.rc, j, i);
+    base[i] = sec_base<R, kTermAlpha<ALPHA>>(idx, P.rc, j, i);
     if (sio.idx) sio.idx[(size_t)s * D + i] = idx;
-    if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<R, ALPHA>(P, base[i], k, i);
+    if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<R, kTermAlpha<ALPHA>>(P, base[i], k, i);
   }
-  R v = sector_value<R, D, TR, ALPHA, KU, KF, POLY>(P, base, k);
-  sio.values[2 * (size_t)s] = (double)v * (double)P.value_scale;
+  R v = sector_value<R, D, TR, kTermAlpha<ALPHA>, KU, KF, POLY>(P, base, k);
+  sio.values[2 * (size_t)s] = (double)v * ((double)P.value_scale * term_scale<D, ALPHA>());
   sio.values[2 * (size_t)s + 1] = 0.0;
 }
 
@@ -854,10 +865,10 @@ __device__ __forceinline__ void eps_body2(const RuleParams<float>& P, double* __
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       uint32_t idx = lattice_index(j, P.g[i], P.n);
-      base[i] = sec_base<float, ALPHA>(idx, P.rc, j, i);
+      base[i] = sec_base<float, kTermAlpha<ALPHA>>(idx, P.rc, j, i);
       if (sio.idx) sio.idx[(size_t)s * D + i] = idx;
-      if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<float, ALPHA>(P, base[i], k, i);
-      z[i] = coord_fx<TR, ALPHA>(base[i] + P.shiftx[k][i], P.kor, w);
+      if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<float, kTermAlpha<ALPHA>>(P, base[i], k, i);
+      z[i] = coord_fx<TR, kTermAlpha<ALPHA>>(base[i] + P.shiftx[k][i], P.kor, w);
     }
     float U, F;
     POLY::template eval<D, 1, 2, float>(P, z, U, F);
@@ -865,7 +876,7 @@ __device__ __forceinline__ void eps_body2(const RuleParams<float>& P, double* __
     if constexpr (TR == TR_KOROBOV) v *= korobov_weight_fx(w);
     const float L = P.eps_b[0] * log_(U) + P.eps_b[1] * log_(F);
     for (int o = 0; o < P.eps_orders; ++o) {
-      sio.values[(size_t)s * sio.stride + o] = (double)v * P.value_scale;
+      sio.values[(size_t)s * sio.stride + o] = (double)v * (P.value_scale * term_scale<D, ALPHA>());
       v = v * L * P.eps_inv[o];
     }
     return;

@@ -87,3 +87,33 @@ def test_fp64_peaked_sectors(Q, d, transform, linear):
     ref = (w / (exact_poly(U, z) ** 2 * exact_poly(F, z))).mean()
     got = estimate(Q, p, "fp64").mean[0]
     assert abs(got - ref) <= 6.6e-16 * abs(ref), float(got / ref - 1)
+
+
+@pytest.mark.parametrize("d", [1, 3, 6, 8])
+@pytest.mark.parametrize("jit", ["1", "0"])
+def test_fp32_single_terms_next_to_faces(Q, monkeypatch, d, jit):
+    """Listed FP32 terms with one coordinate 0.1 to 1e-6 from a face (point 0, which has no dither, under shifts that
+    lie there; two such coordinates' weights would leave float's range): relative to the same value at the
+    coordinate used, at most 3 (2 d + 2) roundings of 2^-24 in the weight's cube and 3 (2 d + 12) in U^-2 F^-1,
+    whatever the weight's size."""
+    monkeypatch.setenv("QMC_JIT", jit)
+    rng = I.SplitMix64(900 + d)
+    m, n = 64, 10007
+    U, F = I.random_poly(rng, d, d, 0), I.random_poly(rng, d, 0, d * (d + 1) // 2)
+    U.coef[0] = F.coef[0] = 2.0
+    shifts = np.array([[rng.uniform_in(0.2, 0.8) for _ in range(d)] for _ in range(m)])
+    for k in range(m):
+        near = 10.0 ** -rng.uniform_in(1, 6)
+        shifts[k, k // 2 % d] = 1.0 - near if k % 2 else near
+    p = I.Problem("faces", d, n, m, shifts, "korobov", alpha=3, U=U, F=F, g=I.random_generating_vector(rng, d, n))
+    f, t = Q.integrand_from_problem(p, "fp32"), Q.transform("korobov", 3)
+    j, k = np.zeros(m, dtype=np.uint64), np.arange(m, dtype=np.int32)
+    v, _, x = Q.qmc_sample_points(d, n, m, p.g, shifts, t, f, j, k)
+    assert np.all(np.abs(x - shifts) <= 2.0 ** -33)  # rounded to 32 bits
+    z, w = exact_transform(x.astype(np.longdouble), "korobov")
+    uu, ff = exact_poly(U, z), exact_poly(F, z)
+    ref = w / (uu * uu * ff)
+    tol = (3 * (2 * d + 2) + 3 * (2 * d + 12)) * 2.0 ** -24
+    assert np.all(np.abs(v[:, 0] - ref) <= tol * ref), float(np.max(np.abs(v[:, 0] / ref - 1)))
+    e = Q.qmc_sample_points_eps(d, n, m, p.g, shifts, t, f, Q.eps_spec(3), j, k)
+    assert np.all(np.abs(e[:, 0] - ref) <= tol * ref), float(np.max(np.abs(e[:, 0] / ref - 1)))
