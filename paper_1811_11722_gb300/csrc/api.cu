@@ -548,13 +548,18 @@ static int build_rule_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
     return fail(QMC_EUNSUPPORTED, "deformed sector integrands are served by the complex kernels");
   } else {
     int fk = f->kind == QMC_F_CONST ? FK_CONST : (f->kind == QMC_F_SEPARABLE_EXP ? FK_SEPEXP : FK_TRIG);
-    func = separable_ptr(fp32, base.tr, base.alpha, fk);
+    // FP64 coordinates in fixed point: none, baker, and Korobov 3 unless a coefficient
+    // makes their last bits count
+    bool fixed = !fp32 && (base.tr != TR_KOROBOV || base.alpha == 3);
+    if (fixed && base.tr == TR_KOROBOV && fk == FK_SEPEXP)
+      for (int i = 0; i < d; ++i) fixed = fixed && std::fabs(f->c[i]) + std::fabs(f->b[i]) <= kSepFixedMax;
+    func = separable_ptr(fp32, base.tr, fixed, fk);
     if (fp32) {
       mc = 8;
     } else {  // one shift row per CTA row, up to kMcMax rows a launch
       mc = kMcMax;
       pl->grid_rows = std::min(m, kMcMax);
-      if (base.tr != TR_KOROBOV || base.alpha == 3) {  // fixed-point coordinates 2^63 z
+      if (fixed) {  // coordinates come as 2^63 z
         for (int i = 0; i < d; ++i) {
           base.sep_c[i] = std::ldexp((double)base.sep_c[i], -63);
           base.sep_b[i] = std::ldexp((double)base.sep_b[i], -63);

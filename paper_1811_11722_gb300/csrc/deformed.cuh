@@ -315,7 +315,7 @@ __device__ __forceinline__ Cx<R> det_ipm_minus1(R (&M)[D][D]) {
 template <bool TERM>
 __device__ __forceinline__ double def_coord64(uint64_t X, int i, double& wt, uint64_t& wf) {
   uint64_t u;
-  const uint64_t z = fx_coord<TR_KOROBOV>(X, u);
+  const uint64_t z = fx_coord_centred(X, u);
   if constexpr (TERM) wt *= __ull2double_rn(u) * (i == 0 ? 1.0 : 0x1p-64);
   else wf = i == 0 ? u : fx_mulhi_add(wf, u, 0);
   const long long bits = __double_as_longlong(__ull2double_rn(z));

@@ -164,6 +164,14 @@ __host__ __device__ __forceinline__ uint64_t fx_coord(uint64_t X, uint64_t& u) {
   }
 }
 
+// The Korobov coordinate for users that convert it to double: fx_coord's truncations
+// leave z 6.5 units too large on average near 0, where a unit counts most (7.5 too
+// small near 1).  The sectors take that off their constants.
+__host__ __device__ __forceinline__ uint64_t fx_coord_centred(uint64_t X, uint64_t& u) {
+  const uint64_t z = fx_coord<TR_KOROBOV>(X, u);
+  return z > 6 ? z - 6 : 0;
+}
+
 // sum_j c_j z_j / 2^64 for constants c_j = (high word, low word / 16) with
 // sum_j c_j < 2^64 and z_j < 2^63: with 28-bit low words the cross products of
 // up to eight terms share one 64-bit sum, so a term is three multiply-adds and

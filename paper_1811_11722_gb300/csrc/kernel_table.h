@@ -65,13 +65,16 @@ QMC_DECL_DEF(double, 5) QMC_DECL_DEF(double, 6) QMC_DECL_DEF(double, 7) QMC_DECL
 #undef QMC_DECL_DEF
 
 // Separable integrands (const / separable exp / trig), runtime d and Korobov
-// weight alpha.
+// weight; fixed: the FP64 kernel with coordinates in fixed point (Korobov 3).
+// Above kSepFixedMax (of |c_i| + |b_i|) a unit of the coordinate, 2^-63, is no longer below the
+// rounding of 1 + c z and of the exponent.
+constexpr double kSepFixedMax = 1024.0;
 template <typename R>
-const void* separable_ptr_t(int tr, int alpha, int fk);
-template <> const void* separable_ptr_t<float>(int tr, int alpha, int fk);
-template <> const void* separable_ptr_t<double>(int tr, int alpha, int fk);
-inline const void* separable_ptr(bool fp32, int tr, int alpha, int fk) {
-  return fp32 ? separable_ptr_t<float>(tr, alpha, fk) : separable_ptr_t<double>(tr, alpha, fk);
+const void* separable_ptr_t(int tr, bool fixed, int fk);
+template <> const void* separable_ptr_t<float>(int tr, bool fixed, int fk);
+template <> const void* separable_ptr_t<double>(int tr, bool fixed, int fk);
+inline const void* separable_ptr(bool fp32, int tr, bool fixed, int fk) {
+  return fp32 ? separable_ptr_t<float>(tr, fixed, fk) : separable_ptr_t<double>(tr, fixed, fk);
 }
 
 // General sparse-polynomial sector kernel, runtime d, transform and powers.

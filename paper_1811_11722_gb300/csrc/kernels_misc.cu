@@ -19,11 +19,11 @@ namespace qmc {
 
 // FP64: one shift row per CTA row (separable64.cuh); FP32: 8 shifts per thread.
 template <>
-const void* separable_ptr_t<QMC_REAL>(int tr, int alpha, int fk) {
+const void* separable_ptr_t<QMC_REAL>(int tr, bool fixed, int fk) {
   if constexpr (sizeof(QMC_REAL) == 8) {
     if (tr == TR_NONE) QMC_SEP_FK(separable64_kernel, TR_NONE, false);
     if (tr == TR_BAKER) QMC_SEP_FK(separable64_kernel, TR_BAKER, false);
-    if (tr == TR_KOROBOV && alpha == 3) QMC_SEP_FK(separable64_kernel, TR_KOROBOV, true);
+    if (tr == TR_KOROBOV && fixed) QMC_SEP_FK(separable64_kernel, TR_KOROBOV, true);
     if (tr == TR_KOROBOV) QMC_SEP_FK(separable64_kernel, TR_KOROBOV, false);
   } else {
     if (tr == TR_NONE) QMC_SEP_FK(separable_kernel, QMC_REAL, 8, TR_NONE);

@@ -6,7 +6,9 @@
 // therefore come from 64-bit fixed point (fx_coord), which leaves per dimension one
 // conversion and the integrand's own three operations: d = 3 takes about 35
 // FP64 operations a value with the exponential, against 75 with the transform in
-// double.  Weights other than 3 keep the double transform.
+// double.  Weights other than 3 keep the double transform, and so do exponents and
+// factors above kSepFixedMax: near 0 the double transform's coordinate is accurate
+// relative to itself, the fixed-point one to about 2 units of 2^-63.
 //
 // Layout.  One shift row per CTA row, a thread's points kThreads apart: a
 // value is worth some 600 clocks of the pipe to a warp, so sharing a point between
@@ -19,13 +21,14 @@
 
 namespace qmc {
 
-template <int TR, bool KOR3, int FK>
+template <int TR, bool KOR3, int FK>  // KOR3: weight 3 in fixed point
 struct Sep64 {
   // TERM: a single listed term, its weight to full relative precision
   template <bool TERM, class BASE>
   static __device__ __forceinline__ double value(const RuleParams<double>& P, int k, BASE base) {
     double w = 1.0, prod = 1.0, lin = 0.0;
     uint64_t wf = ~0ull;
+    int ew = 0;
 #pragma unroll 1
     for (int i = 0; i < P.d; ++i) {
       const uint64_t X = base(i) + P.shift64[k][i];
@@ -33,11 +36,19 @@ struct Sep64 {
       if constexpr (TR == TR_KOROBOV && !KOR3) {
         z = coord_f64<TR, 0>(X, P.kor, P.alpha, w);
       } else {
-        uint64_t u = 0;
-        const uint64_t zf = fx_coord<TR>(X, u);
+        uint64_t u = 0, zf;
         if constexpr (TR == TR_KOROBOV) {
-          if constexpr (TERM) w *= __ull2double_rn(u) * 0x1p-64;
-          else wf = i == 0 ? u : fx_mulhi_add(wf, u, 0);
+          zf = fx_coord_centred(X, u);
+          if constexpr (TERM) {
+            w *= __ull2double_rn(u) * 0x1p-64;
+          } else {  // normalised: of 16 factors only 2^-14 may be left, less where the integrand peaks
+            wf = i == 0 ? u : fx_mulhi_add(wf, u, 0);
+            const int s = fx_clz64(wf);
+            wf <<= s;
+            ew += s;
+          }
+        } else {
+          zf = fx_coord<TR>(X, u);
         }
         if constexpr (FK != FK_CONST) z = __ull2double_rn(zf);
       }
@@ -55,6 +66,7 @@ struct Sep64 {
       if constexpr (KOR3) {
         if constexpr (!TERM) w = __ull2double_rn(wf) * 0x1p-64;
         w = w * w * w;
+        if constexpr (!TERM) w *= 3 * ew < 1000 ? __longlong_as_double((long long)(1023 - 3 * ew) << 52) : 0.0;
       }
       v *= w;
     }

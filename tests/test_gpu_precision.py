@@ -117,3 +117,93 @@ def test_fp32_single_terms_next_to_faces(Q, monkeypatch, d, jit):
     assert np.all(np.abs(v[:, 0] - ref) <= tol * ref), float(np.max(np.abs(v[:, 0] / ref - 1)))
     e = Q.qmc_sample_points_eps(d, n, m, p.g, shifts, t, f, Q.eps_spec(3), j, k)
     assert np.all(np.abs(e[:, 0] - ref) <= tol * ref), float(np.max(np.abs(e[:, 0] / ref - 1)))
+
+
+def exact_deformed(p):
+    """Weighted values of the contour-deformed integrand at every point and shift, in extended precision."""
+    y, w = exact_transform(exact_points(p), p.transform)
+    d, lam = p.d, np.longdouble(p.lam)
+    H = np.zeros((d, d))
+    lin = np.zeros(d)
+    for c, e in zip(p.F.coef, p.F.expo):
+        v = [i for i in range(d) for _ in range(int(e[i]))]
+        if len(v) == 1:
+            lin[v[0]] += c
+        elif len(v) == 2:
+            H[v[0], v[1]] += c
+            H[v[1], v[0]] += c
+    grad = [lin[k] + sum(np.longdouble(H[k, l]) * y[..., l] for l in range(d)) for k in range(d)]
+    a = [y[..., k] * (1 - y[..., k]) for k in range(d)]
+    z = np.stack([y[..., k] - 1j * (lam * a[k] * grad[k]) for k in range(d)], axis=-1)
+    J = [[(1 if k == l else 0) - 1j * (lam * (H[k, l] * a[k] + ((1 - 2 * y[..., k]) * grad[k] if k == l else 0)))
+          for l in range(d)] for k in range(d)]
+    det = np.ones(z.shape[:-1], dtype=z.dtype)
+    for c in range(d):  # diagonally dominant: no pivoting
+        det = det * J[c][c]
+        for r in range(c + 1, d):
+            f = J[r][c] / J[c][c]
+            for q in range(c + 1, d):
+                J[r][q] = J[r][q] - f * J[c][q]
+
+    def poly(P):
+        tot = np.zeros(z.shape[:-1], dtype=z.dtype)
+        for c, e in zip(P.coef, P.expo):
+            term = np.full_like(tot, np.longdouble(c))
+            for i in np.nonzero(e)[0]:
+                term = term * z[..., i] ** int(e[i])
+            tot = tot + term
+        return tot
+    return w * det / (poly(p.U) ** 2 * poly(p.F))
+
+
+def deformed_problem(d, ratio, lam, linear, n=20011, m=4):
+    rng = I.SplitMix64(1000 * d + ratio + int(100 * lam) + 7 * linear)
+    U = I.random_poly(rng, d, d, 0)
+    F = I.random_poly(rng, d, d if linear else 0, d * (d + 1) // 2, neg_quad=min(1, d - 1))
+    for P in (U, F):
+        P.coef[0] = np.abs(P.coef[1:]).sum() / (ratio - 1)
+    return I.Problem("def", d, n, m, I.make_shifts(rng, m, d), "korobov", alpha=3, kind="sector_deformed", U=U, F=F,
+                     aU=-2, aF=-1, lam=lam, g=I.random_generating_vector(rng, d, n))
+
+
+@pytest.mark.parametrize("d,ratio,lam,linear", [(1, 950, 0.02, 1), (1, 950, 0.4, 1), (2, 950, 0.1, 1), (2, 950, 0.4, 0),
+                                                (7, 4, 0.4, 0), (7, 950, 0.1, 1)])
+def test_fp64_deformed_in_double(Q, d, ratio, lam, linear):
+    """FP64 deformed integrands outside of the fixed-point form's range (coordinates in fixed point, the rest in double)
+    against extended precision: six roundings of 2^-53 for the sum, the scale, the mean and the constants."""
+    p = deformed_problem(d, ratio, lam, linear)
+    ref = exact_deformed(p).mean()
+    got = complex(*estimate(Q, p, "fp64").mean)
+    assert abs(got - ref) <= 6.7e-16 * abs(ref), float(abs(got - ref) / abs(ref))
+
+
+@pytest.mark.parametrize("d,b", [(1, -20.0), (1, -1e3), (1, -1e6), (1, -1e8), (2, -1e3), (3, -100.0)])
+def test_fp64_separable_peaks(Q, d, b):
+    """FP64 separable exponentials that peak at z = 0, against extended precision: six roundings of 2^-53 for the sum, the
+    scale, the mean and the factors (those of the exponents, which are small where the values are large, average out)."""
+    rng = I.SplitMix64(5000 + d)
+    n, m = 20011, 4
+    p = I.Problem("peak", d, n, m, I.make_shifts(rng, m, d), "korobov", alpha=3, kind="separable_exp",
+                  b=b * np.array([rng.uniform_in(0.5, 1) for _ in range(d)]), c=np.zeros(d),
+                  g=I.random_generating_vector(rng, d, n))
+    z, w = exact_transform(exact_points(p), "korobov")
+    ref = (w * np.exp((p.b.astype(np.longdouble) * z).sum(axis=-1))).mean()
+    got = estimate(Q, p, "fp64").mean[0]
+    assert abs(got - ref) <= 6.7e-16 * abs(ref), float(got / ref - 1)
+
+
+@pytest.mark.parametrize("kind", ["const", "separable_exp", "trig"])
+@pytest.mark.parametrize("near", [1e-2, 1e-3, 1e-4])
+def test_fp64_separable_small_weights(Q, kind, near):
+    """A rule of three points each of which has five of its fifteen coordinates next to a face: the weights, down to
+    1e-49 of the largest, keep their relative precision: three roundings for each of 15 factors and fifteen for
+    the sum, 6.7e-15 (a factor's own error, a unit of 2^-64 in 4e-4, is below them)."""
+    d, n, m = 15, 3, 2
+    shifts = np.array([[(i % 3) / 3 + near * (1 + 0.1 * i) for i in range(d)], [(i % 3) / 3 + near * (2 - 0.05 * i) for i in range(d)]])
+    p = I.Problem("small", d, n, m, shifts, "korobov", alpha=3, kind=kind, c=np.zeros(d), b=np.zeros(d),
+                  h=np.zeros(d, dtype=np.int32), g=np.ones(d, dtype=np.uint64))
+    _, w = exact_transform(exact_points(p), "korobov")
+    _, ps = Q.qmc_integrate(d, n, m, p.g, shifts, Q.transform("korobov", 3), Q.integrand_from_problem(p, "fp64"),
+                            want_per_shift=True)
+    ref = w.mean(axis=0)
+    assert np.all(np.abs(ps[:, 0] - ref) <= 6.7e-15 * ref), (ps[:, 0], ref)
