@@ -8,24 +8,27 @@
 // F^-1 det J, whose size is not bounded, is formed in double: about 40 FP64
 // operations, which run beside the integer ones.
 //
-// Measured (GB300, d = 5, n = 262139, m = 20): 2.26 -> 0.67 ms; d = 2..4 0.48 to
-// 0.51 ms, d = 6 1.12 ms (double kernels with LU 1.5 to 3.6 and 6.4 ms).  What
-// bounds it now: issue slots at d = 5 (568 multiply-adds of four and 1750 others a
-// value, 78 % of the slots), the FP64 pipe below.  Two CTAs per SM at 128 registers
-// with 70 spilled bytes (d = 5): 0.67 ms, one CTA at 156 registers: 1.03 ms.
+// Measured (GB300, d = 5, n = 262139, m = 20): 2.26 -> 0.70 ms (0.68 with limbs and
+// sums truncated instead of rounded); in that form d = 2..4 took 0.48 to 0.51 ms, d = 6
+// 1.12 ms (double kernels with LU 1.5 to 3.6 and 6.4 ms).  What bounds it: issue
+// slots at d = 5 (568 multiply-adds of four and 1750 others a value, 78 % of the slots),
+// the FP64 pipe below.  Two CTAs per SM at 128 registers with 36 spilled bytes (d = 5);
+// one CTA at 156 registers took 1.5 times as long.
 //
 // Numbers.  An int64 X stands for X 2^-q, |X| < 2^62, and is multiplied by its limbs
 // h = X >> 31 and l = (X >> 3) mod 2^28:
 //   X Y / 2^62 = h h' + (h l' + l h') / 2^28,
 // the cross products short enough (2^59) that the sums of a dot product share one
-// 64-bit accumulator.  The last three bits and l l' are dropped, 2^-58 of the full
-// range at most.  Scales per plan, from bounds over the cube (fixed64.cu): cg for
+// 64-bit accumulator.  The last three bits (rounded) and l l' (its mean put back) are
+// dropped, 2^-58 of the full range at most.  Scales per plan, from bounds over the cube (fixed64.cu): cg for
 // g' = -lambda dF, v = y (1 - y) g', m = y (1 - y) H'_kk + (1 - 2y) g' and the
 // quadratic forms, x for the recursion's nodes.  A product with a Q(cg) number comes
 // out 62 - cg = sh bits low; the sum is shifted back before its low part is added.
-// Error of a value against 80-bit floats, d = 1..6, 48 integrands: median 1.6e-16
-// to 4e-16 (double coordinates and LU: 3e-16 to 1.6e-15), largest 1e-13 (2e-10,
-// from weights next to the cube's faces).
+// Error against 80-bit floats, d = 1..6, lambda 0.02 to 0.4, constants down to 1/250
+// of the coefficients' sum: a value (root mean square over the cube) 3e-16 to 3e-15,
+// an estimate 1e-17 to 1.2e-16.  With truncated limbs and sums and one bit less an
+// estimate was up to 2.4e-15 off, the determinant's truncations being multiplied up
+// its recursion.
 #pragma once
 
 #include "deformed.cuh"
@@ -42,9 +45,17 @@ __device__ __forceinline__ FxLimb fx_limb(int64_t X) {
   return {(int32_t)(X >> 31), (int32_t)(((uint32_t)X >> 3) & 0x0FFFFFFFu)};
 }
 
-// a sum of products
+// A sum of n products, shifted left by sh at the end: the cross sum starts with half
+// a unit, half = 2^(27 - sh), and with what the n products of low limbs amount to on
+// average (2^54 each), so that nothing is lost on average.
+// Results that are taken apart into limbs carry four units more, which rounds the
+// limbs' three dropped bits: from their sum's start (r, or four = 4 2^(28 - sh) in the
+// cross sum), and in the determinant's recursion from its leaves on (x' = x + 4
+// keeps through x - re and x + im), until the root takes them off.
 struct FxProd {
-  int64_t r = 0, c = 0;
+  int64_t r, c;
+  __device__ __forceinline__ explicit FxProd(int n, int32_t start = 1 << 27, int64_t r0 = 0)
+      : r(r0), c(start + (n << 26)) {}
   __device__ __forceinline__ void add(const FxLimb& a, const FxLimb& b) {
     r = fx_mads(a.h, b.h, r);
     c = fx_mads(a.h, b.l, c);
@@ -63,16 +74,17 @@ struct FxCx {
 template <int D, int J, int S>
 __device__ __forceinline__ FxCx defx_node(const DefFxParams& P, const FxLimb* ml, const FxLimb* al) {
   if constexpr (J == D - 1) {
-    FxProd p;
+    FxProd p((S & (S - 1)) != 0 ? 2 : 1, P.half + P.four);
     if constexpr ((S & (S - 1)) != 0) p.add(ml[J], P.hl[S]);
     p.add(al[J], P.hl[S | (1 << J)]);
     return {(S & (S - 1)) != 0 ? P.hs[S] : 0, p.value(P.sh)};
   } else {
     const FxCx x = defx_node<D, J + 1, S>(P, ml, al), y = defx_node<D, J + 1, S | (1 << J)>(P, ml, al);
-    FxProd re, im;
+    constexpr bool kRe = J < D - 2 || (S & (S - 1)) != 0;  // else x.re = 0
+    FxProd re(2, kRe ? P.half : P.half - P.four), im(kRe ? 2 : 1, P.half);
     re.add(ml[J], fx_limb(x.im));
     re.add(al[J], fx_limb(y.im));
-    if constexpr (J < D - 2 || (S & (S - 1)) != 0) im.add(ml[J], fx_limb(x.re));  // else x.re = 0
+    if constexpr (kRe) im.add(ml[J], fx_limb(x.re));
     im.add(al[J], fx_limb(y.re));
     return {x.re - re.value(P.sh), x.im + im.value(P.sh)};
   }
@@ -81,15 +93,15 @@ __device__ __forceinline__ FxCx defx_node(const DefFxParams& P, const FxLimb* ml
 template <int D, int J>
 __device__ __forceinline__ FxCx defx_root(const DefFxParams& P, const int64_t* m, const FxLimb* ml, const FxLimb* al) {
   if constexpr (J == D - 1) {
-    return {0, m[J] >> P.mx};
+    return {0, ((m[J] + P.mround) >> P.mx) + 4};
   } else {
     const FxCx x = defx_root<D, J + 1>(P, m, ml, al), y = defx_node<D, J + 1, 1 << J>(P, ml, al);
-    FxProd re, im;
+    FxProd re(2, J < D - 2 ? P.half : P.half - P.four), im(J < D - 2 ? 2 : 1, P.half);
     re.add(ml[J], fx_limb(x.im));
     re.add(al[J], fx_limb(y.im));
     if constexpr (J < D - 2) im.add(ml[J], fx_limb(x.re));
     im.add(al[J], fx_limb(y.re));
-    return {x.re - re.value(P.sh), (m[J] >> P.mx) + x.im + im.value(P.sh)};
+    return {x.re - re.value(P.sh), ((m[J] + P.mround) >> P.mx) + x.im + im.value(P.sh)};
   }
 }
 
@@ -113,30 +125,30 @@ __device__ __forceinline__ Cx<double> deformed_fx_value(const DefFxParams& P, co
   wt = wt * wt * wt;
   int64_t m[D];
   FxLimb ml[D], al[D], vl[D];
-  FxProd ur, ui, yl, yg, vg, vr;
+  FxProd ur(D), ui(D, P.half), yl(D), yg(D), vg(D, P.half), vr(D, P.half);
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    FxProd p;
+    FxProd p(D);
 #pragma unroll
     for (int l = 0; l < D; ++l) p.add(H(k, l), y[l]);
     const int64_t gk = P.gl[k] + p.value();
     const FxLimb g = fx_limb(gk);
-    FxProd q;
+    FxProd q(1, 1 << 27, 4);
     q.add(y[k], FxLimb{0x7FFFFFFF - y[k].h, 0x0FFFFFFF - y[k].l});
     const int64_t a = q.value();  // y (1 - y), Q62
     const FxLimb af = fx_limb(a);
-    FxProd v;
+    FxProd v(1, 1 << 27, 4);
     v.add(af, g);
     vl[k] = fx_limb(v.value());
     // 1 - 2y in Q62 from y's limbs: (2^31 - 1 - 2h, 2^28 - 1 - 2l) with l's carry
     const int32_t wl = 0x0FFFFFFF - 2 * y[k].l;
     const FxLimb w = {(int32_t)(0x7FFFFFFFu - 2u * (uint32_t)y[k].h + (uint32_t)(wl >> 28)), wl & 0x0FFFFFFF};
-    FxProd d;
+    FxProd d(2, 1 << 27, 4);
     d.add(af, H(k, k));
     d.add(w, g);
     m[k] = d.value();
     ml[k] = fx_limb(m[k]);
-    al[k] = fx_limb(a >> P.sh);
+    al[k] = fx_limb((a + P.around) >> P.sh);
     ur.add(P.u[k], y[k]);
     ui.add(P.u[k], vl[k]);
     yg.add(y[k], g);
@@ -145,7 +157,7 @@ __device__ __forceinline__ Cx<double> deformed_fx_value(const DefFxParams& P, co
   }
 #pragma unroll
   for (int k = 0; k < D; ++k) {
-    FxProd r;
+    FxProd r(D - k, P.half + P.four);
     r.add(P.Q[k], vl[k]);
 #pragma unroll
     for (int l = k + 1; l < D; ++l) r.add(H(k, l), vl[l]);
@@ -159,7 +171,7 @@ __device__ __forceinline__ Cx<double> deformed_fx_value(const DefFxParams& P, co
   fr = fma_(dbl(vr.value(P.sh)), P.c3, fr);
   const int64_t fi = vg.value(P.sh);  // v.g' = sum y (1 - y) g'^2 >= 0
   const Cx<double> F{fr, dbl(fi > 0 ? fi : 0) * -P.c3};
-  const Cx<double> dm1{dbl(del.re) * P.sd, dbl(del.im) * P.sd};
+  const Cx<double> dm1{dbl(del.re - (D > 1 ? 4 : 0)) * P.sd, dbl(del.im - 4) * P.sd};
   const Cx<double> rv = crecip(cmul(cmul(U, U), F));
   const Cx<double> t = cmul(dm1, rv);
   return {(rv.re + t.re) * wt, (rv.im + t.im) * wt};

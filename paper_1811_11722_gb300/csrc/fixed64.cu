@@ -188,7 +188,9 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
   return QMC_OK;
 }
 
+constexpr double kDefFxRange = 250.0;      // largest (coefficient sum) / (constant term): 2e-16 of the estimate
 constexpr double kDefFxMin = 1.0 / 32.0;  // smallest sum of |lambda dF| over the cube
+constexpr int kDefFxNode = 55;            // smallest scale of the determinant's nodes: 1.4e-16 of the estimate, at 54 4e-16
 
 // The deformed FAST integrand in fixed point (deformed_fx.cuh) from DefTab's
 // constants t (F(0), dF(0), Hessian, half diagonal, minors) and U's cu.
@@ -240,15 +242,16 @@ int build_deformed_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
     }
   // near the origin F and U are their constants, against which the sums' absolute
   // errors count; y.g' gives F in units of lambda
-  if (!(std::fabs(t[0]) * kFxRange >= lsum + gsum / lambda) || !(std::fabs(cu[0]) * kFxRange >= usum) ||
+  if (!(std::fabs(t[0]) * kDefFxRange >= lsum + gsum / lambda) || !(std::fabs(cu[0]) * kDefFxRange >= usum) ||
       !(gsum >= kDefFxMin))
     return QMC_EUNSUPPORTED;
-  // the largest scale that keeps `most` below 2^bits
+  // the largest scale that keeps `most` below 2^bits: g' (and with it m, at most 5/4 of
+  // it) and the determinant's nodes (the root carries det J - 1) below 2^62
   const auto scale = [](double most, double bits) { return (int)std::floor(bits - std::log2(std::max(most, 1e-300))); };
-  const int cg = std::min({62, scale(gmax, 60.5), scale(gsum, 61.5)});
-  const int x = std::min(cg, scale(top, 60.5));
-  const int cl = std::min(62, scale(lsum, 60.5)), cuq = std::min(62, scale(usum, 60.5));
-  if (gmax > 4.0 || 62 - cg > 8 || x < 54 || cg - x > 8 || cl < 40 || cuq < 40 || !std::isfinite(top) ||
+  const int cg = std::min({62, scale(gmax, 61.5), scale(gsum, 61.5)});
+  const int x = std::min(cg, scale(top + 1.0, 61.9));
+  const int cl = std::min(62, scale(lsum, 61.5)), cuq = std::min(62, scale(usum, 61.5));
+  if (gmax > 4.0 || 62 - cg > 8 || x < kDefFxNode || cg - x > 8 || cl < 40 || cuq < 40 || !std::isfinite(top) ||
       !std::isfinite(gsum))
     return QMC_EUNSUPPORTED;
 
@@ -268,7 +271,7 @@ int build_deformed_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
   for (int k = 0; k < d; ++k) {
     for (int l = k; l < d; ++l) base.H[at(k, l)] = limb(times(-lambda, Hu[at(k, l)], cg));
     base.Q[k] = limb(times(-0.5 * lambda, Hu[at(k, k)], cg));
-    base.gl[k] = times(-lambda, lin[k], cg);
+    base.gl[k] = times(-lambda, lin[k], cg) + 4;
     base.fl[k] = limb(fixed(lin[k], cl));
     base.u[k] = limb(fixed(cu[1 + k], cuq));
   }
@@ -276,9 +279,14 @@ int build_deformed_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uin
     const double h = minors[S] * std::pow(-lambda, (double)__builtin_popcount(S));
     base.hs[S] = fixed(h, x);
     base.hl[S] = limb(base.hs[S]);
+    base.hs[S] += 4;
   }
   base.sh = 62 - cg;
   base.mx = cg - x;
+  base.half = 1 << (27 - base.sh);
+  base.four = 1 << (30 - base.sh);
+  base.around = ((1 << base.sh) >> 1) - 4 + (4 << base.sh);  // and 4 more for its own limbs
+  base.mround = ((1 << base.mx) >> 1) - 4;
   base.has_lin = lsum > 0.0;
   base.u0 = cu[0];
   base.su = std::ldexp(1.0, -cuq);

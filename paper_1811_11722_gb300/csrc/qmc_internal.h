@@ -184,12 +184,14 @@ struct FxLimb {
 struct DefFxParams : FxBase {
   FxLimb H[kDefFxMax * (kDefFxMax + 1) / 2];  // -lambda times F's Hessian, upper triangle, Q(cg)
   FxLimb Q[kDefFxMax];                        // half its diagonal
-  int64_t gl[kDefFxMax];                      // -lambda times F's linear coefficients, Q(cg)
+  int64_t gl[kDefFxMax];                      // -lambda times F's linear coefficients, Q(cg), plus 4
   FxLimb fl[kDefFxMax];                       // F's linear coefficients, Q(cl)
   FxLimb u[kDefFxMax];                        // U's linear coefficients, Q(cu)
-  int64_t hs[1 << kDefFxMax];                 // (-lambda)^|S| det(H_off restricted to S), Q(x)
+  int64_t hs[1 << kDefFxMax];                 // (-lambda)^|S| det(H_off restricted to S), Q(x), plus 4
   FxLimb hl[1 << kDefFxMax];
   int32_t sh, mx, has_lin;                    // 62 - cg, cg - x
+  int32_t half, four;                         // 1/2 and 4 in a cross sum that is shifted by sh: 2^(27 - sh), 2^(30 - sh)
+  int32_t around, mround;                     // rounding of y (1 - y) >> sh and m >> mx, which carry 4 units more
   double u0, su;                              // U: constant, unit of its sums
   double f0, c1, c2, c3;                      // F: constant, units of y.l, y.g, v.H v and -v.g
   double sd;                                  // 2^-x

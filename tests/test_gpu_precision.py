@@ -207,3 +207,15 @@ def test_fp64_separable_small_weights(Q, kind, near):
                             want_per_shift=True)
     ref = w.mean(axis=0)
     assert np.all(np.abs(ps[:, 0] - ref) <= 6.7e-15 * ref), (ps[:, 0], ref)
+
+
+@pytest.mark.parametrize("d,ratio,lam,linear", [(1, 64, 0.1, 0), (1, 400, 0.02, 0), (1, 400, 0.4, 1), (2, 400, 0.4, 1),
+                                                (3, 4, 0.1, 0), (3, 400, 0.4, 0), (4, 64, 0.4, 1), (5, 4, 0.4, 0),
+                                                (5, 16, 0.1, 1), (6, 4, 0.15, 1), (6, 64, 0.02, 0)])
+def test_fp64_deformed_estimates(Q, d, ratio, lam, linear):
+    """FP64 deformed estimates against extended precision, small and large deformations, constants from 1/4 to 1/400 of
+    the coefficients' sum: six roundings of 2^-53 for the sum, the scale, the mean and the fixed-point scales."""
+    p = deformed_problem(d, ratio, lam, linear)
+    ref = exact_deformed(p).mean()
+    got = complex(*estimate(Q, p, "fp64").mean)
+    assert abs(got - ref) <= 6.7e-16 * abs(ref), float(abs(got - ref) / abs(ref))
