@@ -240,7 +240,8 @@ static uint64_t fraction64(uint32_t idx, const Recip& rc) {
 // corner z = 0.  Emulated against 64 bits, the values' rms error is no larger
 // than the other form's up to a ratio of about 4 (d = 2), 8 (3), 32 (4), 128
 // (5) and 256 (6): the corner's share of the cube shrinks with d.  The line
-// stays below those.
+// stays below those.  Just below it estimates over 1.3e8 values lie 0.57 (d = 2) to
+// 0.78 (6) of the other form's distance from FP64 (eight integrands for each d).
 int korobov_form(int d, const std::vector<double>& cu, const std::vector<double>& cf) {
   const double most = std::ldexp(1.0, d <= 4 ? d : d + 1);
   for (const std::vector<double>* c : {&cu, &cf}) {
