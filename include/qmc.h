@@ -201,7 +201,8 @@ int qmc_plan_tune(qmc_plan plan, void* stream, int32_t* shifts_per_launch_out);
 #ifndef __CUDACC_RTC__  /* function declarations are host-only */
 /* One-line description of the plan's launches (kernel family, dimension,
  * shifts per launch, whether the kernel was specialised at run time for this
- * integrand, grid and tile size), NUL-terminated into buf[len]. */
+ * integrand, grid and tile size, whether FP64 is evaluated in 64-bit fixed point),
+ * NUL-terminated into buf[len]. */
 int qmc_plan_describe(qmc_plan plan, char* buf, int32_t len);
 #endif
 /* Timing hook: when set (non-NULL cudaEvent_t handles passed as void*), every

@@ -1126,18 +1126,19 @@ int qmc_plan_describe(qmc_plan plan, char* buf, int32_t len) {
   if (!plan || !buf || len < 1) return fail(QMC_EINVAL, "null plan or buffer");
   const Plan* pl = reinterpret_cast<const Plan*>(plan);
   const Launch* ln = pl->launches.empty() ? nullptr : &pl->launches[0];
+  const bool fixed = pl->param_kind == 5;  // FP64 in 64-bit fixed point
   int L = 0;
-  if (ln && ln->params.size() >= sizeof(RuleParams<float>)) {
+  if (ln && (fixed || ln->params.size() >= sizeof(RuleParams<float>))) {
     int32_t v;
-    std::memcpy(&v, ln->params.data() + offsetof(RuleParams<float>, L), sizeof(v));
+    std::memcpy(&v, ln->params.data() + (fixed ? offsetof(FxBase, L) : offsetof(RuleParams<float>, L)), sizeof(v));
     L = v;
   }
   snprintf(buf, (size_t)len,
            "d=%d n=%llu m=%d complex=%d orders=%d shifts_per_launch=%d launches=%zu specialised=%d ctas=%d L=%d "
-           "smem_acc=%d min_ctas=%d imm_shifts=%d",
+           "smem_acc=%d min_ctas=%d imm_shifts=%d fixed=%d",
            pl->d, (unsigned long long)pl->n, pl->m, pl->is_complex, pl->orders, pl->mc, pl->launches.size() + 1,
            (ln && ln->cufunc) ? 1 : 0, ln ? (int)(ln->grid.x * ln->grid.y) : pl->nblk, L, (ln && ln->smem) ? 1 : 0, pl->tune.minb,
-           (ln && ln->cufunc) ? pl->imm : 0);
+           (ln && ln->cufunc) ? pl->imm : 0, fixed ? 1 : 0);
   return QMC_OK;
 }
 

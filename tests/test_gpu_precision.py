@@ -244,3 +244,37 @@ def test_fp32_centred_form_at_its_line(Q, monkeypatch, d):
             rel.append((a - b) / b)
         rms.append(float(np.sqrt(np.mean(np.square(rel)))))
     assert rms[0] <= rms[1], rms
+
+
+def described(Q, p, precision="fp64"):
+    return Q.Plan(p.d, p.n, p.m, p.g, p.shifts, Q.transform(p.transform, p.alpha),
+                  Q.integrand_from_problem(p, precision)).describe()
+
+
+@pytest.mark.parametrize("case,fixed", [
+    (dict(d=3), 1), (dict(d=6), 1), (dict(d=7), 0), (dict(d=3, aU=-1), 0), (dict(d=3, quad_u=2), 0), (dict(d=3, alpha=2), 0),
+    (dict(d=3, f0=1 / 240), 1), (dict(d=3, f0=1 / 260), 0), (dict(d=3, u0=1 / 240), 1), (dict(d=3, u0=1 / 260), 0),
+    (dict(d=2, gsum=1.05 / 32), 1), (dict(d=2, gsum=0.95 / 32), 0), (dict(d=1, gsum=3.9), 1), (dict(d=1, gsum=4.1), 0)])
+def test_deformed_dispatch(Q, case, fixed):
+    """Which FP64 deformed plans are evaluated in fixed point: either side of every limit that one integrand can be put at
+    (f0, u0: the constant over the sum it is held against; gsum: the largest sum of |lambda dF|)."""
+    d = case["d"]
+    rng = I.SplitMix64(31 + d)
+    U = I.random_poly(rng, d, d, case.get("quad_u", 0))
+    F = I.random_poly(rng, d, d, d * (d + 1) // 2)
+    coefs = 2.0 * F.coef[1:].sum()  # sum of |dF(0)| twice and of the Hessian's entries
+    F.coef[0] = case.get("f0", 1.0) * coefs
+    U.coef[0] = case.get("u0", 1.0) * U.coef[1:].sum()
+    grads = sum(2 * c if e.sum() == 2 else c for c, e in zip(F.coef[1:], F.expo[1:]))
+    p = I.Problem("def", d, 1021, 4, I.make_shifts(rng, 4, d), "korobov", alpha=case.get("alpha", 3),
+                  kind="sector_deformed", U=U, F=F, aU=case.get("aU", -2), aF=-1,
+                  lam=case["gsum"] / grads if "gsum" in case else 0.05, g=I.random_generating_vector(rng, d, 1021))
+    assert described(Q, p)["fixed"] == str(fixed)
+
+
+def test_plan_description_of_fixed_point_plans(Q):
+    """Points per thread and tile are told for every kind of plan, as before the fixed-point kernels."""
+    for d, kind in ((4, {}), (3, dict(kind="sector_deformed", aU=-2, aF=-1, lam=0.05))):
+        p = random_sector(3, d, 1000003, 8, d, d, transform="korobov", alpha=3, **kind)
+        desc = described(Q, p)
+        assert desc["fixed"] == "1" and int(desc["L"]) >= 1
