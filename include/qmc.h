@@ -503,7 +503,10 @@ int qmc_cv_loss_grad(int32_t d, const qmc_cv_config* cfg, int32_t P, const doubl
  * deg F <= 2, d <= 8 (FP64 or FP32EVAL; Korobov weight 3, baker or none).
  * Returns QMC_EINVAL when m x (CTAs of one resident wave) slots exceed the
  * fixed array, QMC_EUNSUPPORTED for other integrands.  Arguments, outputs and
- * synchronisation as for qmc_integrate. */
+ * synchronisation as for qmc_integrate; the kernels are the ahead-of-time compiled
+ * ones, FP64 in double (five to seven times the time of qmc_integrate's fixed-point
+ * kernels) and FP32EVAL with the plain Korobov coordinate, so per-shift values
+ * agree with qmc_integrate's to rounding only. */
 #ifndef __CUDACC_RTC__  /* function declarations are host-only */
 int qmc_integrate_noalloc(int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
                           qmc_transform t, const qmc_integrand* f, qmc_result* out, double* per_shift,

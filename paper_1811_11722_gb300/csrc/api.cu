@@ -832,7 +832,6 @@ int launch_finalize(const Plan* pl, const Workspace& ws, qmc_result* res_dev, do
   A.nblk = pl->nblk;
   A.m = pl->m;
   A.is_complex = pl->is_complex;
-  A.groups = pl->orders;
   A.dn = (double)pl->n;
   A.value_scale = pl->final_scale;
   A.offset[0] = pl->offset[0];

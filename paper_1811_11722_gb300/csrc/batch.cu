@@ -735,7 +735,6 @@ static int walk_pass(BatchPlan* bp, const std::vector<int>& act, std::vector<Fin
     A.nblk = pl->nblk;
     A.m = pl->m;
     A.is_complex = pl->is_complex;
-    A.groups = 1;
     A.dn = (double)pl->n;
     A.value_scale = pl->final_scale;
     A.offset[0] = pl->offset[0];
@@ -868,7 +867,6 @@ static int walk_pass_persistent(BatchPlan* bp, WalkPersist* W, const std::vector
     A.partial = W->part[i];
     A.nblk = W->nitems[i];
     A.m = problems[i].m;
-    A.groups = 1;
     A.dn = (double)n[i];
     A.value_scale = bp->psec[i].final_scale;
     A.counters = W->cnt[i];

@@ -100,13 +100,13 @@ const void* finalize_ptr();
 const void* finalize_batch_ptr();
 const void* persist_kernel_ptr();  // batched sectors in one persistent launch (persist.cu)
 
-// Arguments of the final pass.
+// Arguments of the final pass; CTA b of finalize_kernel finalises group b (epsilon
+// order b, integrand b).
 struct FinalizeArgs {
   const double* partial;   // [groups][m][nblk][2]
   int32_t nblk;
   int32_t m;
   int32_t is_complex;
-  int32_t groups;          // finalize_kernel: CTA b finalises group b (epsilon order b, integrand b)
   double dn;      // n as a double
   double value_scale;
   double offset[2];  // added to Q^(k) of each part (control-variate integral)

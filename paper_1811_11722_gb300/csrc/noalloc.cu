@@ -1,10 +1,12 @@
 // qmc_integrate_noalloc: the single-problem rule for callers that cannot
 // allocate device memory (for example code running inside a host callback,
 // under an allocator that is locked or exhausted, or embedded in a framework
-// that owns every allocation of the process).  It runs the same sector kernel
-// and final pass as qmc_integrate, but its scratch (the per-CTA result slots,
-// the two counters and the staged result) lives in one file-scope __device__
-// array of fixed size instead of memory from cudaMalloc/cudaMallocAsync.
+// that owns every allocation of the process).  It runs the ahead-of-time compiled
+// sector kernels (FP64 in double, FP32 with the plain Korobov coordinate, neither the
+// fixed-point nor the run-time specialised kernels of qmc_integrate, whose plans are
+// built in host containers) and the same final pass, and its scratch (the per-CTA
+// result slots, the two counters and the staged result) lives in one file-scope
+// __device__ array of fixed size instead of memory from cudaMalloc/cudaMallocAsync.
 //
 // The array exists once per device that loads the library and stays resident
 // until the process exits.  Its device address comes from
