@@ -350,7 +350,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // eightfold at d = 8.  The residuals' FP64 operations, 16 clocks a warp each, are
 // split over the quads' lanes, and the loss is summed in the steps whose loss is
 // read (loss_part not null): 2 us of a step.  16381 pilot points, d = 8, 200 steps:
-// 5.08 -> 3.18 ms.
+// 5.08 -> 3.00 ms.
 __host__ __device__ __forceinline__ int cv_swz(int row, int k) {  // position of degree k in its row
   return ((((k >> 3) ^ (row >> 1)) & 3) << 3) | (k & 7);
 }
