@@ -862,10 +862,9 @@ int plan_execute(Plan* pl, qmc_result* out, double* per_shift, cudaStream_t stre
   const size_t res_bytes = G * sizeof(qmc_result), ps_bytes = G * pl->m * 2 * sizeof(double);
   const bool res_host = !out_dev, ps_host = per_shift && !ps_dev;
   if (res_host || ps_host) {
-    if (res_host && ps_host) {
-      // the workspace holds the results and then the per-shift values: one copy
-      // to pageable memory costs as much as either (8 us of a 70 us call)
-      const size_t ps_at = (size_t)((const char*)pl->ws.per_shift - (const char*)pl->ws.result);
+    // the workspace holds the results and then the per-shift values
+    const size_t ps_at = (size_t)((const char*)pl->ws.per_shift - (const char*)pl->ws.result);
+    if (res_host && ps_host && ps_at + ps_bytes <= kOneCopyMax) {
       std::vector<char> host(ps_at + ps_bytes);
       QMC_CUDA(cudaMemcpyAsync(host.data(), pl->ws.result, host.size(), cudaMemcpyDeviceToHost, stream));
       QMC_CUDA(cudaStreamSynchronize(stream));
@@ -873,7 +872,8 @@ int plan_execute(Plan* pl, qmc_result* out, double* per_shift, cudaStream_t stre
       std::memcpy(per_shift, host.data() + ps_at, ps_bytes);
     } else {
       if (res_host) QMC_CUDA(cudaMemcpyAsync(out, pl->ws.result, res_bytes, cudaMemcpyDeviceToHost, stream));
-      else QMC_CUDA(cudaMemcpyAsync(per_shift, pl->ws.per_shift, ps_bytes, cudaMemcpyDeviceToHost, stream));
+      if (ps_host)
+        QMC_CUDA(cudaMemcpyAsync(per_shift, pl->ws.per_shift, ps_bytes, cudaMemcpyDeviceToHost, stream));
       QMC_CUDA(cudaStreamSynchronize(stream));
     }
     if (!out_dev) {

@@ -753,9 +753,9 @@ static int walk_pass(BatchPlan* bp, const std::vector<int>& act, std::vector<Fin
   e = cudaLaunchKernel(finalize_batch_ptr(), dim3((unsigned)act.size()), dim3(kFinThreads), fargs,
                        (size_t)bp->max_m * 2 * sizeof(double), stream);
   if (e != cudaSuccess) return cuda_fail(e, "walk final pass");
-  if (ps) {  // the results and, after them, the per-shift values in one copy
-    const size_t ps_at = (size_t)((const char*)bp->ps_dev - (const char*)bp->res_dev);
-    const size_t ps_bytes = (size_t)bp->total_m * 2 * sizeof(double);
+  const size_t ps_at = (size_t)((const char*)bp->ps_dev - (const char*)bp->res_dev);
+  const size_t ps_bytes = (size_t)bp->total_m * 2 * sizeof(double);
+  if (ps && ps_at + ps_bytes <= kOneCopyMax) {  // the results and, after them, the per-shift values
     std::vector<char> host(ps_at + ps_bytes);
     e = cudaMemcpyAsync(host.data(), bp->res_dev, host.size(), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -765,6 +765,7 @@ static int walk_pass(BatchPlan* bp, const std::vector<int>& act, std::vector<Fin
     return QMC_OK;
   }
   e = cudaMemcpyAsync(res.data(), bp->res_dev, res.size() * sizeof(qmc_result), cudaMemcpyDeviceToHost, stream);
+  if (e == cudaSuccess && ps) e = cudaMemcpyAsync(ps, bp->ps_dev, ps_bytes, cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return cuda_fail(e, "walk results");
   return QMC_OK;

@@ -142,6 +142,10 @@ int launch_rule(const Plan* pl, const Workspace& ws, cudaStream_t stream, const 
 int launch_finalize(const Plan* pl, const Workspace& ws, qmc_result* res_dev, double* per_shift_dev,
                     cudaStream_t stream);
 int plan_execute(Plan* pl, qmc_result* out, double* per_shift, cudaStream_t stream);
+// Results and the per-shift values behind them come back in one copy up to this
+// many bytes: a second copy to pageable memory costs 8 us, sorting the bytes out on
+// the host about 0.1 us a KB and as much memory again.
+constexpr size_t kOneCopyMax = 64 << 10;
 
 bool jit_enabled();
 bool jit_smacc();

@@ -46,3 +46,27 @@ def test_fit_is_reproducible(Q, d, n_pilot):
         assert np.all(np.isfinite(got))
         first = got if first is None else first
         assert np.array_equal(got, first)
+
+
+@pytest.mark.parametrize("m", [8, 1024])
+def test_host_results_and_per_shift_values(Q, m):
+    """Results and per-shift values wanted on the host together, below and above the size up to which one copy brings
+    both: six orders of an epsilon expansion, and the passes of a walk over eight problems."""
+    d, n = 3, 1 << 9
+    rng = I.SplitMix64(8 + m)
+    shifts = I.make_shifts(rng, m, d)
+    g = np.array([1, 182667, 469891], dtype=np.uint64)
+    U, F = I.random_poly(rng, d, d, 0), I.random_poly(rng, d, 0, 6)
+    f = Q.Integrand(Q.QMC_F_SECTOR, d, Q.QMC_FP64, (U.coef, U.expo), (F.coef, F.expo))
+    t = Q.transform("korobov", 3)
+    res, ps = Q.qmc_integrate_eps(d, n, m, g % n, shifts, t, f, Q.eps_spec(6), want_per_shift=True)
+    ps = np.asarray(ps).reshape(6, m, 2)
+    for o in range(6):
+        assert res[o].status == 0 and np.isclose(res[o].mean[0], ps[o, :, 0].mean(), rtol=1e-13, atol=0)
+    levels = 2
+    walk, lv, passes, _ = Q.qmc_integrate_batch_extensible([(d, n, m, g % n, shifts, t, f)] * 8, levels, g, 1e-18,
+                                                           Q.WALK_EACH)
+    assert passes == levels + 1
+    last = Q.qmc_integrate(d, n << levels, m, g % (n << levels), shifts, t, f)[0]
+    for r in walk:
+        assert np.isclose(r.mean[0], last.mean[0], rtol=1e-14, atol=0)
