@@ -96,7 +96,7 @@ enum {
  *   the error of an estimate within 1.5 2^-53 of it (one rounding of the result),
  *   in 64-bit fixed point: U^-2 F^-1 sectors of degree 1 and 2 with none, baker or
  *   Korobov 3 whose coefficients add up to at most 1000 times the constant term,
- *   and deformed ones under Korobov 3 with d <= 6 and 250 in place of 1000.
+ *   and deformed ones under Korobov 3 with d <= 6, at most 250 (U) and 125 (F) times.
  * FP32EVAL: coordinates from 32-bit fixed point, transform and f in float,
  *   compensated float run sums promoted to double per thread.  Under the
  *   Korobov transform every value enters the compensated sum on its own (its

@@ -24,9 +24,10 @@
 // g' = -lambda dF, v = y (1 - y) g', m = y (1 - y) H'_kk + (1 - 2y) g' and the
 // quadratic forms, x for the recursion's nodes.  A product with a Q(cg) number comes
 // out 62 - cg = sh bits low; the sum is shifted back before its low part is added.
-// Error against 80-bit floats, d = 1..6, lambda 0.02 to 0.4, constants down to 1/250
-// of the coefficients' sum: a value (root mean square over the cube) 3e-16 to 3e-15,
-// an estimate 1e-17 to 1.2e-16.  With truncated limbs and sums and one bit less an
+// Error against 80-bit floats, d = 1..6, lambda 0.02 to 0.4, constants down to 1/120
+// of the coefficients' sum: an estimate 1e-18 to 1.2e-16 (root mean square of eight
+// integrands), a value 3e-16 to 5e-15 over the cube; more where Re F crosses zero and
+// |F| is small (d = 2, lambda <= 0.05: 4e-16 and 3e-13).  With truncated limbs and sums and one bit less an
 // estimate was up to 2.4e-15 off, the determinant's truncations being multiplied up
 // its recursion.
 #pragma once

@@ -188,7 +188,9 @@ int build_fx_plan(Plan* pl, int32_t d, uint64_t n, int32_t m, const uint64_t* g,
   return QMC_OK;
 }
 
-constexpr double kDefFxRange = 250.0;      // largest (coefficient sum) / (constant term): 2e-16 of the estimate
+// largest (sum of U's coefficients) / (its constant), and twice that sum / constant for
+// F (y.dF(0) and y.g come one after the other): 1.2e-16 of the estimate
+constexpr double kDefFxRange = 250.0;
 constexpr double kDefFxMin = 1.0 / 32.0;  // smallest sum of |lambda dF| over the cube
 constexpr int kDefFxNode = 55;            // smallest scale of the determinant's nodes: 1.4e-16 of the estimate, at 54 4e-16
 
