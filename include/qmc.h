@@ -631,8 +631,7 @@ int qmc_integrate_eps(int32_t d, uint64_t n, int32_t m, const uint64_t* g, const
 int qmc_eps_plan_create(int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
                         qmc_transform t, const qmc_integrand* f, const qmc_eps* eps, qmc_plan* plan_out);
 /* Single terms: values [count][orders] (host), order o of the weighted value
- * at point j[s], shift k[s], from the kernel of qmc_integrate_eps (weights as for
- * qmc_sample_points).
+ * at point j[s], shift k[s], by the device code of qmc_integrate_eps.
  * Synchronises `stream`. */
 int qmc_sample_points_eps(int32_t d, uint64_t n, int32_t m, const uint64_t* g, const double* shifts,
                           qmc_transform t, const qmc_integrand* f, const qmc_eps* eps, int32_t count,

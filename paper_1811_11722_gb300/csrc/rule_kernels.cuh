@@ -865,10 +865,10 @@ __device__ __forceinline__ void eps_body2(const RuleParams<float>& P, double* __
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       uint32_t idx = lattice_index(j, P.g[i], P.n);
-      base[i] = sec_base<float, kTermAlpha<ALPHA>>(idx, P.rc, j, i);
+      base[i] = sec_base<float, ALPHA>(idx, P.rc, j, i);
       if (sio.idx) sio.idx[(size_t)s * D + i] = idx;
-      if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<float, kTermAlpha<ALPHA>>(P, base[i], k, i);
-      z[i] = coord_fx<TR, kTermAlpha<ALPHA>>(base[i] + P.shiftx[k][i], P.kor, w);
+      if (sio.coord) sio.coord[(size_t)s * D + i] = sec_coord_used<float, ALPHA>(P, base[i], k, i);
+      z[i] = coord_fx<TR, ALPHA>(base[i] + P.shiftx[k][i], P.kor, w);
     }
     float U, F;
     POLY::template eval<D, 1, 2, float>(P, z, U, F);
@@ -876,7 +876,7 @@ __device__ __forceinline__ void eps_body2(const RuleParams<float>& P, double* __
     if constexpr (TR == TR_KOROBOV) v *= korobov_weight_fx(w);
     const float L = P.eps_b[0] * log_(U) + P.eps_b[1] * log_(F);
     for (int o = 0; o < P.eps_orders; ++o) {
-      sio.values[(size_t)s * sio.stride + o] = (double)v * (P.value_scale * term_scale<D, ALPHA>());
+      sio.values[(size_t)s * sio.stride + o] = (double)v * P.value_scale;
       v = v * L * P.eps_inv[o];
     }
     return;

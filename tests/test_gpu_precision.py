@@ -278,3 +278,13 @@ def test_plan_description_of_fixed_point_plans(Q):
         p = random_sector(3, d, 1000003, 8, d, d, transform="korobov", alpha=3, **kind)
         desc = described(Q, p)
         assert desc["fixed"] == "1" and int(desc["L"]) >= 1
+
+
+def test_fp32_epsilon_estimates(Q):
+    """Three epsilon orders of one integrand over 6.7e7 FP32 values, as recorded with the plain Korobov coordinate, to the
+    sums' rounding.  The coordinate centred on x = 1/2 moves this integrand's by 1.1e-9."""
+    p = random_sector(10, 6, 4194301, 16, 6, 12, transform="korobov", alpha=3)
+    res, _ = Q.qmc_integrate_eps(p.d, p.n, p.m, p.g, p.shifts, Q.transform("korobov", 3),
+                                 Q.integrand_from_problem(p, "fp32"), Q.eps_spec(3))
+    recorded = [0.018633754043793173, -0.010577168001121313, 0.003257045716876482]
+    assert np.allclose([r.mean[0] for r in res], recorded, rtol=1e-11, atol=0)
